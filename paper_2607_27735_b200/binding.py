@@ -1,9 +1,13 @@
-"""ctypes binding of ``libspec_attn.so``: argument marshalling only.
+"""Python binding of ``libspec_attn.so``: argument marshalling only.
 
 Every function takes CUDA torch tensors (torch is used for device memory and streams), checks
 dtypes/devices, passes raw pointers through the C ABI of ``include/spec_attn.h`` and raises
 ``SpecError`` on a non-zero return code.  There is no CPU fallback: if the library is missing
 or the tensors are not on a CUDA device the call fails.
+
+The calls of a speculation round go through the native module ``_spec_native`` (``csrc/py_native.cpp``):
+the checks and the pointers cost it about a microsecond where ctypes took 15-20 us per call, which bounded
+every small call made straight from Python.  ctypes stays for the calls outside a round.
 """
 from __future__ import annotations
 
@@ -62,6 +66,20 @@ class _KV(ctypes.Structure):
 
 
 _lib = None
+_native = None
+
+
+def _nat():
+    """The native marshalling module; raises if it has not been built."""
+    global _native
+    if _native is None:
+        load()
+        try:
+            from . import _spec_native
+        except ImportError as e:
+            raise ImportError("_spec_native is missing: run `python -m paper_2607_27735_b200.build`") from e
+        _native = _spec_native
+    return _native
 
 
 def load() -> ctypes.CDLL:
@@ -167,40 +185,24 @@ def spec_verify_attn(kv, q, ctx_len, max_ctx_len, stat_window=16, out=None, lse=
     selection's first radix pass (spec_verify_attn_hist).
     ``accumulate`` adds this call's statistic to the given ``stats``; ``per_head`` keeps one score per
     attention head (``stats`` is ``[L, B, n_q_heads, stride]``); both go through spec_verify_attn_ex."""
-    lib = load()
-    L, B, n_q, Hq, D = q.shape
-    dev = q.device
-    s = _kv_struct(kv)
     if stat_stride is None:
         stat_stride = (max_ctx_len + 63) // 64 * 64 if stats is None else stats.shape[-1]
-    out_dtype = torch.bfloat16 if out_bf16 else torch.float32
-    if out is None:
-        out = torch.empty(L, B, n_q, Hq, D, dtype=out_dtype, device=dev)
-    if lse is None and want_lse:
-        lse = torch.empty(L, B, n_q, Hq, dtype=torch.float32, device=dev)
-    if stats is None:
-        stats = torch.zeros(L, B, kv.n_q_heads if per_head else kv.n_kv_heads, stat_stride,
-                            dtype=torch.float32, device=dev)
-    if workspace is None:
-        workspace = alloc_workspace(workspace_bytes(WS_VERIFY, kv, n_q, max_ctx_len), dev)
-    if accumulate and stats is None:
-        raise ValueError("accumulate needs the stats tensor that holds the running sums")
-    args = (ctypes.byref(s), _dev(q, torch.bfloat16, "q"), n_q, _dev(ctx_len, torch.int32, "ctx_len"),
-            max_ctx_len, stat_window, _dev(out, out_dtype, "out"),
-            None if lse is None else _dev(lse, torch.float32, "lse"),
-            _dev(stats, torch.float32, "stats"), stat_stride, workspace.data_ptr(), workspace.numel())
-    if stats.shape[2] != (kv.n_q_heads if per_head else kv.n_kv_heads):
-        raise ValueError("stats: wrong head count for this mode")
+    if out is None or stats is None or workspace is None or (lse is None and want_lse):
+        L, B, n_q, Hq, D = q.shape
+        dev = q.device
+        if out is None:
+            out = torch.empty(L, B, n_q, Hq, D, dtype=torch.bfloat16 if out_bf16 else torch.float32, device=dev)
+        if lse is None and want_lse:
+            lse = torch.empty(L, B, n_q, Hq, dtype=torch.float32, device=dev)
+        if stats is None:
+            stats = torch.zeros(L, B, kv.n_q_heads if per_head else kv.n_kv_heads, stat_stride,
+                                dtype=torch.float32, device=dev)
+        if workspace is None:
+            workspace = alloc_workspace(workspace_bytes(WS_VERIFY, kv, n_q, max_ctx_len), dev)
     flags = ((VERIFY_ACCUMULATE_STATS if accumulate else 0) | (VERIFY_STATS_PER_QUERY_HEAD if per_head else 0) |
              (VERIFY_OUT_BF16 if out_bf16 else 0) | (VERIFY_STATS_GROUP_MAX if group_max else 0))
-    if score_hist is not None:
-        if score_hist.shape != stats.shape[:3] + (2048,):
-            raise ValueError("score_hist: expected [L, B, heads, 2048]")
-        rc = lib.spec_verify_attn_hist(*args, flags, _dev(score_hist, torch.int32, "score_hist"), _stream())
-    elif flags:
-        rc = lib.spec_verify_attn_ex(*args, flags, _stream())
-    else:
-        rc = lib.spec_verify_attn(*args, _stream())
+    rc = (_native or _nat()).verify(kv, q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace,
+                                    flags, score_hist)
     if rc != 0:
         raise SpecError(rc, "spec_verify_attn")
     return out, lse, stats, workspace
@@ -245,25 +247,13 @@ def spec_select_recall(stats, sel_len, k_sink, k_recent, k_total, indices=None, 
                        score_hist=None, hist_len=None):
     """Eq. 4 recall selection; returns ``(indices, n_indices)``.  ``score_hist`` / ``hist_len``: the
     counts a verification call left (spec_select_recall_hist); they are cleared."""
-    lib = load()
-    L, B, Hkv, stride = stats.shape
-    dev = stats.device
-    if indices is None:
-        indices = torch.empty(L, B, Hkv, k_total, dtype=torch.int32, device=dev)
-    if n_indices is None:
-        n_indices = torch.empty(L, B, Hkv, dtype=torch.int32, device=dev)
-    if score_hist is not None:
-        rc = lib.spec_select_recall_hist(
-            _dev(stats, torch.float32, "stats"), stride, L, B, Hkv,
-            _dev(sel_len, torch.int32, "sel_len"), k_sink, k_recent, k_total,
-            _dev(indices, torch.int32, "indices"), _dev(n_indices, torch.int32, "n_indices"),
-            _dev(score_hist, torch.int32, "score_hist"), _dev(hist_len, torch.int32, "hist_len"), None, 0, _stream())
-    else:
-        rc = lib.spec_select_recall(
-            _dev(stats, torch.float32, "stats"), stride, L, B, Hkv,
-            _dev(sel_len, torch.int32, "sel_len"), k_sink, k_recent, k_total,
-            _dev(indices, torch.int32, "indices"), _dev(n_indices, torch.int32, "n_indices"), None, 0,
-            _stream())
+    if indices is None or n_indices is None:
+        L, B, Hkv, _ = stats.shape
+        if indices is None:
+            indices = torch.empty(L, B, Hkv, k_total, dtype=torch.int32, device=stats.device)
+        if n_indices is None:
+            n_indices = torch.empty(L, B, Hkv, dtype=torch.int32, device=stats.device)
+    rc = (_native or _nat()).select(stats, sel_len, k_sink, k_recent, k_total, indices, n_indices, score_hist, hist_len)
     if rc != 0:
         raise SpecError(rc, "spec_select_recall")
     return indices, n_indices
@@ -275,74 +265,50 @@ def spec_sparse_draft_attn(kv, q, indices, n_indices, tail_start, cur_len, max_t
     """Eq. 5 sparse draft attention; returns ``(out, lse, workspace)``.  ``per_head``: ``indices`` is
     ``[L, B, n_q_heads, k_total]``, one set per attention head (spec_sparse_draft_attn_ex).
     ``early_gather``: the caller's promise behind SPEC_DRAFT_EARLY_GATHER (see the header)."""
-    lib = load()
-    L, B, Hq, D = q.shape
-    dev = q.device
-    s = _kv_struct(kv)
-    k_total = indices.shape[-1]
-    out_dtype = torch.bfloat16 if out_bf16 else torch.float32
-    if out is None:
-        out = torch.empty(L, B, Hq, D, dtype=out_dtype, device=dev)
-    if lse is None and want_lse:
-        lse = torch.empty(L, B, Hq, dtype=torch.float32, device=dev)
-    if workspace is None:
-        workspace = alloc_workspace(workspace_bytes(WS_DRAFT, kv, k_total=k_total + max_tail), dev)
-    if indices.shape[2] != (kv.n_q_heads if per_head else kv.n_kv_heads):
-        raise ValueError("indices: wrong head count for this mode")
-    args = (ctypes.byref(s), _dev(q, torch.bfloat16, "q"), _dev(indices, torch.int32, "indices"),
-            _dev(n_indices, torch.int32, "n_indices"), k_total,
-            _dev(tail_start, torch.int32, "tail_start"), _dev(cur_len, torch.int32, "cur_len"),
-            max_tail, _dev(out, out_dtype, "out"),
-            None if lse is None else _dev(lse, torch.float32, "lse"), workspace.data_ptr(),
-            workspace.numel())
-    if per_head or out_bf16 or early_gather:
-        flags = ((DRAFT_INDICES_PER_QUERY_HEAD if per_head else 0) | (DRAFT_OUT_BF16 if out_bf16 else 0) |
-                 (DRAFT_EARLY_GATHER if early_gather else 0))
-        rc = lib.spec_sparse_draft_attn_ex(*args, flags, _stream())
-    else:
-        rc = lib.spec_sparse_draft_attn(*args, _stream())
+    if out is None or workspace is None or (lse is None and want_lse):
+        L, B, Hq, D = q.shape
+        dev = q.device
+        if out is None:
+            out = torch.empty(L, B, Hq, D, dtype=torch.bfloat16 if out_bf16 else torch.float32, device=dev)
+        if lse is None and want_lse:
+            lse = torch.empty(L, B, Hq, dtype=torch.float32, device=dev)
+        if workspace is None:
+            workspace = alloc_workspace(workspace_bytes(WS_DRAFT, kv, k_total=indices.shape[-1] + max_tail), dev)
+    flags = ((DRAFT_INDICES_PER_QUERY_HEAD if per_head else 0) | (DRAFT_OUT_BF16 if out_bf16 else 0) |
+             (DRAFT_EARLY_GATHER if early_gather else 0))
+    rc = (_native or _nat()).draft(kv, q, indices, n_indices, tail_start, cur_len, max_tail, out, lse, workspace, flags)
     if rc != 0:
         raise SpecError(rc, "spec_sparse_draft_attn")
     return out, lse, workspace
 
 
+def _check_logits_2d(logits):
+    if not logits.is_cuda or logits.dim() != 2 or logits.stride(1) != 1:
+        raise ValueError("logits: expected a CUDA [rows, vocab] tensor with unit inner stride")
+
+
 def spec_token_entropy(logits, entropy=None):
     """Entropy (nats) of softmax(logits[r]) per row; ``logits`` is [rows, vocab] fp32 or bf16 with a
     unit inner stride (rows may be strided).  Returns ``entropy`` ([rows] fp32)."""
-    if not logits.is_cuda or logits.dim() != 2 or logits.stride(1) != 1:
-        raise ValueError("logits: expected a CUDA [rows, vocab] tensor with unit inner stride")
-    if logits.dtype not in (torch.float32, torch.bfloat16):
-        raise ValueError(f"logits: expected fp32 or bf16, got {logits.dtype}")
-    rows, vocab = logits.shape
     if entropy is None:
-        entropy = torch.empty(rows, dtype=torch.float32, device=logits.device)
-    rc = load().spec_token_entropy(logits.data_ptr(), 1 if logits.dtype == torch.bfloat16 else 0, rows, vocab,
-                                   logits.stride(0) if rows > 1 else max(logits.stride(0), vocab),
-                                   _dev(entropy, torch.float32, "entropy"), _stream())
+        _check_logits_2d(logits)
+        entropy = torch.empty(logits.shape[0], dtype=torch.float32, device=logits.device)
+    rc = (_native or _nat()).rows(logits, None, entropy)
     if rc != 0:
         raise SpecError(rc, "spec_token_entropy")
     return entropy
 
 
-def _logits_2d(logits):
-    if not logits.is_cuda or logits.dim() != 2 or logits.stride(1) != 1:
-        raise ValueError("logits: expected a CUDA [rows, vocab] tensor with unit inner stride")
-    if logits.dtype not in (torch.float32, torch.bfloat16):
-        raise ValueError(f"logits: expected fp32 or bf16, got {logits.dtype}")
-    rows, vocab = logits.shape
-    return rows, vocab, 1 if logits.dtype == torch.bfloat16 else 0, max(logits.stride(0), vocab)
-
-
 def spec_token_argmax(logits, token=None, entropy=None, want_entropy=False):
     """Greedy token per row (smallest index of the largest logit), optionally with the row's entropy
     from the same pass.  Returns ``(token, entropy or None)``."""
-    rows, vocab, dt, stride = _logits_2d(logits)
-    if token is None:
-        token = torch.empty(rows, dtype=torch.int32, device=logits.device)
-    if entropy is None and want_entropy:
-        entropy = torch.empty(rows, dtype=torch.float32, device=logits.device)
-    rc = load().spec_token_argmax(logits.data_ptr(), dt, rows, vocab, stride, _dev(token, torch.int32, "token"),
-                                  None if entropy is None else _dev(entropy, torch.float32, "entropy"), _stream())
+    if token is None or (entropy is None and want_entropy):
+        _check_logits_2d(logits)
+        if token is None:
+            token = torch.empty(logits.shape[0], dtype=torch.int32, device=logits.device)
+        if entropy is None and want_entropy:
+            entropy = torch.empty(logits.shape[0], dtype=torch.float32, device=logits.device)
+    rc = (_native or _nat()).rows(logits, token, entropy)
     if rc != 0:
         raise SpecError(rc, "spec_token_argmax")
     return token, entropy
@@ -351,23 +317,18 @@ def spec_token_argmax(logits, token=None, entropy=None, want_entropy=False):
 def spec_accept_greedy(logits, draft, n_draft=None, target=None, n_accepted=None, next_token=None):
     """Greedy prefix acceptance; ``logits`` is a contiguous CUDA ``[batch, k + 1, vocab]`` tensor, ``draft``
     int32 ``[batch, k]``.  Returns device tensors ``(target, n_accepted, next_token)``."""
-    if not logits.is_cuda or logits.dim() != 3 or not logits.is_contiguous():
-        raise ValueError("logits: expected a contiguous CUDA [batch, k + 1, vocab] tensor")
-    if logits.dtype not in (torch.float32, torch.bfloat16):
-        raise ValueError(f"logits: expected fp32 or bf16, got {logits.dtype}")
-    batch, k1, vocab = logits.shape
-    dev = logits.device
-    if target is None:
-        target = torch.empty(batch, k1, dtype=torch.int32, device=dev)
-    if n_accepted is None:
-        n_accepted = torch.empty(batch, dtype=torch.int32, device=dev)
-    if next_token is None:
-        next_token = torch.empty(batch, dtype=torch.int32, device=dev)
-    rc = load().spec_accept_greedy(
-        logits.data_ptr(), 1 if logits.dtype == torch.bfloat16 else 0, batch, k1, vocab, vocab,
-        _dev(draft, torch.int32, "draft") if k1 > 1 else None,
-        None if n_draft is None else _dev(n_draft, torch.int32, "n_draft"), _dev(target, torch.int32, "target"),
-        _dev(n_accepted, torch.int32, "n_accepted"), _dev(next_token, torch.int32, "next_token"), _stream())
+    if target is None or n_accepted is None or next_token is None:
+        if not logits.is_cuda or logits.dim() != 3:
+            raise ValueError("logits: expected a contiguous CUDA [batch, k + 1, vocab] tensor")
+        batch, k1, _ = logits.shape
+        dev = logits.device
+        if target is None:
+            target = torch.empty(batch, k1, dtype=torch.int32, device=dev)
+        if n_accepted is None:
+            n_accepted = torch.empty(batch, dtype=torch.int32, device=dev)
+        if next_token is None:
+            next_token = torch.empty(batch, dtype=torch.int32, device=dev)
+    rc = (_native or _nat()).accept(logits, draft, n_draft, target, n_accepted, next_token)
     if rc != 0:
         raise SpecError(rc, "spec_accept_greedy")
     return target, n_accepted, next_token
@@ -377,12 +338,7 @@ def spec_advance_lengths(committed, n_accepted, k, ctx_verify=None, cur_len=None
     """committed += n_accepted + 1 on the device (``n_accepted=None``: unchanged), then the lengths of the
     next round: ``ctx_verify`` [batch] and ``cur_len`` [k, batch] (both optional, int32).  ``max_len`` > 0
     holds a sequence whose next round would not fit the cache and records that in ``workspace``."""
-    rc = load().spec_advance_lengths(
-        _dev(committed, torch.int32, "committed"),
-        None if n_accepted is None else _dev(n_accepted, torch.int32, "n_accepted"), committed.numel(), k,
-        int(max_len), None if workspace is None else workspace.data_ptr(),
-        None if ctx_verify is None else _dev(ctx_verify, torch.int32, "ctx_verify"),
-        None if cur_len is None else _dev(cur_len, torch.int32, "cur_len"), _stream())
+    rc = (_native or _nat()).advance(committed, n_accepted, k, ctx_verify, cur_len, max_len, workspace)
     if rc != 0:
         raise SpecError(rc, "spec_advance_lengths")
     return committed
@@ -391,9 +347,7 @@ def spec_advance_lengths(committed, n_accepted, k, ctx_verify=None, cur_len=None
 def spec_controller_update(state, entropy, n_accepted, beta):
     """Eq. "ema" in place on ``state`` ([2] fp32: accepted mean, rejected mean); ``n_accepted`` is a
     device int32 scalar tensor."""
-    rc = load().spec_controller_update(_dev(state, torch.float32, "state"), _dev(entropy, torch.float32, "entropy"),
-                                       entropy.numel(), _dev(n_accepted, torch.int32, "n_accepted"), float(beta),
-                                       _stream())
+    rc = (_native or _nat()).controller_update(state, entropy, n_accepted, beta)
     if rc != 0:
         raise SpecError(rc, "spec_controller_update")
     return state
@@ -408,10 +362,7 @@ def spec_controller_select(state, entropy, cand, c_d, c_v, k_star=None, p=None, 
         p = torch.empty(entropy.numel(), dtype=torch.float32, device=dev)
     if score is None:
         score = torch.empty(cand.numel(), dtype=torch.float32, device=dev)
-    rc = load().spec_controller_select(
-        _dev(state, torch.float32, "state"), _dev(entropy, torch.float32, "entropy"), entropy.numel(),
-        _dev(cand, torch.int32, "cand"), cand.numel(), float(c_d), float(c_v), _dev(k_star, torch.int32, "k_star"),
-        _dev(p, torch.float32, "p"), _dev(score, torch.float32, "score"), _stream())
+    rc = (_native or _nat()).controller_select(state, entropy, cand, c_d, c_v, k_star, p, score)
     if rc != 0:
         raise SpecError(rc, "spec_controller_select")
     return k_star, p, score

@@ -31,6 +31,8 @@
 // All CTAs must become co-resident (they wait on each other's partials): the grid never exceeds
 // the SM count at one CTA per SM (see the launcher).  Every wait is bounded; on expiry the kernel
 // records SPEC_ERR_TIMEOUT in the status word and drains.
+#include <atomic>
+
 #include "sm100_common.cuh"
 
 namespace spec {
@@ -1145,8 +1147,15 @@ int launch_cfg(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& 
                int grid, size_t smem_bytes, cudaStream_t stream)
 {
     auto kern = verify_cached_kernel<NC, CG, LP, PH, SC, F8>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
-        return SPEC_ERR_CUDA;
+    // the largest size any plan of this instance asks for, once per device: the call costs the host as much as a launch
+    static std::atomic<bool> opted_in[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPEC_ERR_CUDA;
+    if (!opted_in[dev]) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+            return SPEC_ERR_CUDA;
+        opted_in[dev] = true;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(128 + 128 * CG);
@@ -1164,9 +1173,7 @@ int launch_cfg(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    static bool pdl_refused[64] = {};  // per device: a driver that refuses the attribute is asked only once
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+    static std::atomic<bool> pdl_refused[64] = {};  // per device: a driver that refuses the attribute is asked only once
     const bool pdl_ok = !pdl_refused[dev];
     cudaError_t err = pdl_ok ? cudaLaunchKernelEx(&cfg, kern, tk, tv, tq, fp) : cudaErrorNotSupported;
     if (err != cudaSuccess) {
