@@ -1,34 +1,61 @@
 // Recall selection of Eq. 4: sink + TopK over the middle span + recent, per (layer, sequence,
 // KV head).  One CTA per problem.  The scores are sums of probabilities (finite, >= 0), so the
-// fp32 bit pattern orders like the value and the K_mid-th largest is found by a three-pass
-// radix select (11 + 11 + 10 bits) on the bit patterns; an ordered compaction then emits, in
-// ascending position, everything above the threshold plus the lowest-position ties.
-// The scores are swept twice when the threshold's first-digit bin fits in shared memory (the usual
-// case): the second sweep marks every candidate above that bin in a position bitmap and keeps the
-// bin's own candidates (score, position) in a list; the last two digits are decided on the list and
-// the index set is read off the bitmap in position order.  Flat scores (a bin too full for the list)
-// and contexts too long for the bitmap fall back to one sweep per digit plus one for an ordered
-// compaction.
-// The first pass's histogram (top 11 bits) may arrive from the verification kernel, which counts
-// every score it writes: the positions outside the candidate span are taken out again here, the
-// sweep over the scores is skipped, and the counts are cleared for the next round.
+// fp32 bit pattern orders like the value and selection works on bit patterns: integer work only.
+//
+// The scores are read ONCE.  A strided sample of 4096 of them gives a floor that the K_mid-th largest lies
+// above with a wide margin (6 sigma); one sweep of 16-byte loads collects what reaches the floor (a few
+// percent: score and position) in shared memory; the threshold is found on that list by a histogram of
+// (bits - floor) scaled to the list's own range, refined until its bin is small, whose entries are ranked
+// pair by pair (larger score, then lower position).  Chosen positions become bits of a position bitmap, which is
+// read off in order.  A span that fits the list needs no sample (every score is a list entry).  Where this
+// fails (a sample that misleads, hundreds of equal scores at the threshold, a budget above the list, contexts
+// above the bitmap's 128 K) one sweep per radix digit and an ordered compaction do it.
+//
+// What bounds it: HBM at many long problems, else the chain of memory latencies, block barriers and first
+// instruction fetches (about 8 us; code that runs once stays rolled and shared).  256 problems (32 layers x
+// 8 heads) of 131 K scores: 105 -> 47 us; of 32 K: 35 -> 20 us.  The two sweeps of
+// histogram and collection that this replaced waited for every load and read the scores twice.
+//
+// The first radix digit's histogram (top 11 bits) may arrive from the verification kernel, which counts
+// every score it writes: the positions outside the candidate span are taken out again here, the bin of the
+// K_mid-th largest is the floor, no sample is taken, and the counts are cleared for the next round.
+#include <atomic>
+
 #include "spec_common.cuh"
 
 namespace spec {
 
 namespace {
 
-constexpr int kThreads = 1024;
+constexpr int kThreads = 512;      // two CTAs per SM at 64 registers: 256 problems (32 layers x 8 heads) are one wave
+constexpr int kWarps = kThreads / 32;
 constexpr int kBins = kScoreBins;
-static_assert(kBins == 2 * kThreads, "two bins per thread");
-constexpr int kItems = 8;  // consecutive candidates per thread in the compaction sweep
-constexpr int kCap = 6144; // candidates (score, position) kept in shared memory
-constexpr int kMapWords = 4096;  // position bitmap: contexts up to 128 K keys
-static_assert(kMapWords == 4 * kThreads, "at most four bitmap words per thread");
-constexpr size_t kDynSmem = (size_t)(2 * kCap + kMapWords) * 4;
+constexpr int kBpt = kBins / kThreads;  // bins per thread
+constexpr int kItems = 16;         // consecutive candidates per thread in the compaction sweep
+constexpr int kListWords = 20480;  // list: 10240 entries (score, position), or 20480 scores in order: 80 KB
+constexpr int kDense = 4096;       // spans up to here are list entries as they are (eight per thread)
+constexpr int kPair = 512;         // entries ranked pair by pair (they reuse the histogram's storage)
+static_assert(2 * kPair <= kBins, "score and position of each");
+constexpr int kSample = 4096;      // eight per thread: a relative error of the floor's rank of 8 % at 3 % kept
+constexpr int kV = 4;              // vectors per thread and trip of the sweep; the next trip's are in flight meanwhile
+constexpr int kTrip = kV * kThreads;           // vectors per trip
+constexpr int kMapWords = 4096;                // position bitmap: contexts up to 128 K keys
+// Bins of the sample's histogram: an exponent and five bits, 32 to the octave, for the 64 octaves below 2^16 (a
+// score is a sum of at most some hundred probabilities); smaller scores share the last one.
+constexpr int kSampleShift = 18;
+constexpr uint32_t kSampleBase = 0x47800000u - ((uint32_t)kBins << kSampleShift);
 
-// Exclusive block-wide prefix sum of one int per thread; `total` gets the block sum.
-__device__ __forceinline__ int block_exclusive_scan(int x, int* warp_tmp, int& total)
+struct Shared {
+    int hist[kBins];
+    uint32_t bitmap[kMapWords];  // chosen positions
+    int warp_tmp[kWarps];
+    int bucket, above, count, total, list_n, pair_n;
+    uint32_t max;
+};
+
+// Exclusive block-wide prefix sum of one int per thread; sh.total gets the block sum (two barriers; every thread
+// may read sh.total and call again).
+__device__ __noinline__ int block_exclusive_scan(Shared& sh, int x)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int inc = x;
@@ -38,26 +65,78 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int* warp_tmp, int& t
         if (lane >= o) inc += y;
     }
     __syncthreads();  // warp_tmp may still be read from a previous scan
-    if (lane == 31) warp_tmp[warp] = inc;
+    if (lane == 31) sh.warp_tmp[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        int w = warp_tmp[lane];
-        int winc = w;
+    int w = lane < kWarps ? sh.warp_tmp[lane] : 0;  // every warp scans the warps' sums for itself
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, winc, o);
-            if (lane >= o) winc += y;
-        }
-        warp_tmp[lane] = winc - w;          // exclusive offset of each warp
-        if (lane == 31) warp_tmp[32] = winc;  // block total
+    for (int o = 1; o < kWarps; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += y;
     }
-    __syncthreads();
-    total = warp_tmp[32];
-    return warp_tmp[warp] + inc - x;
+    if (threadIdx.x == kWarps - 1) sh.total = w;
+    const int before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    return (warp > 0 ? before : 0) + inc - x;
 }
 
-// Calls f(bits, position) for every candidate of [lo, hi): eight loads per thread are in flight before the first
-// is used (a loop of one load and one atomic per trip would pay the memory latency on every trip).
+// Walks the bins of the histogram from the largest digit down (thread t owns reversed bins 4t .. 4t + 3) and
+// leaves the one in which the running count reaches `want` (bucket, above, count); false if the counts do
+// not reach it.  Called with the counts complete (a barrier behind them); clears them for the next use.
+__device__ __noinline__ bool find_bucket(Shared& sh, int want)
+{
+    static_assert(kBpt == 4, "four bins per thread");
+    int4* mine = reinterpret_cast<int4*>(sh.hist + kBins - 4 - 4 * (int)threadIdx.x);
+    const int4 c = *mine;
+    *mine = make_int4(0, 0, 0, 0);
+    int ex = block_exclusive_scan(sh, c.x + c.y + c.z + c.w);
+    const int cc[4] = {c.w, c.z, c.y, c.x};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (ex < want && want <= ex + cc[k]) {
+            sh.bucket = kBins - 1 - 4 * (int)threadIdx.x - k;
+            sh.above = ex;
+            sh.count = cc[k];
+        }
+        ex += cc[k];
+    }
+    __syncthreads();
+    return sh.total >= want;
+}
+
+// 16 bytes of scores; volatile, so that a load written ahead of other work is also issued ahead of it
+__device__ __forceinline__ uint4 load_vec(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+// asks L2 for `bytes` (a multiple of 16) from a 16-byte aligned address; nothing waits for it
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ int sample_bin(uint32_t u)
+{
+    return u <= kSampleBase ? 0 : min((int)((u - kSampleBase) >> kSampleShift), kBins - 1);
+}
+
+// Where u >= floor: stores u and its position in the list slot at shared address `at` (positions `off` bytes further) and
+// moves on by a slot.  Predicated, not branched: a warp has about twenty hits in the 512 scores of a trip, spread over
+// most of its lanes, and a branch per score made the sweep bound by instruction issue (380 per warp and trip, 33 us
+// instead of 25 at 256 x 131 K scores; with a branch per vector 480 and 49 us).
+__device__ __forceinline__ void push_if(uint32_t u, uint32_t floor, uint32_t& at, uint32_t off, int pos)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .u32 q;\n\t"
+        "setp.ge.u32 p, %1, %2;\n\t"
+        "add.u32 q, %0, %3;\n\t"
+        "@p st.shared.u32 [%0], %1;\n\t"
+        "@p st.shared.u32 [q], %4;\n\t"
+        "@p add.u32 %0, %0, 4;\n\t}"
+        : "+r"(at) : "r"(u), "r"(floor), "r"(off), "r"(pos) : "memory");
+}
+
+// Calls f(bits, position) for every candidate of [lo, hi), eight loads per thread in flight (slow path).
 template <typename F>
 __device__ __forceinline__ void sweep(const uint32_t* __restrict__ st, int lo, int hi, F f)
 {
@@ -71,48 +150,91 @@ __device__ __forceinline__ void sweep(const uint32_t* __restrict__ st, int lo, i
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2)  // two CTAs per SM: 32 registers per thread
+// Slow path: one sweep per radix digit, then an ordered compaction.  The histogram is clear.
+__device__ __noinline__ void select_by_sweeps(Shared& sh, const uint32_t* __restrict__ st, int lo, int hi, int k_mid,
+                                              int32_t* __restrict__ out)
+{
+    uint32_t prefix = 0, mask = 0;
+    int need = k_mid;  // how many to take among candidates matching the decided prefix
+    for (int pass = 0; pass < 3; ++pass) {
+        const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+        const uint32_t digits = pass == 2 ? 1023u : 2047u;
+        __syncthreads();
+        sweep(st, lo, hi, [&](uint32_t u, int) {
+            if ((u & mask) == prefix) atomicAdd(&sh.hist[(u >> shift) & digits], 1);
+        });
+        __syncthreads();
+        find_bucket(sh, need);
+        prefix |= (uint32_t)sh.bucket << shift;
+        mask |= digits << shift;
+        need -= sh.above;
+    }
+    const uint32_t thr = prefix;  // take every candidate > thr and the first `need` equal to it
+    // One block scan per trip: the counts of "above the threshold" (high half) and "equal to it" (low
+    // half) travel in one word; a candidate's slot is (candidates above it so far) + (equal ones so far,
+    // capped at the number still needed).
+    int gt_seen = 0, eq_seen = 0;
+    for (int base = lo; base < hi; base += kThreads * kItems) {
+        const int i0 = base + (int)threadIdx.x * kItems;
+        uint32_t u[kItems];
+        int packed = 0;
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            u[k] = (i0 + k < hi) ? __ldg(st + i0 + k) : 0u;
+            if (i0 + k < hi) packed += u[k] > thr ? (1 << 16) : (u[k] == thr ? 1 : 0);
+        }
+        const int ex = block_exclusive_scan(sh, packed);
+        int gt = gt_seen + (ex >> 16), eq = eq_seen + (ex & 0xffff);
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            if (i0 + k < hi) {
+                if (u[k] > thr) {
+                    out[gt + min(eq, need)] = i0 + k;
+                    ++gt;
+                } else if (u[k] == thr) {
+                    if (eq < need) out[gt + eq] = i0 + k;
+                    ++eq;
+                }
+            }
+        }
+        __syncthreads();  // sh.total is written by one thread of the scan
+        gt_seen += sh.total >> 16;
+        eq_seen += sh.total & 0xffff;
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
 select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int batch, int n_kv_heads,
-                     const int32_t* __restrict__ sel_len, int k_sink, int k_recent, int k_total,
+                     const int32_t* __restrict__ sel_len, int k_sink, int k_recent, int k_total, int list_words,
                      int32_t* __restrict__ indices, int32_t* __restrict__ n_indices,
                      uint32_t* __restrict__ hist_g, const int32_t* __restrict__ hist_len)
 {
-    __shared__ int hist[kBins];
-    __shared__ int warp_tmp[33];
-    __shared__ int sh_bucket, sh_above, sh_count, list_n;
-    extern __shared__ uint32_t dyn_smem[];
-    uint32_t* list = dyn_smem;                                // [kCap] score bit patterns
-    int* lpos = reinterpret_cast<int*>(dyn_smem + kCap);      // [kCap] their positions
-    uint32_t* bitmap = dyn_smem + 2 * kCap;                   // [kMapWords] chosen positions
+    __shared__ __align__(16) Shared sh;
+    extern __shared__ __align__(16) uint32_t dyn_smem[];
+    const int cap = list_words / 2;
+    uint32_t* list = dyn_smem;                           // score bit patterns
+    int* lpos = reinterpret_cast<int*>(dyn_smem + cap);  // [cap] their positions (a dense list needs none)
 
     const int64_t prob = blockIdx.x;
     const int b = (int)((prob / n_kv_heads) % batch);
-    const int tid = threadIdx.x;
-    // counts handed over by the verification kernel: requested first (two bins per thread), taken and
-    // cleared whatever happens below
-    uint32_t h0 = 0, h1 = 0;
-    uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
-    if (hg) {
-        h0 = hg[tid];
-        h1 = hg[tid + kThreads];
-    }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int T = sel_len[b];
-    const int HL = hg ? hist_len[b] : 0;
     int32_t* out = indices + prob * k_total;
     const uint32_t* st = reinterpret_cast<const uint32_t*>(stats + prob * stat_stride);
-    // they cover positions [0, hist_len): usable if the candidate span lies inside.  The positions outside
-    // the span that were counted (sink, recent window, rows beyond the committed length: a few dozen)
-    // are fetched now and taken out of the counts below.
+    // counts handed over by the verification kernel: taken and cleared whatever happens below.  They cover
+    // positions [0, hist_len): usable if the candidate span lies inside
+    uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
+    const int HL = hg ? hist_len[b] : 0;
     const bool have_hist = hg && T <= HL && T > k_total;
-    uint32_t excl = 0xffffffffu;
-    if (have_hist && tid < k_sink + (HL - (T - k_recent)))
-        excl = __ldg(st + (tid < k_sink ? tid : T - k_recent + (tid - k_sink))) >> 21;
-    if (hg) {
-        hist[tid] = (int)h0;
-        hist[tid + kThreads] = (int)h1;
-        hg[tid] = 0u;
-        hg[tid + kThreads] = 0u;
-        __syncthreads();
+    for (int i = tid; i < kBins; i += kThreads) {
+        sh.hist[i] = have_hist ? (int)hg[i] : 0;
+        if (hg) hg[i] = 0u;
+    }
+    for (int i = tid; i < kMapWords / 4; i += kThreads) reinterpret_cast<uint4*>(sh.bitmap)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        sh.list_n = 0;
+        sh.pair_n = 0;
+        sh.max = 0u;
     }
 
     if (T <= k_total) {  // everything fits: keep every position
@@ -127,192 +249,249 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     if (tid == 0) n_indices[prob] = k_total;
     if (k_mid == 0) return;
 
-    // ---- radix select: bit pattern `thr` of the k_mid-th largest candidate ----
-    uint32_t prefix = 0, mask = 0;
-    int need = k_mid;  // how many to take among candidates matching the decided prefix
-    int n_list = 0;
-    bool use_list = false;
-    const bool map_ok = hi <= kMapWords * 32;
-    const int map_words = map_ok ? (hi + 31) >> 5 : 0;
-    const int wpt = (map_words + kThreads - 1) / kThreads;  // bitmap words per thread (consecutive ones)
-    // walks the buckets of `hist` from the largest digit down (thread t owns reversed bins 2t, 2t+1) and
-    // leaves the one in which the running count reaches `want`; false if the counts do not reach it
-    auto find_bucket = [&](int nb, int want) -> bool {
-        const int j0 = 2 * tid, j1 = 2 * tid + 1;
-        const int c0 = j0 < nb ? hist[nb - 1 - j0] : 0;
-        const int c1 = j1 < nb ? hist[nb - 1 - j1] : 0;
-        int total;
-        const int ex = block_exclusive_scan(c0 + c1, warp_tmp, total);
-        if (ex < want && want <= ex + c0) {
-            sh_bucket = nb - 1 - j0;
-            sh_above = ex;
-            sh_count = c0;
-        } else if (ex + c0 < want && want <= ex + c0 + c1) {
-            sh_bucket = nb - 1 - j1;
-            sh_above = ex + c0;
-            sh_count = c1;
-        }
-        __syncthreads();
-        return total >= want;
+    const int span = hi - lo;
+    // whole 16-byte vectors of the span start at va; at most three scores at either end are left over
+    const int va = lo + (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(st + lo) & 15)) >> 2 & 3);
+    const int nv = hi > va ? (hi - va) >> 2 : 0;
+    const uint4* vec = reinterpret_cast<const uint4*>(st + va);
+    const int n_head = min(va, hi) - lo, n_end = max(hi - va - 4 * nv, 0);
+    const int pad = (4 - (va - lo)) & 3;  // a dense list keeps position lo + i - pad at index i: va falls on 16 bytes
+    // Short spans, and spans of which a large part is kept, are list entries as they are.
+    const bool dense = span + 3 <= list_words && (span <= kDense || k_mid > span / 4);
+    const int trips = (nv + kTrip - 1) / kTrip;
+    bool fast = hi <= kMapWords * 32;
+    auto prefetch_trip = [&](int t) {
+        const int v0 = t * kTrip;
+        if (v0 < nv) prefetch_l2(vec + v0, (uint32_t)min(kTrip, nv - v0) * 16u);
     };
-    for (int pass = 0; pass < 3; ++pass) {
-        const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-        const int nb = pass == 2 ? 1024 : 2048;
-        if (pass == 0 && have_hist) {
-            if (excl != 0xffffffffu) atomicSub(&hist[excl], 1);
-            for (int i = tid + kThreads; i < lo + (HL - hi); i += kThreads) {  // (more than 1024 positions outside)
+
+    // ---- the floor ----
+    uint32_t floor_bits = 0;
+    if (fast && !dense) {
+        int want = k_mid;
+        uint32_t u[8];
+        if (have_hist) {
+            __syncthreads();
+            for (int i = tid; i < lo + (HL - hi); i += kThreads) {  // positions outside the span that were counted
                 const int pos = i < lo ? i : hi + (i - lo);
-                atomicSub(&hist[__ldg(st + pos) >> 21], 1);
+                atomicSub(&sh.hist[__ldg(st + pos) >> 21], 1);
             }
         } else {
-            for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+            // 256 blocks of four vectors (64 bytes), evenly spread: eight scores per thread
+            uint4 s[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int k = (tid >> 2) + r * (kThreads / 4);
+                s[r] = load_vec(vec + (int)((int64_t)k * (nv - 4) / (kSample / 16 - 1)) + (tid & 3));
+            }
+            // rank in the sample: the expected one plus 6 sigma (neighbours may be alike), within what the list holds
+            const float r = (float)k_mid * kSample / span;
+            want = min((int)(r + 6.f * sqrtf(r) + 8.f), (int)(0.9f * cap * kSample / span));
+            u[0] = s[0].x; u[1] = s[0].y; u[2] = s[0].z; u[3] = s[0].w;
+            u[4] = s[1].x; u[5] = s[1].y; u[6] = s[1].z; u[7] = s[1].w;
             __syncthreads();
-            if (pass > 0 && use_list) {  // the candidates that share the first digit sit in shared memory
-                for (int i = tid; i < n_list; i += kThreads) {
-                    const uint32_t u = list[i];
-                    if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & (nb - 1)], 1);
-                }
-            } else if (pass == 0) {
-                // The first trip (8 K candidates) is counted in full; the bin in which ITS count reaches
-                // k_mid bounds the threshold's bin from below, so the remaining trips count only what
-                // lies at or above it: a few percent of the candidates instead of all of them (the
-                // counts below the threshold's bin are never looked at).
-                const int mid = min(hi, lo + 8 * kThreads);
-                sweep(st, lo, mid, [&](uint32_t u, int) { atomicAdd(&hist[u >> 21], 1); });
-                if (mid < hi) {
-                    __syncthreads();
-                    const uint32_t floor_bin = find_bucket(nb, need) ? (uint32_t)sh_bucket : 0u;
-                    sweep(st, mid, hi, [&](uint32_t u, int) {
-                        if ((u >> 21) >= floor_bin) atomicAdd(&hist[u >> 21], 1);
-                    });
-                }
-            } else {
-                sweep(st, lo, hi, [&](uint32_t u, int) {
-                    if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & (nb - 1)], 1);
-                });
+#pragma unroll
+            for (int k = 0; k < 8; ++k) atomicAdd(&sh.hist[sample_bin(u[k])], 1);
+        }
+        // The span is asked into L2 four trips (128 KB) ahead of the sweep: a trip waits for L2 and not for HBM.
+        if (tid < 4) prefetch_trip(tid);
+        __syncthreads();
+        fast = find_bucket(sh, want);
+        const uint32_t bin = (uint32_t)sh.bucket;
+        if (have_hist) {
+            floor_bits = bin << 21;
+            fast = fast && sh.above + sh.count <= cap;
+        } else {
+            floor_bits = kSampleBase + (bin << kSampleShift);
+            if (bin == 0u) {
+                floor_bits = 0u;
+            } else if (fast && sh.count * 4 > want) {  // flat scores, for which 2 % is a coarse step: eleven more bits
+                const int rest = want - sh.above;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (sample_bin(u[k]) == (int)bin) atomicAdd(&sh.hist[(u[k] >> (kSampleShift - 11)) & 2047u], 1);
+                __syncthreads();
+                find_bucket(sh, rest);
+                floor_bits |= (uint32_t)sh.bucket << (kSampleShift - 11);
             }
         }
+        floor_bits = max(floor_bits, 1u);  // (zero scores stay out: if they are needed the list is too short)
+    }
+
+    // ---- one sweep: the candidates at or above the floor ----
+    int n_list = 0;
+    if (fast) {
         __syncthreads();
-        find_bucket(nb, need);
-        prefix |= (uint32_t)sh_bucket << shift;
-        mask |= (uint32_t)(nb - 1) << shift;
-        need -= sh_above;
-        const int in_bucket = sh_count;
-        __syncthreads();
-        if (pass == 0 && in_bucket <= kCap) {
-            // One sweep collects the candidates of the threshold's bin (usually a few hundred of the tens
-            // of thousands) with their positions and marks everything above that bin in the position
-            // bitmap; the two remaining digits are then decided on the list instead of by two more
-            // sweeps over all scores.  A bin too full for the list (flat scores) keeps the sweeps.
-            if (tid == 0) list_n = 0;
-            for (int i = tid; i < map_words; i += kThreads) bitmap[i] = 0u;
-            __syncthreads();
-            const uint32_t bucket = prefix >> 21;
-            sweep(st, lo, hi, [&](uint32_t u, int pos) {
-                const uint32_t bin = u >> 21;
-                if (bin == bucket) {
-                    const int at = atomicAdd(&list_n, 1);
-                    if (at < kCap) {
-                        list[at] = u;
-                        lpos[at] = pos;
-                    }
-                } else if (bin > bucket && map_ok) {
-                    atomicOr(&bitmap[pos >> 5], 1u << (pos & 31));
+        uint32_t mx = 0u;
+        const bool edge = tid < n_head + n_end;  // this thread takes one of the scores outside the vectors
+        const int edge_pos = tid < n_head ? lo + tid : hi - n_end + (tid - n_head);
+        if (dense) {
+#pragma unroll 1
+            for (int i = tid; i < nv; i += kThreads) {
+                const uint4 w = load_vec(vec + i);
+                *reinterpret_cast<uint4*>(list + pad + (va - lo) + 4 * i) = w;
+                mx = max(mx, max(max(w.x, w.y), max(w.z, w.w)));
+            }
+            if (edge) {
+                const uint32_t u = __ldg(st + edge_pos);
+                list[pad + edge_pos - lo] = u;
+                mx = max(mx, u);
+            }
+        } else {
+            if (edge) {
+                const uint32_t u = __ldg(st + edge_pos);
+                const int at = u >= floor_bits ? atomicAdd(&sh.list_n, 1) : cap;
+                if (at < cap) {
+                    list[at] = u;
+                    lpos[at] = edge_pos;
                 }
+            }
+            const uint32_t list_s = (uint32_t)__cvta_generic_to_shared(list);
+            uint4 w[kV], x[kV];
+            auto load = [&](uint4 (&d)[kV], int base) {
+#pragma unroll
+                for (int k = 0; k < kV; ++k)
+                    d[k] = base + k * kThreads < nv ? load_vec(vec + base + k * kThreads) : make_uint4(0u, 0u, 0u, 0u);
+            };
+            load(w, tid);
+#pragma unroll 1
+            for (int t = 0; t < trips; ++t) {
+                const int base = t * kTrip + tid;
+                load(x, base + kTrip);
+                if (tid == 0) prefetch_trip(t + 4);
+                int mine = 4 * kV;  // hits: less the signs of (score - floor), without a branch
+#pragma unroll
+                for (int k = 0; k < kV; ++k)  // (scores past the end read as 0 and the floor is above 0)
+                    mine -= (int)(((w[k].x - floor_bits) >> 31) + ((w[k].y - floor_bits) >> 31) +
+                                  ((w[k].z - floor_bits) >> 31) + ((w[k].w - floor_bits) >> 31));
+                int inc = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                int at = 0;  // one shared counter update per warp
+                if (lane == 31 && inc) at = atomicAdd(&sh.list_n, inc);
+                at = __shfl_sync(0xffffffffu, at, 31) + inc - mine;
+                if (at + mine <= cap) {  // (a list that overflows is not used)
+                    uint32_t la = list_s + 4 * at;
+#pragma unroll
+                    for (int k = 0; k < kV; ++k) {
+                        const int pos = va + 4 * (base + k * kThreads);
+                        push_if(w[k].x, floor_bits, la, 4 * cap, pos);
+                        push_if(w[k].y, floor_bits, la, 4 * cap, pos + 1);
+                        push_if(w[k].z, floor_bits, la, 4 * cap, pos + 2);
+                        push_if(w[k].w, floor_bits, la, 4 * cap, pos + 3);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kV; ++k) w[k] = x[k];
+            }
+            __syncthreads();
+            const int n = min(sh.list_n, cap);
+#pragma unroll 1
+            for (int i = 4 * tid; i < n; i += 4 * kThreads) {
+                const uint4 q = *reinterpret_cast<const uint4*>(list + i);
+                mx = max(mx, max(max(q.x, i + 1 < n ? q.y : 0u), max(i + 2 < n ? q.z : 0u, i + 3 < n ? q.w : 0u)));
+            }
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) atomicMax(&sh.max, mx);
+        __syncthreads();
+        n_list = dense ? span : sh.list_n;
+        fast = n_list >= k_mid && (dense || n_list <= cap);
+    }
+
+    // ---- the threshold on the list: bins over its own range, refined until the threshold's bin is small ----
+    const int i0 = dense ? pad : 0, i1 = i0 + n_list;  // list entries
+    uint32_t bin_lo = floor_bits, width = 0xffffffffu;  // the threshold lies in [bin_lo, bin_lo + width)
+    int need = k_mid;                                   // entries to take from there
+    auto each_entry = [&](auto f) {  // f(bits, list index), four neighbouring entries per thread and trip
+#pragma unroll 1
+        for (int i = 4 * tid; i < i1; i += 4 * kThreads) {
+            const uint4 q = *reinterpret_cast<const uint4*>(list + i);
+            if (i >= i0) f(q.x, i);
+            if (i + 1 >= i0 && i + 1 < i1) f(q.y, i + 1);
+            if (i + 2 >= i0 && i + 2 < i1) f(q.z, i + 2);
+            if (i + 3 >= i0 && i + 3 < i1) f(q.w, i + 3);
+        }
+    };
+    if (fast) {
+        int shift = max(0, 21 - __clz((int)(sh.max - floor_bits)));
+#pragma unroll 1
+        for (;;) {
+            each_entry([&](uint32_t u, int) {
+                const uint32_t d = u - bin_lo;
+                if (d < width) atomicAdd(&sh.hist[d >> shift], 1);
             });
             __syncthreads();
-            n_list = list_n;
-            use_list = n_list <= kCap;
-        }
-    }
-    const uint32_t thr = prefix;  // take every candidate > thr and the first `need` equal to it
-
-    bool off_map = use_list && map_ok;
-    int n_eq = 0;
-    int* eqpos = hist;  // the tie positions reuse the histogram's storage
-    if (off_map) {
-        // list entries above the threshold join the bitmap; the ties (bit pattern equal to the
-        // threshold) are set aside
-        if (tid == 0) list_n = 0;
-        __syncthreads();
-        for (int i = tid; i < n_list; i += kThreads) {
-            const uint32_t u = list[i];
-            const int pos = lpos[i];
-            if (u > thr) {
-                atomicOr(&bitmap[pos >> 5], 1u << (pos & 31));
-            } else if (u == thr) {
-                const int at = atomicAdd(&list_n, 1);
-                if (at < kBins) eqpos[at] = pos;
+            find_bucket(sh, need);
+            need -= sh.above;
+            bin_lo += (uint32_t)sh.bucket << shift;
+            width = 1u << shift;
+            if (sh.count <= kPair) break;
+            if (shift == 0) {  // more than a thousand equal scores at the threshold
+                fast = false;
+                break;
             }
+            shift = max(0, shift - 11);
+            __syncthreads();  // (sh.bucket and its fellows are read before the next search writes them)
         }
         __syncthreads();
-        n_eq = list_n;
-        off_map = n_eq <= kBins;  // (thousands of equal scores: the ordered compaction below handles them)
     }
-    if (off_map) {
-        // ---- the index set off the bitmap ----
-        // the ties are ranked by position among themselves and the lowest `need` join
-        for (int i = tid; i < n_eq; i += kThreads) {
-            const int pos = eqpos[i];
-            int rank = 0;
-            if (n_eq > need)
-                for (int j = 0; j < n_eq; ++j) rank += eqpos[j] < pos ? 1 : 0;
-            if (rank < need) atomicOr(&bitmap[pos >> 5], 1u << (pos & 31));
-        }
-        __syncthreads();
-        uint32_t w[4];
-        int cnt = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            w[k] = (k < wpt && wpt * tid + k < map_words) ? bitmap[wpt * tid + k] : 0u;
-            cnt += __popc(w[k]);
-        }
-        int total;
-        int at = k_sink + block_exclusive_scan(cnt, warp_tmp, total);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t m = w[k];
-            while (m) {
-                const int bit = __ffs(m) - 1;
-                m &= m - 1;
-                out[at++] = (wpt * tid + k) * 32 + bit;
-            }
-        }
+    if (!fast) {
+        select_by_sweeps(sh, st, lo, hi, k_mid, out + k_sink);
         return;
     }
-
-    // ---- ordered compaction over the candidate span (flat scores or very long contexts) ----
-    // One block scan per trip: the counts of "above the threshold" (high half) and "equal to it" (low
-    // half) travel in one word; a candidate's slot is (candidates above it so far) + (equal ones so far,
-    // capped at the number still needed).
-    int gt_seen = 0, eq_seen = 0;
-    for (int base = lo; base < hi; base += kThreads * kItems) {
-        const int i0 = base + tid * kItems;
-        uint32_t u[kItems];
-        int packed = 0;
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            u[k] = (i0 + k < hi) ? __ldg(st + i0 + k) : 0u;
-            if (i0 + k < hi) packed += u[k] > thr ? (1 << 16) : (u[k] == thr ? 1 : 0);
+    // above the bin: chosen; inside: set aside and ranked pair by pair
+    uint32_t* pu = reinterpret_cast<uint32_t*>(sh.hist);
+    int* pp = sh.hist + kPair;
+    each_entry([&](uint32_t u, int i) {
+        const uint32_t d = u - bin_lo;
+        if ((int)d < 0) return;  // below the bin (scores and their differences stay below 2^31)
+        const int pos = dense ? lo + i - pad : lpos[i];
+        if (d >= width) {
+            atomicOr(&sh.bitmap[pos >> 5], 1u << (pos & 31));
+        } else {
+            const int at = atomicAdd(&sh.pair_n, 1);
+            pu[at] = u;
+            pp[at] = pos;
         }
-        int total;
-        const int ex = block_exclusive_scan(packed, warp_tmp, total);
-        int gt = gt_seen + (ex >> 16), eq = eq_seen + (ex & 0xffff);
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            if (i0 + k < hi) {
-                if (u[k] > thr) {
-                    out[k_sink + gt + min(eq, need)] = i0 + k;
-                    ++gt;
-                } else if (u[k] == thr) {
-                    if (eq < need) out[k_sink + gt + eq] = i0 + k;
-                    ++eq;
-                }
-            }
+    });
+    __syncthreads();
+    const int np = sh.pair_n;
+#pragma unroll 1
+    for (int e = tid >> 3; e < np; e += kThreads / 8) {  // eight lanes per entry
+        const uint32_t u = pu[e];
+        const int pos = pp[e];
+        int rank = 0;
+#pragma unroll 2
+        for (int j = tid & 7; j < np; j += 8) {
+            const uint32_t v = pu[j];
+            rank += (v > u) | ((v == u) & (pp[j] < pos));
         }
-        gt_seen += total >> 16;
-        eq_seen += total & 0xffff;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffu << (lane & 24), rank, o);
+        if ((tid & 7) == 0 && rank < need) atomicOr(&sh.bitmap[pos >> 5], 1u << (pos & 31));
     }
+    __syncthreads();
+    // ---- the index set off the bitmap: consecutive words per thread, gathered in the list's storage (read for the
+    // last time above) so that the store is coalesced ----
+    const int wpt = (hi + 32 * kThreads - 1) / (32 * kThreads);  // at most eight
+    const uint32_t* bits = sh.bitmap + wpt * tid;
+    int cnt = 0;
+#pragma unroll 1
+    for (int k = 0; k < wpt; ++k) cnt += __popc(bits[k]);
+    int at = block_exclusive_scan(sh, cnt);
+#pragma unroll 1
+    for (int k = 0; k < wpt; ++k) {
+        const int pos0 = 32 * (wpt * tid + k) - 1;
+#pragma unroll 1
+        for (uint32_t m = bits[k]; m; m &= m - 1) list[at++] = (uint32_t)(pos0 + __ffs((int)m));
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < k_mid; i += kThreads) out[k_sink + i] = (int)list[i];
 }
 
 // Top-11-bit counts of stats[prob][0 : len[b]) for the verification kernels that do not count while
@@ -336,17 +515,21 @@ int select_launch(const float* stats, int64_t stat_stride, int n_layers, int bat
                   int32_t* n_indices, uint32_t* hist, const int32_t* hist_len, cudaStream_t stream)
 {
     const long probs = (long)n_layers * batch * n_kv_heads;
-    static bool opted_in[64] = {};  // per device: the kernel's dynamic shared memory exceeds the default limit
+    static std::atomic<bool> opted_in[64] = {};  // per device: the kernel's dynamic shared memory exceeds the default limit
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPEC_ERR_CUDA;
     if (!opted_in[dev]) {
-        if (cudaFuncSetAttribute(select_recall_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem) !=
-            cudaSuccess)
+        if (cudaFuncSetAttribute(select_recall_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kListWords * 4) != cudaSuccess)
             return SPEC_ERR_CUDA;
         opted_in[dev] = true;
     }
-    select_recall_kernel<<<(unsigned)probs, kThreads, kDynSmem, stream>>>(
-        stats, stat_stride, batch, n_kv_heads, sel_len, k_sink, k_recent, k_total, indices, n_indices, hist, hist_len);
+    // no context is longer than a row of scores: short rows take less shared memory, and more CTAs share an SM
+    const int64_t row = (stat_stride + 7) / 4 * 4;
+    const int list_words = (int)(row < kListWords ? row : kListWords);
+    select_recall_kernel<<<(unsigned)probs, kThreads, (size_t)list_words * 4, stream>>>(
+        stats, stat_stride, batch, n_kv_heads, sel_len, k_sink, k_recent, k_total, list_words, indices, n_indices, hist,
+        hist_len);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
 }

@@ -1,0 +1,51 @@
+"""Selection at the edges of its forms: spans at and around the dense list's length and a sweep trip, rows that do not
+start on 16 bytes, flat scores, scores whose large values sit in one stretch or only between the sample's blocks, zeros,
+hundreds of equal scores at the threshold.  Integer work: bit-exact against the oracle."""
+import pytest
+import torch
+
+import oracle
+from paper_2607_27735_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def check(stats, sel_len, k_sink, k_recent, k_total):
+    idx, n = binding.spec_select_recall(stats, sel_len, k_sink, k_recent, k_total)
+    r_idx, r_n = oracle.select_recall(stats.cpu(), sel_len.cpu(), k_sink, k_recent, k_total)
+    assert torch.equal(idx.cpu(), r_idx) and torch.equal(n.cpu(), r_n)
+
+
+# span = T - 68: 4096 is the longest dense one at a small budget, 8192 scores are a trip of the sweep
+@pytest.mark.parametrize("span", [510, 4095, 4096, 4097, 8192, 8195, 20477, 20480, 40961])
+@pytest.mark.parametrize("keep", [3, 400, "half"])
+def test_spans_and_unaligned_rows(span, keep):
+    g = torch.Generator(device="cuda").manual_seed(span)
+    T = span + 68
+    k_mid = span // 2 if keep == "half" else keep
+    stats = torch.randn(1, 2, 3, T + 5, generator=g, device="cuda").exp_()  # row starts cycle through all alignments
+    sel_len = torch.tensor([T, T - 1], dtype=torch.int32, device="cuda")
+    check(stats, sel_len, 4, 64, k_mid + 68)
+
+
+@pytest.mark.parametrize("T", [6000, 33333])
+@pytest.mark.parametrize("kind", ["flat", "one_stretch", "between_samples", "zeros", "ties"])
+def test_distributions(T, kind):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    stats = torch.rand(1, 2, 2, T, generator=g, device="cuda")
+    if kind == "flat":
+        stats = 0.5 + 1e-5 * stats
+    elif kind == "one_stretch":
+        stats[..., T // 3:T // 3 + 1500] += 10.0
+    elif kind == "between_samples":  # a sample of every fourth vector of a stretch of 16 sees none of the large ones
+        big = torch.zeros(T, dtype=torch.bool, device="cuda")
+        big[68:] = (torch.arange(T - 68, device="cuda") * 256 // (T - 68)) % 7 == 3
+        stats = torch.where(big, stats + 10.0, stats)
+    elif kind == "zeros":
+        stats = torch.where(stats > 0.99, stats, torch.zeros_like(stats))
+    else:
+        kth = stats[..., 4:T - 71].topk(932, dim=-1).values[..., -1:]
+        where = torch.rand(1, 2, 2, T, generator=g, device="cuda").argsort(dim=-1)[..., :700]
+        stats.scatter_(-1, where, kth.expand(1, 2, 2, 700).contiguous())
+    sel_len = torch.tensor([T, T - 7], dtype=torch.int32, device="cuda")
+    check(stats.contiguous(), sel_len, 4, 64, 1000)
