@@ -14,6 +14,7 @@ constexpr int kTile = 128;            // keys per tile = UMMA M
 constexpr int kD = 128;               // head_dim the tiles are laid out for (head_dim 64 uses the lower half)
 constexpr int kSlotBytes = 32768;     // one K or V tile: 2 halves x 128 rows x 128 B (SW128)
 constexpr int kThreads = 384;
+constexpr int kMaxClass = 4;          // whole teams, then halves, quarters and eighths
 constexpr int kRing = 4;              // partial buffers are recycled every kRing units
 constexpr uint64_t kEvictFirst = 0x12F0000000000000ull;
 constexpr uint64_t kEvictLast = 0x14F0000000000000ull;
@@ -28,10 +29,17 @@ struct FastParams {
     int D;                            // head_dim: 128, or 64 (score-cache kernel only)
     int box_rows, boxes;              // TMA boxes per 64-wide half of a tile
     float scale_log2;
-    int* counters;                    // [2][n_units * HG]: P1 partials done, O partials done; then one
+    // score-cache kernel: HG teams of cph CTAs; sequences short enough run on a team's parts (see Sched)
+    int n_cls;                        // classes in use
+    int cls_size[kMaxClass];          // CTAs of a part
+    int cls_subs[kMaxClass];          // parts of a team
+    int n_sid;                        // parts of all teams in the finest class
+    int n_counters;                   // ints to zero at the end, the "CTAs finished" word being the one after them
+    int* counters;                    // two-sweep: [2][n_units * HG]: P1 partials done, O partials done; score cache:
+                                      // [3][n_units * n_sid], the third: reductions done; then one
                                       // "CTAs finished" word.  All zero between calls.
-    float2* ml_part;                  // [kRing][HG][cph][R]
-    float* o_part;                    // [kRing][HG][cph][R][kD] (columns >= head_dim unused)
+    float2* ml_part;                  // [kRing][CTAs][R]
+    float* o_part;                    // [kRing][CTAs][R][kD] (columns >= head_dim unused)
     int* status;
     int n_pages;
     int n_cache;                      // S tiles the TMEM cache holds (cached variant)
@@ -285,7 +293,7 @@ int launch_cached(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMa
 // costs more than the whole prologue of this kernel).  Call after the CTA's last use of them.
 __device__ __forceinline__ void reset_counters_if_last(const FastParams& p, int* smem_flag)
 {
-    const int n = 2 * p.n_units * p.HG;
+    const int n = p.n_counters;
     if (threadIdx.x == 0) {
         __threadfence();
         *smem_flag = atomicAdd(p.counters + n, 1) == (int)gridDim.x - 1;

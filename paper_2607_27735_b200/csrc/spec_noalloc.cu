@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "spec_common.cuh"
+#include "verify_sm100.cuh"
 
 namespace {
 
@@ -56,10 +57,13 @@ int spec_verify_attn_noalloc(const spec_kv_t* kv, const void* q, int32_t n_q, co
     const int rc = scratch_address(&scratch);
     if (rc != SPEC_OK) return rc;
     // The array keeps whatever the previous call left (possibly laid out for another shape): the
-    // cross-CTA counters behind the status block (at most two per (layer, sequence, KV head) plus
-    // one) must start at zero.  The status word itself is left alone, so that an error nobody has
-    // read yet survives until spec_noalloc_read_status(), as with a caller's workspace.
-    size_t head = (2 * (size_t)kv->n_layers * kv->batch * kv->n_kv_heads + 1) * sizeof(int) + 256;
+    // cross-CTA counters behind the status block must start at zero.  The status word itself is left alone, so that
+    // an error nobody has read yet survives until spec_noalloc_read_status(), as with a caller's workspace.
+    spec::KvView shape = {};
+    shape.n_layers = kv->n_layers;
+    shape.batch = kv->batch;
+    shape.n_kv_heads = kv->n_kv_heads;
+    size_t head = spec::verify_counter_bytes(shape);
     if (spec::kStatusBytes + head > need) head = need > spec::kStatusBytes ? need - spec::kStatusBytes : 0;
     if (head > 0 && cudaMemsetAsync(static_cast<char*>(scratch) + spec::kStatusBytes, 0, head,
                                     static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)

@@ -32,6 +32,7 @@ EncodeTiledFn encode_fn()
 struct Plan {
     bool cached;
     int HG, cph, n_units, N, n_slots, p_bufs, box_rows, boxes, n_cache, n_raw;
+    int n_cls, cls_size[kMaxClass], cls_subs[kMaxClass], n_sid, n_counters;
     size_t smem_bytes;
     size_t ctr_off, ctr_bytes, ml_off, o_off, total;
 };
@@ -63,21 +64,31 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
 
     int best_hg = 0;
     bool cached = false;
-    if (variant != 1) {  // score-cache kernel: a CTA's share of a head must fit the TMEM cache
-        double best = -1.0;
-        for (int hg = 1; hg <= kv.n_kv_heads; ++hg) {
-            if (kv.n_kv_heads % hg) continue;
-            const int cph = nsm / hg;
-            if (cph < 1) continue;
+    int best_cph = 0;
+    if (variant != 1) {
+        // Score-cache kernel: HG teams of cph CTAs, each team a problem (one KV head of one (layer, sequence)) at a
+        // time.  A CTA's share of the longest context must fit the TMEM cache; among the team sizes that do, the
+        // one with the least time by a simple model: rounds of problems x (fixed cycles of a round + cycles of a
+        // key tile's K and V at the SM's share of HBM x tiles per CTA).  A round of a team of one has no exchange
+        // between CTAs.  (Shorter sequences of the batch may run on parts of a team: see Sched in the kernel.)
+        const long probs = lb * kv.n_kv_heads;
+        double best = 1e300;
+        for (int cph = nsm < nb ? nsm : nb; cph >= 1; --cph) {
             const int tpc = (nb + cph - 1) / cph;
-            if (tpc > n_cache) continue;
-            const double score = (double)nb * hg / ((double)nsm * tpc) + 0.001 * hg;
-            if (score > best) {
-                best = score;
-                best_hg = hg;
+            if (tpc > n_cache) break;
+            int teams = nsm / cph;
+            if (teams > probs) teams = (int)probs;
+            const long rounds = (probs + teams - 1) / teams;
+            const double t = (double)rounds * ((cph > 1 ? 9000.0 : 6000.0) + 2900.0 * tpc);
+            if (t < best) {
+                best = t;
+                best_hg = teams;
+                best_cph = cph;
             }
         }
         cached = best_hg != 0;
+        // CTAs that the teams leave over join them
+        if (cached && best_cph < nb) best_cph = nsm / best_hg < nb ? nsm / best_hg : nb;
     }
     if (!cached) {
         if (variant == 2 || kv.head_dim != kD || kv.fp8) return false;
@@ -102,8 +113,19 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     pl->cached = cached;
     pl->n_cache = n_cache;
     pl->HG = best_hg;
-    pl->cph = nsm / best_hg;
-    pl->n_units = (int)(lb * (kv.n_kv_heads / best_hg));
+    pl->cph = cached ? best_cph : nsm / best_hg;
+    pl->n_units = cached ? (int)((lb * kv.n_kv_heads + best_hg - 1) / best_hg) : (int)(lb * (kv.n_kv_heads / best_hg));
+    pl->n_cls = 1;
+    pl->cls_size[0] = pl->cph;
+    pl->cls_subs[0] = 1;
+    for (int f = 1; cached && f < kMaxClass && (pl->cph >> f) >= 1; ++f) {
+        pl->cls_size[f] = pl->cph >> f;
+        pl->cls_subs[f] = pl->cph / pl->cls_size[f];
+        pl->n_cls = f + 1;
+    }
+    pl->n_sid = pl->HG * pl->cls_subs[pl->n_cls - 1];
+    // score cache: every class may end in a round that is not full
+    pl->n_counters = cached ? 3 * (pl->n_units + kMaxClass) * pl->n_sid : 2 * pl->n_units * pl->HG;
     pl->N = N;
     pl->box_rows = box_rows;
     pl->boxes = kTile / box_rows;
@@ -158,7 +180,7 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     pl->smem_bytes = fixed + (size_t)slots * kSlotBytes;
     size_t off = kStatusBytes;
     pl->ctr_off = off;
-    pl->ctr_bytes = ((size_t)2 * pl->n_units * pl->HG + 1) * sizeof(int);
+    pl->ctr_bytes = verify_counter_bytes(kv);
     off += pl->ctr_bytes;
     off = (off + 255) & ~(size_t)255;
     pl->ml_off = off;
@@ -267,6 +289,14 @@ __global__ void add_stats_kernel(float* stats, int64_t stat_stride, const float*
 }
 
 }  // namespace
+
+// A team has at most 15 parts (cph / (cph >> 3)) and the parts of all teams are at most one per SM, so the counters
+// of a plan, 3 (units + kMaxClass) parts, stay below this whatever the split.
+size_t verify_counter_bytes(const KvView& kv)
+{
+    const size_t probs = (size_t)kv.n_layers * kv.batch * kv.n_kv_heads;
+    return (3 * (16 * probs + (kMaxClass + 1) * (size_t)sm_count()) + 1) * sizeof(int);
+}
 
 bool verify_sm100_supported(const KvView& kv, int n_q, int variant)
 {
@@ -392,13 +422,21 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
     FastParams fp;
     fp.a = a;
     fp.HG = pl.HG;
-    fp.NHG = a.kv.n_kv_heads / pl.HG;
+    fp.NHG = pl.cached ? 1 : a.kv.n_kv_heads / pl.HG;
     fp.cph = pl.cph;
-    set_divisor(&fp, 0, a.kv.batch * fp.NHG);
-    set_divisor(&fp, 1, fp.NHG);
+    // two-sweep: units per layer and head groups per sequence; score cache: problems per sequence and KV heads
+    set_divisor(&fp, 0, pl.cached ? a.kv.n_layers * a.kv.n_kv_heads : a.kv.batch * fp.NHG);
+    set_divisor(&fp, 1, pl.cached ? a.kv.n_kv_heads : fp.NHG);
     set_divisor(&fp, 2, fp.cph);
+    fp.n_cls = pl.n_cls;
+    for (int f = 0; f < pl.n_cls; ++f) {
+        fp.cls_size[f] = pl.cls_size[f];
+        fp.cls_subs[f] = pl.cls_subs[f];
+    }
+    fp.n_sid = pl.n_sid;
+    fp.n_counters = pl.n_counters;
     set_divisor(&fp, 3, a.kv.n_q_heads / a.kv.n_kv_heads);
-    fp.n_units = pl.n_units;
+    fp.n_units = pl.cached ? pl.n_units + kMaxClass : pl.n_units;
     fp.N = pl.N;
     fp.R = a.n_q * G;
     fp.G = G;

@@ -7,6 +7,9 @@ namespace spec {
 // else the two-sweep kernel), 1 = two-sweep only, 2 = score-cache only
 bool verify_sm100_supported(const KvView& kv, int n_q, int variant);
 size_t verify_sm100_workspace(const KvView& kv, int n_q, int max_ctx_len);
+// Bytes behind the status block that the cross-CTA counters of a call may take: the same for every split of the same
+// number of problems, so that calls with different row counts may share a workspace.
+size_t verify_counter_bytes(const KvView& kv);
 // Clears the status word itself; *used_variant gets 1 (two-sweep) or 2 (score-cache).
 int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, int* used_variant);
 // whether that call would accept the arguments (nothing is launched)
