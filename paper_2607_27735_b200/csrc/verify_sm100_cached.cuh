@@ -46,18 +46,24 @@ namespace {
 constexpr int kMaxCache = 32;
 constexpr int kLsePubMax = 48;  // CTAs per head up to which the publisher warp alone combines the LSE partials
 
-// Cross-lane reduction of per-column (max, sum of exp2(x - max)) pairs.  While the number of
-// columns a lane carries is even, partners exchange halves (the lane with bit `o` set keeps the
-// upper half), so the traffic halves at every step; an odd count is reduced in place on both
-// partners.  Afterwards a lane holds ml_final_n(NH) columns starting at `col`, and lanes that
-// differ only in the bits of ml_dupmask(NH) hold the same ones.
-__host__ __device__ constexpr int ml_final_n(int n)
+// Largest of the 32 lanes' values, on every lane.
+__device__ __forceinline__ float warp_max_all(float x)
+{
+    float y;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Sums over the 32 lanes of n columns per lane.  While the number of columns a lane carries is even, partners exchange
+// halves (the lane with bit `o` set keeps the upper half), so the traffic halves at every step; an odd count is
+// summed in place on both partners.  Afterwards a lane holds sum_final_n(n) columns starting at `col`, and lanes that
+// differ only in the bits of sum_dupmask(n) hold the same ones.
+__host__ __device__ constexpr int sum_final_n(int n)
 {
     for (int o = 16; o >= 1; o >>= 1)
         if (n % 2 == 0) n /= 2;
     return n;
 }
-__host__ __device__ constexpr uint32_t ml_dupmask(int n)
+__host__ __device__ constexpr uint32_t sum_dupmask(int n)
 {
     uint32_t d = 0;
     for (int o = 16; o >= 1; o >>= 1) {
@@ -67,7 +73,7 @@ __host__ __device__ constexpr uint32_t ml_dupmask(int n)
     return d;
 }
 template <int NHT, int n, int o>
-__device__ __forceinline__ void ml_step(float (&m)[NHT], float (&l)[NHT], int lane, int& col)
+__device__ __forceinline__ void sum_step(float (&l)[NHT], int lane, int& col)
 {
     if constexpr (o >= 1) {
         if constexpr (n % 2 == 0) {
@@ -75,24 +81,15 @@ __device__ __forceinline__ void ml_step(float (&m)[NHT], float (&l)[NHT], int la
             const bool up = (lane & o) != 0;
 #pragma unroll
             for (int j = 0; j < h; ++j) {
-                const float sm = up ? m[j] : m[j + h], sl = up ? l[j] : l[j + h];
-                const float km = up ? m[j + h] : m[j], kl = up ? l[j + h] : l[j];
-                const float rm = __shfl_xor_sync(0xffffffffu, sm, o), rl = __shfl_xor_sync(0xffffffffu, sl, o);
-                const float M = fmaxf(km, rm);
-                m[j] = M;
-                l[j] = kl * ex2(km - M) + rl * ex2(rm - M);
+                const float give = up ? l[j] : l[j + h], keep = up ? l[j + h] : l[j];
+                l[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
             }
             col += up ? h : 0;
-            ml_step<NHT, h, o / 2>(m, l, lane, col);
+            sum_step<NHT, h, o / 2>(l, lane, col);
         } else {
 #pragma unroll
-            for (int j = 0; j < n; ++j) {
-                const float rm = __shfl_xor_sync(0xffffffffu, m[j], o), rl = __shfl_xor_sync(0xffffffffu, l[j], o);
-                const float M = fmaxf(m[j], rm);
-                l[j] = l[j] * ex2(m[j] - M) + rl * ex2(rm - M);
-                m[j] = M;
-            }
-            ml_step<NHT, n, o / 2>(m, l, lane, col);
+            for (int j = 0; j < n; ++j) l[j] += __shfl_xor_sync(0xffffffffu, l[j], o);
+            sum_step<NHT, n, o / 2>(l, lane, col);
         }
     }
 }
@@ -184,6 +181,24 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
 }
 __device__ __forceinline__ Work get_work(const Sched& sc, int unit) { return sc.work[unit % kWorkTab]; }
 
+// The waits of this kernel poll the abort flag and carry no clock of their own: whatever they wait for comes from the
+// MMA warp, whose idle timer is the watchdog of all of them, or follows a cross-CTA counter, whose wait is timed
+// (counter_wait).  A timer inlined at each of the thirty sites made the function 12 KB longer, and code that does not
+// fit the instruction cache is fetched again every unit.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const Ctl& c)
+{
+    while (!mbar_try_wait(bar, parity))
+        if (*c.abort_flag) return false;
+    return true;
+}
+// Barrier among the softmax warps, on an mbarrier so that the wait can be abandoned.
+__device__ __forceinline__ bool warps_sync(uint32_t bar, uint32_t& n, const Ctl& c)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+    return bar_wait(bar, n++ & 1, c);
+}
+
 struct CBars {  // mbarrier addresses (shared space)
     uint32_t slot_full, slot_empty, q_full, q_empty, s_full, s_free, p_full, p_empty, o_full, o_empty, sm_sync,
         pub_p1, pub_o, lse_ready, raw_full, raw_empty, q_ready;
@@ -245,12 +260,13 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         B.raw_empty = o; o += 32; // F8: every softmax warp has expanded its part of the stage
         B.q_ready = o; o += 8;    // F8: Q is fp16 in shared memory
     }
-    float* lse_s = reinterpret_cast<float*>(misc + 1024);                 // [128] global row LSE (log2 domain)
+    int* roff_s = reinterpret_cast<int*>(misc + 1024);                    // [128] offset of a row in the output, from row 0
     float* loc_s = reinterpret_cast<float*>(misc + 1024 + 512);           // [128] CTA-local row LSE
     float* fac_s = reinterpret_cast<float*>(misc + 2048);                 // [128] exp2(local - global)
     uint32_t* hist_s = reinterpret_cast<uint32_t*>(misc + 2560);          // [1024] packed 16-bit counts of score bins, 4 KB
     Sched& sc = *reinterpret_cast<Sched*>(misc + 6656);
-    float2* red = reinterpret_cast<float2*>(misc + 8192);                 // [kSW warps][NC] (m, l), <= 4 KB
+    float* red_m = reinterpret_cast<float*>(misc + 8192);                 // [kSW warps][NC], <= 2 KB
+    float* red_l = red_m + 512;                                           // the same
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 12288);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -298,8 +314,11 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             *reinterpret_cast<uint4*>(sgen + (s_slots - sbase) + (i >> 10) * kSlotBytes + 16384 + 16 * (i & 1023)) =
                 make_uint4(0, 0, 0, 0);
     }
+    if (threadIdx.x < R) {
+        const int j = fast_div(p, 3, threadIdx.x);
+        roff_s[threadIdx.x] = (j * p.a.kv.n_q_heads + (threadIdx.x - j * G)) * p.D;
+    }
     for (int r = R + threadIdx.x; r < 128; r += kBlock) {  // padded rows: P = 0
-        lse_s[r] = 1.0e30f;
         loc_s[r] = 1.0e30f;
         fac_s[r] = 0.f;
     }
@@ -319,7 +338,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     const uint32_t tmem_base = *tmem_slot;
     {  // the schedule (see Sched): lengths, their order, classes
         const int B = p.a.kv.batch;
-        int* raw = reinterpret_cast<int*>(red);
+        int* raw = reinterpret_cast<int*>(red_m);
         int T = 0;
         const bool sorted = B <= kSortMax;
         if (threadIdx.x < kMaxClass) sc.cnt[threadIdx.x] = 0;
@@ -330,6 +349,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         __syncthreads();
         if (sorted && threadIdx.x < B) {
             int before = 0;
+#pragma unroll 1
             for (int j = 0; j < B; ++j) before += (raw[j] > T || (raw[j] == T && j < (int)threadIdx.x)) ? 1 : 0;
             sc.ord[before] = (uint16_t)threadIdx.x;
             const int nb = (T + kTile - 1) / kTile;
@@ -342,6 +362,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const int LH = p.a.kv.n_layers * p.a.kv.n_kv_heads;
             sc.sorted = sorted ? 1 : 0;
             if (!sorted) sc.cnt[0] = B;
+#pragma unroll 1
             for (int f = p.n_cls - 1; f > 0; --f) {
                 if (2 * sc.cnt[f] * LH <= p.HG * p.cls_subs[f]) {
                     sc.cnt[f - 1] += sc.cnt[f];
@@ -349,6 +370,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 }
             }
             int u = 0, q = 0;
+#pragma unroll 1
             for (int f = 0; f < kMaxClass; ++f) {
                 sc.unit0[f] = u;
                 sc.seq0[f] = q;
@@ -371,7 +393,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
     if (warp == 0) {
         // =========================== TMA producer ===========================
-        uint32_t slot_idx = 0, qn = 0;
+        uint32_t ring = 0, ring_ph = 0, qn = 0;  // next slot (F8: raw stage), its phase; Q buffers filled
         const int boxes = p.boxes, box_rows = p.box_rows;
         const uint32_t box_bytes = box_rows * 128;
         const int halves = p.D / 64;  // 64-wide halves of the head dimension
@@ -379,10 +401,13 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         auto load_tile = [&](const CUtensorMap* map, const Work& sg, int tile) -> bool {
             if (F8) {
                 // the tile's bytes (128 per key) go to a raw stage; the softmax warps expand them into a slot
-                const uint32_t r = slot_idx % p.n_raw, rph = (slot_idx / p.n_raw) & 1;
-                ++slot_idx;
+                const uint32_t r = ring, rph = ring_ph;
+                if (++ring == (uint32_t)p.n_raw) {
+                    ring = 0;
+                    ring_ph ^= 1;
+                }
                 bool got = true;
-                if (lane == 0) got = mbar_wait(B.raw_empty + 8 * r, rph ^ 1, ctl, 3);
+                if (lane == 0) got = bar_wait(B.raw_empty + 8 * r, rph ^ 1, ctl);
                 if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
                 const int key0 = tile * kTile;
                 const int n_box = min(boxes, (sg.T - key0 + box_rows - 1) / box_rows);
@@ -403,10 +428,13 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 __syncwarp();
                 return true;
             }
-            const uint32_t s = slot_idx % p.n_slots, ph = (slot_idx / p.n_slots) & 1;
-            ++slot_idx;
+            const uint32_t s = ring, ph = ring_ph;
+            if (++ring == (uint32_t)p.n_slots) {
+                ring = 0;
+                ring_ph ^= 1;
+            }
             bool got = true;
-            if (lane == 0) got = mbar_wait(B.slot_empty + 8 * s, ph ^ 1, ctl, 1);  // one lane polls
+            if (lane == 0) got = bar_wait(B.slot_empty + 8 * s, ph ^ 1, ctl);  // one lane polls
             if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
             // boxes of this tile that hold at least one key < T (pages past the context may not exist)
             const int key0 = tile * kTile;
@@ -441,15 +469,15 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             }
             const Work sg = get_work(sc, u);
             if (!sg.valid()) continue;
-            const uint32_t qb = 0, qph = qn & 1;
+            const uint32_t qph = qn & 1;
             ++qn;
-            ok = mbar_wait(B.q_empty + 8 * qb, qph ^ 1, ctl, 2);
+            ok = bar_wait(B.q_empty, qph ^ 1, ctl);
             if (!ok) break;
             if (lane == 0) {
-                mbar_expect_tx(B.q_full + 8 * qb, (uint32_t)halves * R * 128);
+                mbar_expect_tx(B.q_full, (uint32_t)halves * R * 128);
                 const int row0 = (sg.layer * p.a.kv.batch + sg.b) * p.a.n_q;
-                tma_load_3d(s_q + qb * q_bytes, &tm_q, B.q_full + 8 * qb, 0, sg.h * G, row0);
-                if (halves == 2) tma_load_3d(s_q + qb * q_bytes + N * 128, &tm_q, B.q_full + 8 * qb, 64, sg.h * G, row0);
+                tma_load_3d(s_q, &tm_q, B.q_full, 0, sg.h * G, row0);
+                if (halves == 2) tma_load_3d(s_q + N * 128, &tm_q, B.q_full, 64, sg.h * G, row0);
             }
             __syncwarp();
             for (int t = sg.t0; t < sg.t1 && ok; ++t) ok = load_tile(&tm_k, sg, t);
@@ -471,121 +499,108 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             // Two independent queues, issued in whichever order their inputs become ready: the
             // QK^T tiles of unit u+1 may overtake the P V tiles of unit u that still wait for P.
             struct Queue {
-                int u = -1, t = 0, t0 = 0, t1 = 0;
-                uint32_t slot_base = 0;  // ring index of the unit's first K tile
-                uint32_t next_base = 0;  // ring index where the following unit starts
-                uint32_t qn = 0, qb = 0, qph = 0;
-                bool done = false, pending = false;  // pending: the next unit is not in the table yet
+                int u = -1, c = 0, n_t = 0;   // unit, its tile, its tiles
+                uint32_t slot = 0, ph = 0;    // ring position of the tile and the slot's phase
+                bool seek = true, done = false;
             } qq, pq;
-            auto seek = [&](Queue& c) {  // advance to the next unit with tiles
-                for (;;) {
-                    c.pending = false;
-                    if (c.u + 1 >= U) {
-                        c.done = true;
-                        return;
-                    }
-                    if (c.u + 1 >= sc.limit) {
-                        c.pending = true;
-                        return;
-                    }
+            // slots of a unit: its K tiles, then its V tiles
+            auto skip = [&](Queue& c, int n) {
+                c.slot += n;
+                while (c.slot >= (uint32_t)p.n_slots) {
+                    c.slot -= p.n_slots;
+                    c.ph ^= 1;
+                }
+            };
+            auto seek = [&](Queue& c, bool v) {  // on to the next unit with work, as far as the table goes
+                skip(c, v ? 0 : c.n_t);          // past the V tiles of the unit left behind
+                c.n_t = 0;
+                while (c.u + 1 < U && c.u + 1 < sc.limit) {
                     ++c.u;
                     const Work sg = get_work(sc, c.u);
                     if (sg.valid()) {
-                        c.t0 = sg.t0;
-                        c.t1 = sg.t1;
-                        c.t = sg.t0;
-                        c.slot_base = c.next_base;
-                        c.next_base += 2 * (sg.t1 - sg.t0);
-                        c.qb = 0;
-                        c.qph = c.qn & 1;
-                        ++c.qn;
+                        c.n_t = sg.t1 - sg.t0;
+                        c.c = 0;
+                        c.seek = false;
+                        if (v) skip(c, c.n_t);  // past the K tiles
                         return;
                     }
                 }
+                c.done = c.u + 1 >= U;
             };
-            seek(qq);
-            seek(pq);
             uint32_t sfree_par = 0;  // per cache region: parity of the next "region free" phase
-            uint32_t pv_idx = 0, o_phase = 0;
+            uint32_t region = 0;     // of the next K Q^T tile: regions are taken in turn, across units
+            uint32_t pb = 0, pph = 0, pe = 0, o_phase = 0, q_phase = 0;
             bool ok = true;
             auto qk_ready = [&]() -> bool {
-                const int c = qq.t - qq.t0;
-                const uint32_t slot = qq.slot_base + c;
-                const uint32_t s = slot % p.n_slots, sph = (slot / p.n_slots) & 1;
-                if (c == 0 && !mbar_test_wait(F8 ? B.q_ready : B.q_full + 8 * qq.qb, qq.qph)) return false;
-                if (!mbar_test_wait(B.slot_full + 8 * s, sph)) return false;
-                return mbar_test_wait(B.s_free + 8 * c, ((sfree_par >> c) & 1) ^ 1);
+                if (qq.c == 0 && !mbar_test_wait(F8 ? B.q_ready : B.q_full, q_phase)) return false;
+                if (!mbar_test_wait(B.slot_full + 8 * qq.slot, qq.ph)) return false;
+                return mbar_test_wait(B.s_free + 8 * region, ((sfree_par >> region) & 1) ^ 1);
             };
             auto issue_qk = [&]() {
-                const int c = qq.t - qq.t0;
-                const uint32_t slot = qq.slot_base + c;
-                const uint32_t s = slot % p.n_slots;
-                sfree_par ^= 1u << c;
+                sfree_par ^= 1u << region;
                 tc_fence_after();
-                const uint32_t k_addr = s_slots + s * kSlotBytes;
-                const uint32_t q_addr = s_q + qq.qb * q_bytes;
-                const uint32_t d_s = tmem_base + col_s + c * N;
+                const uint32_t k_addr = s_slots + qq.slot * kSlotBytes;
+                const uint32_t d_s = tmem_base + col_s + region * N;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     if (ks * 16 < p.D) {  // head_dim 64: the first four 16-wide steps
                         const uint64_t a = desc_kmajor(k_addr + (ks >> 2) * 16384 + (ks & 3) * 32);
-                        const uint64_t b = desc_kmajor(q_addr + (ks >> 2) * (N * 128) + (ks & 3) * 32);
+                        const uint64_t b = desc_kmajor(s_q + (ks >> 2) * (N * 128) + (ks & 3) * 32);
                         tc_mma(d_s, a, b, idesc_qk, ks ? 1u : 0u);
                     }
                 }
-                tc_commit(B.s_full + 8 * c);
-                tc_commit(B.slot_empty + 8 * s);
-                if (qq.t == qq.t1 - 1) tc_commit(B.q_empty + 8 * qq.qb);  // last use of this Q buffer
-                if (++qq.t == qq.t1) seek(qq);
+                tc_commit(B.s_full + 8 * region);
+                tc_commit(B.slot_empty + 8 * qq.slot);
+                if (++region == (uint32_t)p.n_cache) region = 0;
+                skip(qq, 1);
+                if (++qq.c == qq.n_t) {
+                    tc_commit(B.q_empty);  // last use of this Q
+                    q_phase ^= 1;
+                    qq.seek = true;
+                }
             };
             auto pv_ready = [&]() -> bool {
-                const int c = pq.t - pq.t0;
-                const uint32_t slot = pq.slot_base + (pq.t1 - pq.t0) + c;
-                const uint32_t s = slot % p.n_slots, sph = (slot / p.n_slots) & 1;
-                const uint32_t pb = pv_idx % p.p_bufs, pph = (pv_idx / p.p_bufs) & 1;
                 if (!mbar_test_wait(B.p_full + 8 * pb, pph)) return false;
-                if (!mbar_test_wait(B.slot_full + 8 * s, sph)) return false;
-                if (c == 0 && !mbar_test_wait(B.o_empty, o_phase ^ 1)) return false;
-                return true;
+                if (!mbar_test_wait(B.slot_full + 8 * pq.slot, pq.ph)) return false;
+                return pq.c != 0 || mbar_test_wait(B.o_empty, o_phase ^ 1);
             };
             auto issue_pv = [&]() {
-                const int c = pq.t - pq.t0;
-                const uint32_t slot = pq.slot_base + (pq.t1 - pq.t0) + c;
-                const uint32_t s = slot % p.n_slots;
-                const uint32_t pb = pv_idx % p.p_bufs;
-                const uint32_t pe = pv_idx & 3;
-                ++pv_idx;
-                const bool first = c == 0, last = pq.t == pq.t1 - 1;
                 tc_fence_after();
-                const uint32_t v_addr = s_slots + s * kSlotBytes;
+                const uint32_t v_addr = s_slots + pq.slot * kSlotBytes;
                 const uint32_t p_addr = s_p + pb * p_bytes;
                 const uint32_t d_o = tmem_base + col_o;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     const uint64_t a = desc_mnmajor(v_addr + ks * 2048);
                     const uint64_t b = desc_mnmajor_nosw(p_addr + ks * 256);
-                    tc_mma(d_o, a, b, idesc_pv, (first && ks == 0) ? 0u : 1u);
+                    tc_mma(d_o, a, b, idesc_pv, (pq.c == 0 && ks == 0) ? 0u : 1u);
                 }
-                tc_commit(B.slot_empty + 8 * s);
+                tc_commit(B.slot_empty + 8 * pq.slot);
                 tc_commit(B.p_empty + 8 * pe);
-                if (last) {
+                pe = (pe + 1) & 3;
+                if (++pb == (uint32_t)p.p_bufs) {
+                    pb = 0;
+                    pph ^= 1;
+                }
+                skip(pq, 1);
+                if (++pq.c == pq.n_t) {
                     tc_commit(B.o_full);
                     o_phase ^= 1;
+                    pq.seek = true;
                 }
-                if (++pq.t == pq.t1) seek(pq);
             };
             long long t_idle = clock64();
             uint32_t spins = 0;
             while (ok && !(qq.done && pq.done)) {
                 bool progressed = false;
-                if (qq.pending && !qq.done) seek(qq);
-                if (pq.pending && !pq.done) seek(pq);
-                // a unit's P V tiles can only follow its own QK^T tiles
-                if (!pq.done && !pq.pending && (qq.done || qq.pending || qq.u > pq.u) && pv_ready()) {
+                if (qq.seek && !qq.done) seek(qq, false);
+                if (pq.seek && !pq.done) seek(pq, true);
+                // a unit's P V tiles can only follow its own K Q^T tiles
+                if (!pq.seek && (qq.seek || qq.u > pq.u) && pv_ready()) {
                     issue_pv();
                     progressed = true;
                 }
-                if (!qq.done && !qq.pending && qk_ready()) {
+                if (!qq.seek && qk_ready()) {
                     issue_qk();
                     progressed = true;
                 }
@@ -635,7 +650,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 }
             }
             if (lane == 0) {
-                ok = mbar_wait(B.pub_p1, unit & 1, ctl, 34);
+                ok = bar_wait(B.pub_p1, unit & 1, ctl);
                 if (ok && shared) {
                     __threadfence();
                     atomicAdd(c_p1, 1);
@@ -662,7 +677,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 #pragma unroll
                             for (int u = 0; u < 20; ++u) {
                                 x[u] = make_float2(-1.0e30f, 0.f);
-                                if (u < n_ld) x[u] = __ldcg(q + u * 2 * R);
+                                if (u < n_ld) x[u] = __ldcg(q);
+                                q += 2 * R;
                             }
                             float Mn = M;
 #pragma unroll
@@ -680,7 +696,6 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     M = Mn;
                     if (sub == 0 && r < R) {
                         const float lse2 = M + log2f(Ls);
-                        lse_s[r] = lse2;
                         const float loc = loc_s[r];
                         fac_s[r] = loc < 1.0e29f ? ex2(loc - lse2) : 0.f;  // local -> global normaliser
                         if (sg.rank == 0 && p.a.lse) {
@@ -696,7 +711,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive(B.lse_ready);
             if (lane == 0) {
-                ok = mbar_wait(B.pub_o, unit & 1, ctl, 35);
+                ok = bar_wait(B.pub_o, unit & 1, ctl);
                 if (ok && shared) {
                     __threadfence();
                     atomicAdd(c_o, 1);
@@ -719,31 +734,39 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const int lo = sg.rank * E4 / sg.n, hi = (sg.rank + 1) * E4 / sg.n;
             const float4* src = reinterpret_cast<const float4*>(
                 p.o_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R * kD);
-            // sixteen loads in flight: of up to four partials for four elements, or of sixteen for one
-            const int ne = sg.n <= 4 ? 4 : 1, np = 16 / ne;
+            // Sixteen loads in flight as four groups of four: with up to four partials the groups are four elements, 32
+            // apart, else they are sixteen partials of one element.
+            const bool few = sg.n <= 4;
+            const int ne = few ? 4 : 1;
+            const int64_t out0 = ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D;
+#pragma unroll 1
             for (int e0 = lo + tid; e0 < hi; e0 += 32 * ne) {
                 float4 acc[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int k0 = 0; k0 < sg.n; k0 += np) {
+#pragma unroll 1
+                for (int k0 = 0; k0 < sg.n; k0 += 16) {
                     float4 x[16];
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {  // (partial k, element j): ne == 4: j = u / 4; ne == 1: k = u
-                        const int k = k0 + (ne == 4 ? u & 3 : u), e = e0 + (ne == 4 ? (u >> 2) * 32 : 0);
-                        x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (k < sg.n && e < hi) x[u] = __ldcg(src + k * E4 + e);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                    for (int u = 0; u < 4; ++u) {
+                        const int left = few ? (e0 + 32 * u < hi ? sg.n : 0) : sg.n - k0 - 4 * u;  // partials of this group
+                        const float4* q = src + (few ? e0 + 32 * u : (k0 + 4 * u) * E4 + e0);
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            acc[u].x += x[4 * u + k].x;
-                            acc[u].y += x[4 * u + k].y;
-                            acc[u].z += x[4 * u + k].z;
-                            acc[u].w += x[4 * u + k].w;
+                            x[4 * u + k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (k < left) x[4 * u + k] = __ldcg(q);
+                            q += E4;
                         }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) {
+                        acc[u >> 2].x += x[u].x;
+                        acc[u >> 2].y += x[u].y;
+                        acc[u >> 2].z += x[u].z;
+                        acc[u >> 2].w += x[u].w;
+                    }
                 }
-                if (ne == 1) {  // the sixteen belong to one element
+                if (!few) {
 #pragma unroll
                     for (int u = 1; u < 4; ++u) {
                         acc[0].x += acc[u].x;
@@ -754,18 +777,15 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + 32 * u;
-                    if (u >= ne || e >= hi) break;
-                    const int r = e / (kD / 4), d4 = e - r * (kD / 4);
-                    if (d4 * 4 >= p.D) continue;  // head_dim 64: the partial's upper columns are padding
-                    const int j = fast_div(p, 3, r), g = r - j * G;
-                    const int64_t row =
-                        (((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q + j) * p.a.kv.n_q_heads + sg.h * G + g;
-                    if (p.a.out_bf16)
-                        reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.a.out) + row * p.D)[d4] =
-                            make_uint2(pack_bf16(acc[u].x, acc[u].y), pack_bf16(acc[u].z, acc[u].w));
-                    else
-                        reinterpret_cast<float4*>(p.a.out + row * p.D)[d4] = acc[u];
+                    const int e = e0 + 32 * u, d = 4 * (e & (kD / 4 - 1));
+                    if (u < ne && e < hi && d < p.D) {  // (head_dim 64: the partial's upper columns are padding)
+                        const int64_t at = out0 + roff_s[e / (kD / 4)] + d;
+                        if (p.a.out_bf16)
+                            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.a.out) + at) =
+                                make_uint2(pack_bf16(acc[u].x, acc[u].y), pack_bf16(acc[u].z, acc[u].w));
+                        else
+                            *reinterpret_cast<float4*>(p.a.out + at) = acc[u];
+                    }
                 }
             }
             __syncwarp();
@@ -823,8 +843,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 cv_s = 0;
                 cv_sph ^= 1;
             }
-            if (!mbar_wait(B.raw_full + 8 * r, rph, ctl, 40)) return false;
-            if (!mbar_wait(B.slot_empty + 8 * s, sph ^ 1, ctl, 41)) return false;
+            if (!bar_wait(B.raw_full + 8 * r, rph, ctl)) return false;
+            if (!bar_wait(B.slot_empty + 8 * s, sph ^ 1, ctl)) return false;
             const uint8_t* raw = sgen + (s_raw - sbase) + r * 16384;
             uint8_t* slot = sgen + (s_slots - sbase) + s * kSlotBytes;
             uint4 in[kIter];
@@ -865,7 +885,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             for (; q_next <= unit && q_next < U; ++q_next) {
                 const Work s2 = get_work(sc, q_next);
                 if (!s2.valid()) continue;
-                if (!mbar_wait(B.q_full, qn_s & 1, ctl, 42)) return false;
+                if (!bar_wait(B.q_full, qn_s & 1, ctl)) return false;
                 ++qn_s;
                 uint32_t* qw = reinterpret_cast<uint32_t*>(sgen + (s_q - sbase));
                 for (int i = tid_s; i < q_bytes / 4; i += 128 * CG) {
@@ -881,13 +901,19 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         };
         constexpr float kNegBig = -1.0e30f;      // finite stand-in for -inf: keeps ex2 arguments NaN-free
         uint32_t pv_idx = 0, slot_base = 0, o_phase = 0, sync_n = 0, sfull_par = 0;
+        uint32_t rbase = 0;                      // region of the unit's first tile (see the MMA warp)
+        auto region_of = [&](int c) -> uint32_t {  // of tile c of the unit (c <= n_cache)
+            const uint32_t r = rbase + c;
+            return r >= (uint32_t)p.n_cache ? r - p.n_cache : r;
+        };
+        uint32_t pb = 0;                         // P buffer of the next tile
         bool ok = true;
 
         // O^T (d on lanes, rows on columns, hi and lo parts), rescaled from the CTA-local to the
         // global normaliser -> this CTA's partial [r][d]
         auto epilogue = [&](int unit, const Work& sg) -> bool {
             const int64_t obase = ((int64_t)(unit % kRing) * gridDim.x + blockIdx.x) * R * kD;
-            if (!mbar_wait(B.o_full, o_phase, ctl, 25)) return false;
+            if (!bar_wait(B.o_full, o_phase, ctl)) return false;
             o_phase ^= 1;
             tc_fence_after();
             uint32_t v[NH], w[NH];
@@ -896,26 +922,22 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(B.o_empty);
-            const bool alone = sg.n == 1;  // no other CTA has a part of this problem: this is the output
-            int j = c0 / G, g = c0 - j * G;
-            const int64_t row0 = ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q;
+            // no other CTA has a part of the problem: this is the output; else a partial
+            const bool alone = sg.n == 1, half = alone && p.a.out_bf16;
+            const int64_t out0 =
+                ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D;
+            char* dst = reinterpret_cast<char*>(alone ? p.a.out : p.o_part) +
+                        ((alone ? out0 : obase) + key_l) * (half ? 2 : 4);
+            const int R_key = alone && key_l >= p.D ? 0 : R;  // (head_dim 64: the upper half of the lanes is padding)
 #pragma unroll
             for (int i = 0; i < NH; ++i) {
                 const int r = c0 + i;
-                if (r < R) {
+                if (r < R_key) {
                     const float o = (F8 ? fmaf(__uint_as_float(w[i]), 1.f / kLoExp, __uint_as_float(v[i]))
                                         : __uint_as_float(v[i]) + __uint_as_float(w[i])) * (SC ? fac_s[r] * vsc : fac_s[r]);
-                    if (!alone) {
-                        p.o_part[obase + (int64_t)r * kD + key_l] = o;
-                    } else if (key_l < p.D) {
-                        const int64_t at = ((row0 + j) * p.a.kv.n_q_heads + sg.h * G + g) * p.D + key_l;
-                        if (p.a.out_bf16) reinterpret_cast<__nv_bfloat16*>(p.a.out)[at] = __float2bfloat16_rn(o);
-                        else p.a.out[at] = o;
-                    }
-                }
-                if (++g == G) {
-                    g = 0;
-                    ++j;
+                    const int off = alone ? roff_s[r] : r * kD;
+                    if (half) *reinterpret_cast<__nv_bfloat16*>(dst + 2 * off) = __float2bfloat16_rn(o);
+                    else *reinterpret_cast<float*>(dst + 4 * off) = o;
                 }
             }
             __syncwarp();
@@ -927,7 +949,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const Work sg = get_work(sc, unit);
             if (!sg.valid()) {  // keeps step with the publisher warp
                 if (sw == kSW - 1 && lane == 0) mbar_arrive(B.pub_p1);
-                ok = mbar_wait(B.lse_ready, unit & 1, ctl, 32);
+                ok = bar_wait(B.lse_ready, unit & 1, ctl);
                 if (lane == 0) mbar_arrive(B.pub_o);
                 continue;
             }
@@ -964,27 +986,22 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     ok = ensure_converted(slot_base + c + f8_ahead);
                     if (!ok) break;
                 }
-                ok = mbar_wait(B.s_full + 8 * c, (sfull_par >> c) & 1, ctl, 20);
+                const uint32_t rg = region_of(c);
+                ok = bar_wait(B.s_full + 8 * rg, (sfull_par >> rg) & 1, ctl);
                 if (!ok) break;
-                sfull_par ^= 1u << c;
+                sfull_par ^= 1u << rg;
                 tc_fence_after();
                 uint32_t v[NH];
-                load_cols<NH>(t_lane + col_s + c * N + c0, v);
+                load_cols<NH>(t_lane + col_s + rg * N + c0, v);
                 float sc[NH];
 #pragma unroll
                 for (int i = 0; i < NH; ++i) sc[i] = __uint_as_float(v[i]) * cs;
                 if (t * kTile + kTile > sg.T - p.a.n_q + 1) {
                     // tile holds keys some window rows may not see (or keys beyond the context)
-                    const int key = t * kTile + key_l;
-                    int j = c0 / G, gg = c0 - j * G;
+                    const int hidden = (t * kTile + key_l - (sg.T - p.a.n_q)) * G - c0;  // columns before it do not see the key
 #pragma unroll
-                    for (int i = 0; i < NH; ++i) {
-                        if (key > sg.T - p.a.n_q + j) sc[i] = kNegBig;
-                        if (++gg == G) {
-                            gg = 0;
-                            ++j;
-                        }
-                    }
+                    for (int i = 0; i < NH; ++i)
+                        if (i < hidden) sc[i] = kNegBig;
                 }
                 // running max is refreshed only when some lane's score beats it by 2^8: one
                 // warp-uniform branch per tile, one ex2 per element otherwise
@@ -1003,19 +1020,29 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 for (int i = 0; i < NH; ++i) l[i] += ex2(sc[i] - m[i]);
             }
             if (!ok) break;
-            // reduce (m, l) over the 32 key lanes of this warp, then over the 4 warps via smem:
-            // a butterfly that halves the columns a lane carries at every step (see ml_step)
+            // reduce (m, l) over the 32 key lanes of this warp, then over the 4 warps via smem
             {
+#pragma unroll
+                for (int i = 0; i < NH; ++i) {
+                    const float M = warp_max_all(m[i]);
+                    l[i] *= ex2(m[i] - M);
+                    m[i] = M;
+                }
+                if (lane == 0) {
+#pragma unroll
+                    for (int i = 0; i < NH; i += 4)
+                        *reinterpret_cast<float4*>(red_m + sw * NC + i) = make_float4(m[i], m[i + 1], m[i + 2], m[i + 3]);
+                }
                 int col = 0;
-                ml_step<NH, NH, 16>(m, l, lane, col);
-                constexpr uint32_t kDup = ml_dupmask(NH);
-                constexpr int kLeft = ml_final_n(NH);
+                sum_step<NH, NH, 16>(l, lane, col);
+                constexpr uint32_t kDup = sum_dupmask(NH);
+                constexpr int kLeft = sum_final_n(NH);
                 if ((lane & kDup) == 0) {
 #pragma unroll
-                    for (int j = 0; j < kLeft; ++j) red[sw * NC + col + j] = make_float2(m[j], l[j]);
+                    for (int j = 0; j < kLeft; ++j) red_l[sw * NC + col + j] = l[j];
                 }
             }
-            ok = group_sync(B.sm_sync, sync_n, ctl, 26);
+            ok = warps_sync(B.sm_sync, sync_n, ctl);
             if (!ok) break;
             if (sw == kSW - 1) {
                 // the last softmax warp merges the four lane quarters of every column, publishes the
@@ -1025,13 +1052,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     const int wgi = col / NC, ci = col - wgi * NC;
                     float M = kNegBig;
 #pragma unroll
-                    for (int w = 0; w < 4; ++w) M = fmaxf(M, red[(wgi * 4 + w) * NC + ci].x);
+                    for (int w = 0; w < 4; ++w) M = fmaxf(M, red_m[(wgi * 4 + w) * NC + ci]);
                     float Ls = 0.f;
 #pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        const float2 ml = red[(wgi * 4 + w) * NC + ci];
-                        Ls += ml.y * ex2(ml.x - M);
-                    }
+                    for (int w = 0; w < 4; ++w) Ls += red_l[(wgi * 4 + w) * NC + ci] * ex2(red_m[(wgi * 4 + w) * NC + ci] - M);
                     const bool has = M > 0.5f * kNegBig;              // the row saw at least one key here
                     const float loc = has ? M + log2f(Ls) : 1.0e30f;  // no key: P = exp2(s - big) = 0
                     loc_s[col] = loc;
@@ -1049,7 +1073,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 __syncwarp();
                 if (lane == 0) mbar_arrive(B.pub_p1);  // the publisher warp takes it from here
             }
-            ok = group_sync(B.sm_sync, sync_n, ctl, 27);
+            ok = warps_sync(B.sm_sync, sync_n, ctl);
             if (!ok) break;
             {
                 // ------------------------------ P2a: P V with the CTA-local normaliser ------------------
@@ -1062,16 +1086,11 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 {
                     const float4* loc4 = reinterpret_cast<const float4*>(loc_s + c0);
                     uint32_t v[NH];
-                    if (n_t > 0) {
 #pragma unroll
-                        for (int q = 0; q < NH; q += 8) tmem_ld8(t_lane + col_s + c0 + q, v + q);
-                    }
+                    for (int q = 0; q < NH; q += 8) tmem_ld8(t_lane + col_s + rbase * N + c0 + q, v + q);
                     for (int c = 0; c < n_t && ok; ++c) {
                         const int t = sg.t0 + c;
-                        const uint32_t vslot = slot_base + n_t + c;
-                        const uint32_t vs = vslot % p.n_slots, vsph = (vslot / p.n_slots) & 1;
                         const uint32_t pvi = pv_idx + c;
-                        const uint32_t pb = pvi % p.p_bufs;
                         const int key = t * kTile + key_l;
                         if (F8) {  // V tile c + 2 (or the next unit's first K tiles) becomes an operand meanwhile
                             ok = ensure_converted(slot_base + n_t + c + f8_ahead);
@@ -1090,29 +1109,24 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                         }
                         if (c + 1 < n_t) {  // next tile's columns: in flight during the rest of this tile
 #pragma unroll
-                            for (int q = 0; q < NH; q += 8) tmem_ld8(t_lane + col_s + (c + 1) * N + c0 + q, v + q);
+                            for (int q = 0; q < NH; q += 8) tmem_ld8(t_lane + col_s + region_of(c + 1) * N + c0 + q, v + q);
                         }
                         if (t * kTile + kTile > sg.T - p.a.n_q + 1) {
-                            int j = c0 / G, gg = c0 - j * G;
+                            const int hidden = (key - (sg.T - p.a.n_q)) * G - c0;
 #pragma unroll
-                            for (int i = 0; i < NH; ++i) {
-                                if (key > sg.T - p.a.n_q + j) pr[i] = 0.f;  // select, so NaN-safe
-                                if (++gg == G) {
-                                    gg = 0;
-                                    ++j;
-                                }
-                            }
+                            for (int i = 0; i < NH; ++i)
+                                if (i < hidden) pr[i] = 0.f;  // select, so NaN-safe
                         }
                         // P~ replaces the tile's scores in tensor memory: the statistic pass then only
                         // weights it with exp2(lse_local - LSE) per row, no second exponential
 #pragma unroll
                         for (int q = 0; q < NH; q += 8)
-                            tmem_st8(t_lane + col_s + c * N + c0 + q, reinterpret_cast<const uint32_t*>(pr) + q);
+                            tmem_st8(t_lane + col_s + region_of(c) * N + c0 + q, reinterpret_cast<const uint32_t*>(pr) + q);
                         // the P buffer is free once the P V product p_bufs tiles back is done ("done"
                         // barriers are indexed by the tile's sequence number mod 4)
                         if (pvi >= (uint32_t)p.p_bufs) {
                             const uint32_t prev = pvi - p.p_bufs;
-                            ok = mbar_wait(B.p_empty + 8 * (prev & 3), (prev >> 2) & 1, ctl, 23);
+                            ok = bar_wait(B.p_empty + 8 * (prev & 3), (prev >> 2) & 1, ctl);
                             if (!ok) break;
                         }
                         // [P_hi | P_lo]^T as the B operand, rows contiguous (MN-major, no swizzle): the
@@ -1150,7 +1164,9 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                         if (t * kTile + kTile > sg.T) {
                             // ragged last tile: V rows at or beyond T may hold anything; zero them in
                             // shared memory so that 0 * garbage never reaches the accumulator
-                            ok = mbar_wait(B.slot_full + 8 * vs, vsph, ctl, 24);
+                            const uint32_t vslot = slot_base + n_t + c;
+                            const uint32_t vs = vslot % p.n_slots, vsph = (vslot / p.n_slots) & 1;
+                            ok = bar_wait(B.slot_full + 8 * vs, vsph, ctl);
                             if (!ok) break;
                             if (key >= sg.T && wg < 2) {  // warpgroups 0 and 1 clear one 64-wide half each
                                 uint8_t* vrow = sgen + (s_slots - sbase) + vs * kSlotBytes + wg * 16384 + key_l * 128;
@@ -1161,6 +1177,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                         fence_proxy_async();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(B.p_full + 8 * pb);
+                        if (++pb == (uint32_t)p.p_bufs) pb = 0;
                     }
                 }
                 if (!ok) break;
@@ -1169,7 +1186,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 pv_idx += n_t;
                 slot_base += 2 * n_t;
                 // ---- the row LSE and the rescale factors, combined by the publisher warp meanwhile ----
-                ok = mbar_wait(B.lse_ready, unit & 1, ctl, 31);
+                ok = bar_wait(B.lse_ready, unit & 1, ctl);
                 if (!ok) break;
                 if (!LP && sg.n > 1) {  // many CTAs per head: too many partials for one warp, all softmax threads fold them
                     if (lane == 0) ok = counter_wait(p.counters + unit * p.n_sid + sg.sid, sg.n, ctl, 33);
@@ -1205,7 +1222,6 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     }
                     if (sub == 0 && r < R) {
                         const float lse2 = M + log2f(Ls);
-                        lse_s[r] = lse2;
                         const float loc = loc_s[r];
                         fac_s[r] = loc < 1.0e29f ? ex2(loc - lse2) : 0.f;  // local -> global normaliser
                         if (sg.rank == 0 && p.a.lse) {
@@ -1219,7 +1235,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     ok = ensure_q(unit + 1);
                     if (!ok) break;
                 }
-                ok = group_sync(B.sm_sync, sync_n, ctl, 22);  // every warp is done with the P V pass
+                ok = warps_sync(B.sm_sync, sync_n, ctl);  // every warp is done with the P V pass
                 if (!ok) break;
                 tc_fence_after();  // the P~ stores of the other warps, ordered by the barrier
                 // ------------------------------ P2b: the Eq. 3 statistic ------------------------------
@@ -1230,6 +1246,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 for (int c = wg; c < n_t; c += CG) {
                     const int t = sg.t0 + c;
                     const int key = t * kTile + key_l;
+                    const uint32_t rg = region_of(c);
                     float st = 0.f;
                     float sth[PH ? 8 : 1];  // PH: column i belongs to head i mod G, and G divides 8
 #pragma unroll
@@ -1238,8 +1255,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     for (int cb = 0; cb < N; cb += 16) {
                         if (cb + 16 <= stat_r0) continue;  // rows outside the statistic window
                         uint32_t v[16];
-                        tmem_ld8(t_lane + col_s + c * N + cb, v);
-                        tmem_ld8(t_lane + col_s + c * N + cb + 8, v + 8);
+                        tmem_ld8(t_lane + col_s + rg * N + cb, v);
+                        tmem_ld8(t_lane + col_s + rg * N + cb + 8, v + 8);
                         tc_wait_ld();
                         const float4* fac4 = reinterpret_cast<const float4*>(fac_s + cb);
                         float pr[16];
@@ -1274,7 +1291,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(B.s_free + 8 * c);
+                    if (lane == 0) mbar_arrive(B.s_free + 8 * rg);
                     if (PH) {
                         // fast path: fold the eight residues mod 8 down to the G residues mod G
                         if (ph_fast && G <= 4) {
@@ -1324,7 +1341,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 if (!PH && p.a.hist) {
                     // the CTA's counts of this head join the global ones: one reduction per bin that is not
                     // empty (a few dozen), and the shared-memory copy is clear again for the next unit
-                    ok = group_sync(B.sm_sync, sync_n, ctl, 28);
+                    ok = warps_sync(B.sm_sync, sync_n, ctl);
                     if (!ok) break;
                     uint32_t* hg = p.a.hist + (int64_t)sg.prob * kScoreBins;
                     for (int w = tid_s; w < kScoreBins / 2; w += 128 * CG) {
@@ -1337,6 +1354,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     }
                 }
             }
+            rbase = region_of(n_t);
             // ---- this unit's accumulator: rescale and hand to the reducers ----
             ok = epilogue(unit, sg);
             if (!ok) break;
