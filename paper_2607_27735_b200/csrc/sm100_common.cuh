@@ -33,6 +33,8 @@ struct FastParams {
     int n_cls;                        // classes in use
     int cls_size[kMaxClass];          // CTAs of a part
     int cls_subs[kMaxClass];          // parts of a team
+    uint32_t cls_mul[kMaxClass];      // division by cls_size (see div_by)
+    int32_t cls_sh[kMaxClass];
     int n_sid;                        // parts of all teams in the finest class
     int n_counters;                   // ints to zero at the end, the "CTAs finished" word being the one after them
     int* counters;                    // two-sweep: [2][n_units * HG]: P1 partials done, O partials done; score cache:
@@ -53,21 +55,26 @@ struct FastParams {
 };
 
 // Host side: magic numbers of an exact division by d >= 1 (see FastParams::div_mul).
-inline void set_divisor(FastParams* p, int which, int d)
+inline void set_divisor(uint32_t* mul, int32_t* sh, int d)
 {
     if (d <= 1) {
-        p->div_mul[which] = 0;
-        p->div_sh[which] = -1;
+        *mul = 0;
+        *sh = -1;
         return;
     }
     int c = 0;
     while ((1ull << c) < (unsigned)d) ++c;
-    p->div_mul[which] = (uint32_t)(((1ull << (31 + c)) + d - 1) / d);
-    p->div_sh[which] = c - 1;
+    *mul = (uint32_t)(((1ull << (31 + c)) + d - 1) / d);
+    *sh = c - 1;
+}
+inline void set_divisor(FastParams* p, int which, int d) { set_divisor(&p->div_mul[which], &p->div_sh[which], d); }
+__device__ __forceinline__ int div_by(uint32_t mul, int32_t sh, int x)
+{
+    return sh < 0 ? x : (int)(__umulhi((uint32_t)x, mul) >> sh);
 }
 __device__ __forceinline__ int fast_div(const FastParams& p, int which, int x)
 {
-    return p.div_sh[which] < 0 ? x : (int)(__umulhi((uint32_t)x, p.div_mul[which]) >> p.div_sh[which]);
+    return div_by(p.div_mul[which], p.div_sh[which], x);
 }
 
 // ---------------------------------------------------------------------------------------------

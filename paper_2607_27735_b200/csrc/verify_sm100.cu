@@ -432,6 +432,7 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
     for (int f = 0; f < pl.n_cls; ++f) {
         fp.cls_size[f] = pl.cls_size[f];
         fp.cls_subs[f] = pl.cls_subs[f];
+        set_divisor(&fp.cls_mul[f], &fp.cls_sh[f], pl.cls_size[f]);
     }
     fp.n_sid = pl.n_sid;
     fp.n_counters = pl.n_counters;

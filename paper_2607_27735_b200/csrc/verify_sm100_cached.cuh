@@ -112,7 +112,7 @@ __device__ __forceinline__ void e4m3x4_to_f16x4(uint32_t w, uint32_t& lo, uint32
 // 700-token one on a team sized for 6 K, would spend most of its time on the former.  The sequences are taken
 // longest first (the lengths are in device memory, so every CTA sorts them for itself), the order of the parts
 // alternates from unit to unit, and a class that would not fill half of a round joins the coarser one.
-constexpr int kSortMax = 192;  // sequences; larger batches keep their order and whole teams
+constexpr int kSortMax = 64;  // sequences, two per lane of the warp that sorts them; larger batches keep their order and whole teams
 // What a CTA does in one unit.  The first units are worked out in the prologue, by a thread each, and every role reads
 // them from shared memory: the arithmetic in each role's loop would be fetched from the instruction cache again every
 // unit.  Later units (launches over many layers) take the places of old ones: the publisher warp writes kWorkAhead
@@ -136,7 +136,7 @@ struct Sched {
     volatile int limit;
     int unit0[kMaxClass + 1];   // first unit of a class
     int seq0[kMaxClass + 1];    // first sequence (in sorted order) of a class
-    int cnt[kMaxClass];
+    int len[kSortMax];          // as they come
     uint16_t ord[kSortMax];
 };
 static_assert(sizeof(Sched) <= 1536, "fits between the histogram and the row partials");
@@ -148,7 +148,7 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     while (f + 1 < p.n_cls && unit >= sc.unit0[f + 1]) ++f;
     const int size = p.cls_size[f], subs = p.cls_subs[f], slots = p.HG * subs;
     const int team = fast_div(p, 2, blockIdx.x), local = blockIdx.x - team * p.cph;
-    const int sub = local / size, rank = local - sub * size;
+    const int sub = div_by(p.cls_mul[f], p.cls_sh[f], local), rank = local - sub * size;
     const int slot = team * subs + sub;
     const int i = (unit - sc.unit0[f]) * slots + ((unit & 1) ? slots - 1 - slot : slot);
     bool valid = sub < subs && i >= 0;
@@ -166,8 +166,9 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     const int nb = (w.T + kTile - 1) / kTile;
     const int n = min(size, nb);  // every CTA of a problem has a tile
     valid = valid && rank < n;
-    w.t0 = valid ? rank * nb / n : 0;
-    w.t1 = valid ? (rank + 1) * nb / n : 0;
+    // shares of nb / n tiles; n < size means a tile each
+    w.t0 = !valid ? 0 : (n < size ? rank : div_by(p.cls_mul[f], p.cls_sh[f], rank * nb));
+    w.t1 = !valid ? 0 : (n < size ? rank + 1 : div_by(p.cls_mul[f], p.cls_sh[f], (rank + 1) * nb));
     w.layer = (uint16_t)layer;
     w.b = (uint16_t)b;
     w.h = (uint16_t)h;
@@ -336,58 +337,70 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
-    {  // the schedule (see Sched): lengths, their order, classes
-        const int B = p.a.kv.batch;
-        int* raw = reinterpret_cast<int*>(red_m);
-        int T = 0;
+    if (warp == 0) {  // the schedule (see Sched): lengths, their order, classes, this CTA's first units
+        const int B = p.a.kv.batch, LH = p.a.kv.n_layers * p.a.kv.n_kv_heads;
         const bool sorted = B <= kSortMax;
-        if (threadIdx.x < kMaxClass) sc.cnt[threadIdx.x] = 0;
-        if (sorted && threadIdx.x < B) {
-            T = min(max(p.a.ctx_len[threadIdx.x], p.a.n_q), p.a.max_ctx_len);
-            raw[threadIdx.x] = T;
+        int cnt[kMaxClass];
+#pragma unroll
+        for (int f = 0; f < kMaxClass; ++f) cnt[f] = 0;
+        if (!sorted) cnt[0] = B;
+#pragma unroll 1
+        for (int i = 0; i < 2 && sorted; ++i) {
+            const int b = lane + 32 * i;
+            sc.len[b] = b < B ? min(max(p.a.ctx_len[b], p.a.n_q), p.a.max_ctx_len) : 0;
+            if (B <= 32) break;
         }
-        __syncthreads();
-        if (sorted && threadIdx.x < B) {
+        __syncwarp();
+#pragma unroll 1
+        for (int i = 0; i < 2 && sorted && 32 * i < B; ++i) {
+            const int b = lane + 32 * i, T = sc.len[b];
             int before = 0;
 #pragma unroll 1
-            for (int j = 0; j < B; ++j) before += (raw[j] > T || (raw[j] == T && j < (int)threadIdx.x)) ? 1 : 0;
-            sc.ord[before] = (uint16_t)threadIdx.x;
-            const int nb = (T + kTile - 1) / kTile;
-            int f = p.n_cls - 1;
-            while (f > 0 && p.cls_size[f] * p.n_cache < nb) --f;
-            atomicAdd(&sc.cnt[f], 1);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int LH = p.a.kv.n_layers * p.a.kv.n_kv_heads;
-            sc.sorted = sorted ? 1 : 0;
-            if (!sorted) sc.cnt[0] = B;
-#pragma unroll 1
-            for (int f = p.n_cls - 1; f > 0; --f) {
-                if (2 * sc.cnt[f] * LH <= p.HG * p.cls_subs[f]) {
-                    sc.cnt[f - 1] += sc.cnt[f];
-                    sc.cnt[f] = 0;
-                }
+            for (int j = 0; j < B; ++j) before += (sc.len[j] > T || (sc.len[j] == T && j < b)) ? 1 : 0;
+            int f = -1;
+            if (b < B) {
+                sc.ord[before] = (uint16_t)b;
+                const int nb = (T + kTile - 1) / kTile;
+                f = p.n_cls - 1;
+                while (f > 0 && p.cls_size[f] * p.n_cache < nb) --f;
             }
-            int u = 0, q = 0;
-#pragma unroll 1
-            for (int f = 0; f < kMaxClass; ++f) {
+#pragma unroll
+            for (int c = 0; c < kMaxClass; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, f == c));
+        }
+#pragma unroll
+        for (int f = kMaxClass - 1; f > 0; --f) {
+            if (f < p.n_cls && 2 * cnt[f] * LH <= p.HG * p.cls_subs[f]) {
+                cnt[f - 1] += cnt[f];
+                cnt[f] = 0;
+            }
+        }
+        // rounds of a class, a class per lane
+        int mine = 0;
+#pragma unroll
+        for (int f = 0; f < kMaxClass; ++f) mine = lane == f ? cnt[f] : mine;
+        const int slots = lane < p.n_cls ? p.HG * p.cls_subs[lane] : 1;
+        const int rounds = (mine * LH + slots - 1) / slots;
+        int u = 0, q = 0;
+#pragma unroll
+        for (int f = 0; f <= kMaxClass; ++f) {
+            if (lane == 0) {
                 sc.unit0[f] = u;
                 sc.seq0[f] = q;
-                if (f < p.n_cls) {
-                    const int slots = p.HG * p.cls_subs[f];
-                    u += (sc.cnt[f] * LH + slots - 1) / slots;
-                    q += sc.cnt[f];
-                }
             }
-            sc.unit0[kMaxClass] = sc.n_units = u;
-            sc.seq0[kMaxClass] = q;
+            u += __shfl_sync(0xffffffffu, rounds, f);
+            if (f < kMaxClass) q += cnt[f];
         }
-        __syncthreads();
-        if (threadIdx.x < kWorkTab && threadIdx.x < sc.n_units) put_work(p, sc, threadIdx.x);
-        if (threadIdx.x == 0) sc.limit = min(sc.n_units, kWorkTab);
-        __syncthreads();
+        u -= __shfl_sync(0xffffffffu, rounds, kMaxClass);
+        if (lane == 0) {
+            sc.n_units = u;
+            sc.sorted = sorted ? 1 : 0;
+            sc.limit = min(u, kWorkTab);
+        }
+        __syncwarp();
+        static_assert(kWorkTab == 32, "a unit per lane");
+        if (lane < u) put_work(p, sc, lane);
     }
+    __syncthreads();
     const int U = sc.n_units;
     const uint32_t col_o = 0, col_s = 2 * N;  // O^T (hi | lo) first, then the cached S^T tiles
 
@@ -789,7 +802,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 }
             }
             __syncwarp();
-            if (lane == 0) {  // the partials have been read: their places may be used again
+            if (lane == 0 && unit + kRing - 1 < U) {  // the partials have been read: their places may be used again
                 __threadfence();
                 atomicAdd(c_o + p.n_units * p.n_sid, 1);
             }
