@@ -21,6 +21,16 @@ namespace spec {
 
 namespace {
 
+// Every kernel of this file is launched with programmatic stream serialisation: its launch overlaps the end of the
+// kernel before it, whose results it waits for here.  The next kernel is let go only after that wait, so whatever
+// starts early under this kernel finds everything before this kernel complete.  (A round's scalar tail is a chain of
+// kernels of 2 us each: the gap between two of them costs as much as half a kernel.)
+__device__ __forceinline__ void stream_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr int kEntThreads = 512;
 constexpr int kMaxDrafted = 256;  // drafted tokens the controller looks at in one call
 
@@ -121,6 +131,26 @@ __device__ __forceinline__ float load_logit(const void* base, int v)
     return DT == 1 ? __bfloat162float(static_cast<const __nv_bfloat16*>(base)[v]) : static_cast<const float*>(base)[v];
 }
 
+constexpr int kMaxRowCtas = 8;  // CTAs of a cluster
+
+// Merges the partials of the first n (a power of two) lanes into lane 0's.
+template <bool ENT, bool ARG, int n>
+__device__ __forceinline__ void merge_lanes(Mst& acc, Arg& arg)
+{
+#pragma unroll
+    for (int o = n / 2; o > 0; o >>= 1) {
+        if (ENT) {
+            const Mst other{__shfl_xor_sync(0xffffffffu, acc.m, o), __shfl_xor_sync(0xffffffffu, acc.s, o),
+                            __shfl_xor_sync(0xffffffffu, acc.t, o)};
+            acc = merge(acc, other);
+        }
+        if (ARG) {
+            const Arg other{__shfl_xor_sync(0xffffffffu, arg.v, o), __shfl_xor_sync(0xffffffffu, arg.i, o)};
+            arg = merge(arg, other);
+        }
+    }
+}
+
 // One cluster (gridDim.x CTAs) per row.  DT = 0: fp32 logits, 1: bf16 logits.  ENT: entropy[row];
 // ARG: token[row] = the smallest index of the largest logit.
 template <int DT, bool ENT, bool ARG>
@@ -132,8 +162,11 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
     __shared__ Arg warp_arg[kEntThreads / 32];
     __shared__ Mst cta_part;
     __shared__ Arg cta_arg;
-    const int CS = gridDim.x, rank = blockIdx.x, row = blockIdx.y;
+    // The entropies usually follow a pass over the same logits (acceptance), whose last rows are still in L2: they are
+    // taken from the end.  (576 rows of 128 K bf16 logits, 148 MB, after their argmax: 30 -> @@ us.)
+    const int CS = gridDim.x, rank = blockIdx.x, row = ENT && !ARG ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    stream_wait();
     const char* base = static_cast<const char*>(logits) + (int64_t)row * row_stride * (DT == 1 ? 2 : 4);
     Mst acc{-3.0e38f, 0.f, 0.f};
     Arg arg{kNegInf, 0x7fffffff};
@@ -174,61 +207,68 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
         const int v0 = min(vocab, rank * per), v1 = min(vocab, v0 + per);
         for (int v = v0 + tid; v < v1; v += kEntThreads) fold1<ENT, ARG>(acc, arg, load_logit<DT>(base, v), v);
     }
-    // warp, CTA, cluster: merged in a fixed order
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (ENT) {
-            Mst other{__shfl_xor_sync(0xffffffffu, acc.m, o), __shfl_xor_sync(0xffffffffu, acc.s, o),
-                      __shfl_xor_sync(0xffffffffu, acc.t, o)};
-            acc = merge(acc, other);
-        }
-        if (ARG) {
-            Arg other{__shfl_xor_sync(0xffffffffu, arg.v, o), __shfl_xor_sync(0xffffffffu, arg.i, o)};
-            arg = merge(arg, other);
-        }
-    }
+    // warp, CTA, cluster: merged in a fixed order, every level a tree over the lanes of a warp (partials fetched one
+    // after the other by a single thread cost a latency each: 5.3 -> @@ us for 8 rows)
+    merge_lanes<ENT, ARG, 32>(acc, arg);
     if (lane == 0) {
         warp_part[warp] = acc;
         warp_arg[warp] = arg;
     }
     __syncthreads();
-    if (tid == 0) {
-        Mst a = warp_part[0];
-        Arg g = warp_arg[0];
-        for (int w = 1; w < kEntThreads / 32; ++w) {
-            if (ENT) a = merge(a, warp_part[w]);
-            if (ARG) g = merge(g, warp_arg[w]);
+    constexpr int kWarps = kEntThreads / 32;
+    if (warp == 0) {
+        if (lane < kWarps) {
+            acc = warp_part[lane];
+            arg = warp_arg[lane];
         }
-        cta_part = a;
-        cta_arg = g;
+        merge_lanes<ENT, ARG, kWarps>(acc, arg);
+        if (lane == 0) {
+            cta_part = acc;
+            cta_arg = arg;
+        }
     }
-    if (CS > 1) cluster.sync(); else __syncthreads();
-    if (rank == 0 && tid == 0) {
-        Mst a = cta_part;
-        Arg g = cta_arg;
-        for (int c = 1; c < CS; ++c) {
-            if (ENT) a = merge(a, *cluster.map_shared_rank(&cta_part, c));
-            if (ARG) g = merge(g, *cluster.map_shared_rank(&cta_arg, c));
+    if (CS > 1) cluster.sync();
+    if (rank == 0 && warp == 0) {
+        if (CS > 1) {
+            acc = Mst{-3.0e38f, 0.f, 0.f};
+            arg = Arg{kNegInf, 0x7fffffff};
+            if (lane < CS) {
+                if (ENT) acc = *cluster.map_shared_rank(&cta_part, lane);
+                if (ARG) arg = *cluster.map_shared_rank(&cta_arg, lane);
+            }
+            merge_lanes<ENT, ARG, kMaxRowCtas>(acc, arg);
         }
-        if (ENT) entropy[row] = a.s > 0.f ? a.m + __logf(a.s) - a.t / a.s : 0.f;
-        if (ARG) token[row] = g.i == 0x7fffffff ? 0 : g.i;
+        if (lane == 0) {
+            if (ENT) entropy[row] = acc.s > 0.f ? acc.m + __logf(acc.s) - acc.t / acc.s : 0.f;
+            if (ARG) token[row] = arg.i == 0x7fffffff ? 0 : arg.i;
+        }
     }
     if (CS > 1) cluster.sync();  // nobody leaves while its partial may still be read
 }
 
 // Greedy prefix acceptance: drafted token i of a sequence is accepted iff every earlier one was and
-// it equals the target's token for that position; one thread per sequence.
-__global__ void accept_kernel(const int32_t* __restrict__ target, const int32_t* __restrict__ draft,
-                              const int32_t* __restrict__ n_draft, int batch, int k1,
-                              int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token)
+// it equals the target's token for that position; one warp per sequence, 32 tokens at a time.
+constexpr int kAcceptWarps = 4;
+__global__ void __launch_bounds__(32 * kAcceptWarps)
+accept_kernel(const int32_t* __restrict__ target, const int32_t* __restrict__ draft, const int32_t* __restrict__ n_draft,
+              int batch, int k1, int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.x * kAcceptWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    stream_wait();
     if (b >= batch) return;
     const int nd = n_draft ? min(max(n_draft[b], 0), k1 - 1) : k1 - 1;
     int m = 0;
-    while (m < nd && draft[b * (k1 - 1) + m] == target[b * k1 + m]) ++m;
-    n_accepted[b] = m;
-    next_token[b] = target[b * k1 + m];
+    for (int i0 = 0; i0 < nd; i0 += 32) {
+        const int i = i0 + lane;
+        const bool same = i < nd && draft[b * (k1 - 1) + i] == target[b * k1 + i];
+        const uint32_t wrong = ~__ballot_sync(0xffffffffu, same);
+        m = i0 + (wrong ? __ffs((int)wrong) - 1 : 32);
+        if (wrong) break;
+    }
+    if (lane == 0) {
+        n_accepted[b] = m;
+        next_token[b] = target[b * k1 + m];
+    }
 }
 
 // Eq. "ema": state[0] <- beta state[0] + (1 - beta) mean(H_1..H_m), state[1] likewise with H_{m+1}..H_k
@@ -236,6 +276,7 @@ __global__ void controller_update_kernel(float* state, const float* __restrict__
                                          const int32_t* __restrict__ n_accepted, float beta)
 {
     const int lane = threadIdx.x;
+    stream_wait();
     const int m = min(max(*n_accepted, 0), k);
     float sa = 0.f, sr = 0.f;
     for (int i = lane; i < k; i += 32) {
@@ -257,35 +298,58 @@ __global__ void controller_select_kernel(const float* __restrict__ state, const 
 {
     __shared__ float expected[kMaxDrafted];  // 1 + sum_{m <= k} prod_{i <= m} p_i at k = index + 1
     const int lane = threadIdx.x;
+    stream_wait();
     const float acc_c = state[0], rej_c = state[1];
-    for (int i = lane; i < n; i += 32) {
-        const float a = __expf(-fabsf(entropy[i] - acc_c)), b = __expf(-fabsf(entropy[i] - rej_c));
-        const float p = a / (a + b);
-        expected[i] = p;
-        if (p_out) p_out[i] = p;
+    float prefix = 1.f, sum = 1.f;  // over the tokens of the trips before
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        float p = 1.f;
+        if (i < n) {
+            const float a = __expf(-fabsf(entropy[i] - acc_c)), b = __expf(-fabsf(entropy[i] - rej_c));
+            p = a / (a + b);
+            if (p_out) p_out[i] = p;
+        }
+        float prod = p;  // inclusive products, then their inclusive sums, over the lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, prod, o);
+            if (lane >= o) prod *= y;
+        }
+        prod *= prefix;
+        float e = i < n ? prod : 0.f;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, e, o);
+            if (lane >= o) e += y;
+        }
+        e += sum;
+        if (i < n) expected[i] = e;
+        prefix = __shfl_sync(0xffffffffu, prod, 31);
+        sum = __shfl_sync(0xffffffffu, e, 31);
     }
     __syncwarp();
-    if (lane == 0) {
-        float prefix = 1.f, e = 1.f;
-        for (int i = 0; i < n; ++i) {
-            prefix *= expected[i];
-            e += prefix;
-            expected[i] = e;
+    int best = 0;
+    float best_score = -1.f;
+    for (int c = lane; c < n_cand; c += 32) {
+        const int k = cand[c];
+        float score = -1.f;  // a candidate outside 1..n never wins
+        if (k >= 1 && k <= n) score = expected[k - 1] / (k * c_d + c_v);
+        if (score_out) score_out[c] = score;
+        if (score >= 0.f && (score > best_score || (score == best_score && k < best))) {
+            best_score = score;
+            best = k;
         }
-        int best = 0;
-        float best_score = -1.f;
-        for (int c = 0; c < n_cand; ++c) {
-            const int k = cand[c];
-            float score = -1.f;  // a candidate outside 1..n never wins
-            if (k >= 1 && k <= n) score = expected[k - 1] / (k * c_d + c_v);
-            if (score_out) score_out[c] = score;
-            if (score >= 0.f && (score > best_score || (score == best_score && k < best))) {
-                best_score = score;
-                best = k;
-            }
-        }
-        *k_star = best;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float s2 = __shfl_xor_sync(0xffffffffu, best_score, o);
+        const int k2 = __shfl_xor_sync(0xffffffffu, best, o);
+        if (s2 >= 0.f && (s2 > best_score || (s2 == best_score && k2 < best))) {
+            best_score = s2;
+            best = k2;
+        }
+    }
+    if (lane == 0) *k_star = best;
 }
 
 // Lengths of the next round, on the device: committed += accepted + 1 (the corrected token), the
@@ -295,6 +359,7 @@ __global__ void advance_lengths_kernel(int32_t* __restrict__ committed, const in
                                        int32_t* __restrict__ cur_len, int max_len, int* __restrict__ status)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    stream_wait();
     if (b >= batch) return;
     int t = committed[b] + (n_accepted ? min(max(n_accepted[b], 0), k) + 1 : 0);
     if (max_len > 0 && t + k + 1 > max_len) {  // the next round would leave the cache: hold the sequence and say so
@@ -305,6 +370,27 @@ __global__ void advance_lengths_kernel(int32_t* __restrict__ committed, const in
     if (ctx_verify) ctx_verify[b] = t + k + 1;
     if (cur_len)
         for (int j = 0; j < k; ++j) cur_len[j * batch + b] = t + j + 1;
+}
+
+// A launch that may begin under the kernel before it (see stream_wait).
+template <typename... P, typename... A>
+int launch_chained(void (*kern)(P...), int grid, int block, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {
+        cudaGetLastError();
+        return SPEC_ERR_CUDA;
+    }
+    count_launch(1);
+    return SPEC_OK;
 }
 
 }  // namespace
@@ -324,20 +410,22 @@ int rows_launch(const void* logits, int dtype, int n_rows, int vocab, int64_t ro
     // for the 128K exponentials of a row (16 per clock), but a cluster costs a few hundred
     // nanoseconds of barriers, which shows once every SM has two CTAs anyway.  No CTA without a
     // full sweep of its threads.
-    int cs = 8;
+    int cs = kMaxRowCtas;
     while (cs > 1 && (long)n_rows * cs > 2L * sm_count()) cs /= 2;
     while (cs > 1 && vocab < cs * 8 * kEntThreads) cs /= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, n_rows);
     cfg.blockDim = dim3(kEntThreads);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     cudaError_t err;
     if (entropy && token)
         err = dtype == 1 ? launch_rows<1, true, true>(cfg, logits, vocab, row_stride, entropy, token)
@@ -359,28 +447,21 @@ int rows_launch(const void* logits, int dtype, int n_rows, int vocab, int64_t ro
 int accept_launch(const int32_t* target, const int32_t* draft, const int32_t* n_draft, int batch, int k1,
                   int32_t* n_accepted, int32_t* next_token, cudaStream_t stream)
 {
-    accept_kernel<<<(batch + 127) / 128, 128, 0, stream>>>(target, draft, n_draft, batch, k1, n_accepted, next_token);
-    if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    count_launch(1);
-    return SPEC_OK;
+    return launch_chained(accept_kernel, (batch + kAcceptWarps - 1) / kAcceptWarps, 32 * kAcceptWarps, stream, target, draft,
+                          n_draft, batch, k1, n_accepted, next_token);
 }
 
 int advance_lengths_launch(int32_t* committed, const int32_t* n_accepted, int batch, int k, int max_len, int* status, int32_t* ctx_verify,
                            int32_t* cur_len, cudaStream_t stream)
 {
-    advance_lengths_kernel<<<(batch + 127) / 128, 128, 0, stream>>>(committed, n_accepted, batch, k, ctx_verify, cur_len, max_len, status);
-    if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    count_launch(1);
-    return SPEC_OK;
+    return launch_chained(advance_lengths_kernel, (batch + 127) / 128, 128, stream, committed, n_accepted, batch, k, ctx_verify,
+                          cur_len, max_len, status);
 }
 
 int controller_update_launch(float* state, const float* entropy, int k, const int32_t* n_accepted, float beta,
                              cudaStream_t stream)
 {
-    controller_update_kernel<<<1, 32, 0, stream>>>(state, entropy, k, n_accepted, beta);
-    if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    count_launch(1);
-    return SPEC_OK;
+    return launch_chained(controller_update_kernel, 1, 32, stream, state, entropy, k, n_accepted, beta);
 }
 
 int controller_select_launch(const float* state, const float* entropy, int n, const int32_t* cand, int n_cand,
@@ -388,10 +469,8 @@ int controller_select_launch(const float* state, const float* entropy, int n, co
                              cudaStream_t stream)
 {
     if (n > kMaxDrafted) return SPEC_ERR_UNSUPPORTED_SHAPE;
-    controller_select_kernel<<<1, 32, 0, stream>>>(state, entropy, n, cand, n_cand, c_d, c_v, k_star, p_out, score_out);
-    if (cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
-    count_launch(1);
-    return SPEC_OK;
+    return launch_chained(controller_select_kernel, 1, 32, stream, state, entropy, n, cand, n_cand, c_d, c_v, k_star, p_out,
+                          score_out);
 }
 
 }  // namespace spec
