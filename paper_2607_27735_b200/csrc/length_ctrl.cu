@@ -162,9 +162,7 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
     __shared__ Arg warp_arg[kEntThreads / 32];
     __shared__ Mst cta_part;
     __shared__ Arg cta_arg;
-    // The entropies usually follow a pass over the same logits (acceptance), whose last rows are still in L2: they are
-    // taken from the end.  (576 rows of 128 K bf16 logits, 148 MB, after their argmax: 30 -> @@ us.)
-    const int CS = gridDim.x, rank = blockIdx.x, row = ENT && !ARG ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    const int CS = gridDim.x, rank = blockIdx.x, row = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     stream_wait();
     const char* base = static_cast<const char*>(logits) + (int64_t)row * row_stride * (DT == 1 ? 2 : 4);
@@ -208,7 +206,7 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
         for (int v = v0 + tid; v < v1; v += kEntThreads) fold1<ENT, ARG>(acc, arg, load_logit<DT>(base, v), v);
     }
     // warp, CTA, cluster: merged in a fixed order, every level a tree over the lanes of a warp (partials fetched one
-    // after the other by a single thread cost a latency each: 5.3 -> @@ us for 8 rows)
+    // after the other by a single thread cost a latency each: 5.3 -> 4.5 us for 8 rows)
     merge_lanes<ENT, ARG, 32>(acc, arg);
     if (lane == 0) {
         warp_part[warp] = acc;
