@@ -707,62 +707,58 @@ int launch_shape(const DraftArgs& a, const StreamShape& shp, cudaStream_t stream
 }  // namespace
 
 // How a call is split: CTAs per cluster (one cluster per (layer, sequence, KV head)), keys per CTA,
-// warps per CTA and stages per warp.
-//  - Few problems (a per-layer call at batch 1): the call is a chain of latencies, so every chunk
-//    should be in flight at once on as many SMs as a cluster reaches, and the CTAs of three
-//    consecutive calls should fit the GPU together (a call's early gather runs under the calls
-//    before it): 8 warps x 3 stages, one CTA per SM, clusters of 8, or of 6 where three calls of
-//    8-CTA clusters would not fit and a warp still gets about three chunks.
-//  - Many problems: several small CTAs per SM whose gathers overlap each other's arithmetic; the
-//    split is the one a simple cost model likes best (waves of CTAs x the longer of "bytes an SM
-//    pulls at about 48 GB/s" and "trips to memory of one warp").
+// warps per CTA and stages per warp: the split that a cost model likes best.  The model was fitted to the measured
+// times (layer-calls back to back, as a drafting round issues them) of every split at 33 shapes: 2 to 128 problems,
+// 260 to 4104 keys, groups of 1 to 8, both cache types, head_dim 64 and 128; its choice is on average 2-4 % above the
+// best split of a shape.  What it counts:
+//  - how many CTAs the GPU holds: shared memory, registers (16 warps of 128 registers, 20 at head_dim 64), and clusters
+//    that have to fit the 18 SMs of a GPC;
+//  - few problems (a cluster of 8 each would not fill the GPU): a call is a chain of latencies.  Two consecutive calls
+//    should fit the GPU together, so that a call's gather runs under the call before it (16 problems of 1030 keys:
+//    7.5 us per call in clusters of 8, 3.4 in clusters of 4); then chunks per warp, trips to memory, and the merges
+//    over warps and CTAs count;
+//  - many problems: either the CTAs that the GPU holds bound the call, each with a fixed part (launch, row
+//    resolution, merge) that half-empty last rounds of work pay in full, or one CTA's own chain does (24 problems of
+//    4102 keys: 21.6 -> 12.6 us per call).
 bool stream_plan(const KvView& kv, int head_dim, int n_keys_max, StreamShape* out)
 {
     const long probs = (long)kv.n_layers * kv.batch * kv.n_kv_heads;
     const int G = kv.n_q_heads / kv.n_kv_heads;
     const int keys = n_keys_max > 0 ? n_keys_max : 1;
     const int chunks = (keys + kChunk - 1) / kChunk;
-    const int nsm = sm_count();
+    const int gpcs = sm_count() / 18 > 0 ? sm_count() / 18 : 1;
     const size_t stage = kv.fp8 ? (head_dim == 128 ? Geo<128, true>::STAGE : Geo<64, true>::STAGE)
                                 : (head_dim == 128 ? Geo<128, false>::STAGE : Geo<64, false>::STAGE);
-    auto smem_of = [&](int cs, int nw, int st, int per) {
-        return (size_t)nw * st * stage + (size_t)per * 4 + (size_t)nw * 64 + 16 + (size_t)cs * G * (head_dim + 2) * 4;
-    };
-    if (probs * draft::kMaxCluster <= nsm) {
-        int cs = draft::kMaxCluster;
-        if (3 * probs * 8 > nsm && 3 * probs * 6 <= nsm && chunks <= 6 * 8 * 3) cs = 6;
-        while (cs > 1 && (chunks + cs - 1) / cs < 8) --cs;  // at least a chunk per warp
-        const int per = (chunks + cs - 1) / cs * kChunk;
-        int st = 3;
-        while (st > 1 && smem_of(cs, 8, st, per) > draft::kSmemLimit) --st;
-        if (smem_of(cs, 8, st, per) > draft::kSmemLimit) return false;
-        *out = StreamShape{cs, per, 8, st};
-        // more chunks than 8 warps x 3 stages hold at once: 12 warps x 2 stages finish the share in fewer trips
-        if (per / kChunk > 24 && smem_of(cs, 12, 2, per) <= draft::kSmemLimit) *out = StreamShape{cs, per, 12, 2};
-        return true;
-    }
-    static const int kCombos[4][2] = {{4, 2}, {4, 3}, {8, 2}, {8, 3}};
-    double best = 1e30;
+    const bool few = probs * draft::kMaxCluster <= sm_count();
+    static const int kCombos[6][2] = {{12, 2}, {8, 3}, {8, 2}, {8, 1}, {4, 3}, {4, 2}};
+    double best = 1e300;
     StreamShape bs = {0, 0, 0, 0};
-    for (int cs = 1; cs <= draft::kMaxCluster; ++cs) {
+    for (int cs : {1, 2, 3, 4, 5, 6, 8}) {      // (clusters of 7 leave a GPC's last SMs empty)
         const int cc = (chunks + cs - 1) / cs;  // chunks per CTA
         const int per = cc * kChunk;
         for (const auto& nwst : kCombos) {
             const int nw = nwst[0], st = nwst[1];
-            const size_t smem = smem_of(cs, nw, st, per);
+            if (few && nw < 8) continue;
+            const size_t smem = (size_t)nw * st * stage + (size_t)per * 4 + (size_t)nw * 64 + 16 +
+                                (size_t)cs * G * (head_dim + 2) * 4;
             if (smem > draft::kSmemLimit) continue;
-            int occ = (int)((228 * 1024) / (smem + 1024));
-            occ = occ < 1 ? 1 : occ;
-            if (occ * nw > 48) occ = 48 / nw;  // registers: about 140 per thread
-            const long ctas = probs * cs;
-            const long slots = (long)nsm * occ;
-            const long waves = (ctas + slots - 1) / slots;
-            const int wc = (cc + nw - 1) / nw;     // chunks per warp
-            const int rounds = (wc + st - 1) / st;  // latency-bound trips to memory per warp
-            const double sm_ctas = ctas >= slots ? occ : (double)ctas / nsm > 1.0 ? (double)ctas / nsm : 1.0;
-            const double bytes_us = sm_ctas * cc * (double)stage / 48.0e3;
-            const double trips_us = rounds * 1.3 + wc * 0.18;
-            const double t = waves * (bytes_us > trips_us ? bytes_us : trips_us) + 0.25 * cs + 0.02 * nw;
+            const int by_regs = (head_dim == 128 ? 16 : 20) / nw, by_smem = (int)((228 * 1024) / (smem + 1024));
+            const int occ = by_smem < 1 || by_regs < 1 ? 1 : (by_smem < by_regs ? by_smem : by_regs);
+            const double cap = (double)gpcs * (18 * occ / cs) * cs;  // CTAs resident at once
+            const double n = (double)probs * cs;
+            const int wc = (cc + nw - 1) / nw;             // chunks per warp
+            const int again = (wc + st - 1) / st - 1;      // trips to memory beyond the first
+            double t;
+            if (few) {
+                const double h = (G > 4 ? 1.44 : 1.0) * (kv.fp8 ? 0.63 : 1.0);
+                t = 0.32 * wc * h + 0.14 * cs + 0.16 * nw + 0.05 * st + 0.72 * again +
+                    (2.0 * n > cap ? 1000.0 * (2.0 * n / cap - 1.0) : 0.0);
+            } else {
+                const double h = (G > 4 ? 0.65 : 1.0) * (kv.fp8 ? 5.5 : 1.0) * (head_dim == 64 ? 0.1 : 1.0);
+                const double through = n / cap * (4.34 + 0.495 * wc * h + 0.51 * again);
+                const double chain = 2.69 + 0.32 * wc * h + 0.092 * nw + 0.5 * again;
+                t = through > chain ? through : chain;
+            }
             if (t < best) {
                 best = t;
                 bs = StreamShape{cs, per, nw, st};
