@@ -141,6 +141,15 @@ struct Sched {
 };
 static_assert(sizeof(Sched) <= 1536, "fits between the histogram and the row partials");
 
+// A sequence's length as it is in memory now, clamped: a length outside [n_q, max_ctx_len] (the launch, the score cache
+// and the output rows were sized for that range) is reported once the launch's dependency is resolved.
+__device__ __forceinline__ int read_len(const FastParams& p, int b, int* raw = nullptr)
+{
+    const int t = __ldcg(p.a.ctx_len + b);
+    if (raw) *raw = t;
+    return min(max(t, p.a.n_q), p.a.max_ctx_len);
+}
+
 __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
 {
     Work w;
@@ -158,11 +167,7 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     valid = valid && seq < sc.seq0[f + 1] - sc.seq0[f];
     const int at = sc.seq0[f] + (valid ? seq : 0);
     const int b = sc.sorted ? sc.ord[at] : at;
-    // a length outside [n_q, max_ctx_len] is clamped (the launch, the score cache and the output rows were
-    // sized for that range) and reported
-    const int t = p.a.ctx_len[b];
-    w.T = min(max(t, p.a.n_q), p.a.max_ctx_len);
-    if (t != w.T) set_status(p.status, SPEC_ERR_BAD_INDEX);
+    w.T = sc.sorted ? sc.len[b] : read_len(p, b);
     const int nb = (w.T + kTile - 1) / kTile;
     const int n = min(size, nb);  // every CTA of a problem has a tile
     valid = valid && rank < n;
@@ -180,6 +185,73 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     w.prob = (layer * p.a.kv.batch + b) * p.a.kv.n_kv_heads + h;
     sc.work[unit % kWorkTab] = w;
 }
+// Lengths, their order, classes and this CTA's first units: one warp.
+__device__ __noinline__ void make_schedule(const FastParams& p, Sched& sc)
+{
+    const int lane = threadIdx.x & 31;
+    const int B = p.a.kv.batch, LH = p.a.kv.n_layers * p.a.kv.n_kv_heads;
+    const bool sorted = B <= kSortMax;
+    int cnt[kMaxClass];
+#pragma unroll
+    for (int f = 0; f < kMaxClass; ++f) cnt[f] = 0;
+    if (!sorted) cnt[0] = B;
+#pragma unroll 1
+    for (int i = 0; i < 2 && sorted; ++i) {
+        const int b = lane + 32 * i;
+        sc.len[b] = b < B ? read_len(p, b) : 0;
+        if (B <= 32) break;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < 2 && sorted && 32 * i < B; ++i) {
+        const int b = lane + 32 * i, T = sc.len[b];
+        int before = 0;
+#pragma unroll 1
+        for (int j = 0; j < B; ++j) before += (sc.len[j] > T || (sc.len[j] == T && j < b)) ? 1 : 0;
+        int f = -1;
+        if (b < B) {
+            sc.ord[before] = (uint16_t)b;
+            const int nb = (T + kTile - 1) / kTile;
+            f = p.n_cls - 1;
+            while (f > 0 && p.cls_size[f] * p.n_cache < nb) --f;
+        }
+#pragma unroll
+        for (int c = 0; c < kMaxClass; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, f == c));
+    }
+#pragma unroll
+    for (int f = kMaxClass - 1; f > 0; --f) {
+        if (f < p.n_cls && 2 * cnt[f] * LH <= p.HG * p.cls_subs[f]) {
+            cnt[f - 1] += cnt[f];
+            cnt[f] = 0;
+        }
+    }
+    // rounds of a class, a class per lane
+    int mine = 0;
+#pragma unroll
+    for (int f = 0; f < kMaxClass; ++f) mine = lane == f ? cnt[f] : mine;
+    const int slots = lane < p.n_cls ? p.HG * p.cls_subs[lane] : 1;
+    const int rounds = (mine * LH + slots - 1) / slots;
+    int u = 0, q = 0;
+#pragma unroll
+    for (int f = 0; f <= kMaxClass; ++f) {
+        if (lane == 0) {
+            sc.unit0[f] = u;
+            sc.seq0[f] = q;
+        }
+        u += __shfl_sync(0xffffffffu, rounds, f);
+        if (f < kMaxClass) q += cnt[f];
+    }
+    u -= __shfl_sync(0xffffffffu, rounds, kMaxClass);
+    if (lane == 0) {
+        sc.n_units = u;
+        sc.sorted = sorted ? 1 : 0;
+        sc.limit = min(u, kWorkTab);
+    }
+    __syncwarp();
+    static_assert(kWorkTab == 32, "a unit per lane");
+    if (lane < u) put_work(p, sc, lane);
+}
+
 __device__ __forceinline__ Work get_work(const Sched& sc, int unit) { return sc.work[unit % kWorkTab]; }
 
 // The waits of this kernel poll the abort flag and carry no clock of their own: whatever they wait for comes from the
@@ -324,6 +396,12 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         fac_s[r] = 0.f;
     }
     fence_proxy_async();
+    // The schedule is made from the lengths as they are now, before the launch's dependency is resolved (the kernel
+    // before may still be writing them: they are read again and compared after the wait below): its latencies and
+    // first instruction fetches then hide behind the previous launch's end.
+    if (warp == 0) make_schedule(p, sc);
+    if (warp == 3 && lane < 3)
+        asm volatile("prefetch.tensormap [%0];" ::"l"(lane == 0 ? &tm_k : (lane == 1 ? &tm_v : &tm_q)) : "memory");
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -337,68 +415,17 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
-    if (warp == 0) {  // the schedule (see Sched): lengths, their order, classes, this CTA's first units
-        const int B = p.a.kv.batch, LH = p.a.kv.n_layers * p.a.kv.n_kv_heads;
-        const bool sorted = B <= kSortMax;
-        int cnt[kMaxClass];
-#pragma unroll
-        for (int f = 0; f < kMaxClass; ++f) cnt[f] = 0;
-        if (!sorted) cnt[0] = B;
-#pragma unroll 1
-        for (int i = 0; i < 2 && sorted; ++i) {
-            const int b = lane + 32 * i;
-            sc.len[b] = b < B ? min(max(p.a.ctx_len[b], p.a.n_q), p.a.max_ctx_len) : 0;
-            if (B <= 32) break;
+    if (warp == 0) {
+        // the schedule stands if the lengths are what they were when it was made; lengths out of range are reported
+        const bool sorted = p.a.kv.batch <= kSortMax;
+        bool same = sorted;
+        for (int b = lane; b < p.a.kv.batch; b += 32) {
+            int raw;
+            const int T = read_len(p, b, &raw);
+            if (raw != T) set_status(p.status, SPEC_ERR_BAD_INDEX);
+            if (sorted) same = same && sc.len[b] == T;
         }
-        __syncwarp();
-#pragma unroll 1
-        for (int i = 0; i < 2 && sorted && 32 * i < B; ++i) {
-            const int b = lane + 32 * i, T = sc.len[b];
-            int before = 0;
-#pragma unroll 1
-            for (int j = 0; j < B; ++j) before += (sc.len[j] > T || (sc.len[j] == T && j < b)) ? 1 : 0;
-            int f = -1;
-            if (b < B) {
-                sc.ord[before] = (uint16_t)b;
-                const int nb = (T + kTile - 1) / kTile;
-                f = p.n_cls - 1;
-                while (f > 0 && p.cls_size[f] * p.n_cache < nb) --f;
-            }
-#pragma unroll
-            for (int c = 0; c < kMaxClass; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, f == c));
-        }
-#pragma unroll
-        for (int f = kMaxClass - 1; f > 0; --f) {
-            if (f < p.n_cls && 2 * cnt[f] * LH <= p.HG * p.cls_subs[f]) {
-                cnt[f - 1] += cnt[f];
-                cnt[f] = 0;
-            }
-        }
-        // rounds of a class, a class per lane
-        int mine = 0;
-#pragma unroll
-        for (int f = 0; f < kMaxClass; ++f) mine = lane == f ? cnt[f] : mine;
-        const int slots = lane < p.n_cls ? p.HG * p.cls_subs[lane] : 1;
-        const int rounds = (mine * LH + slots - 1) / slots;
-        int u = 0, q = 0;
-#pragma unroll
-        for (int f = 0; f <= kMaxClass; ++f) {
-            if (lane == 0) {
-                sc.unit0[f] = u;
-                sc.seq0[f] = q;
-            }
-            u += __shfl_sync(0xffffffffu, rounds, f);
-            if (f < kMaxClass) q += cnt[f];
-        }
-        u -= __shfl_sync(0xffffffffu, rounds, kMaxClass);
-        if (lane == 0) {
-            sc.n_units = u;
-            sc.sorted = sorted ? 1 : 0;
-            sc.limit = min(u, kWorkTab);
-        }
-        __syncwarp();
-        static_assert(kWorkTab == 32, "a unit per lane");
-        if (lane < u) put_work(p, sc, lane);
+        if (!__all_sync(0xffffffffu, same)) make_schedule(p, sc);
     }
     __syncthreads();
     const int U = sc.n_units;
