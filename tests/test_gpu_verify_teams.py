@@ -1,0 +1,77 @@
+"""Verification of batches whose sequences run on teams of CTAs, parts of a team and single CTAs (score-cache kernel):
+lengths around the edges of key tiles and of a part's capacity, more rounds than the work table holds, more sequences
+than the schedule sorts, many short sequences back to back.  Against the oracle at 2e-3, the bar of every
+verification test, and bit for bit between repeated passes (the reductions run in a fixed order)."""
+import dataclasses
+
+import pytest
+import torch
+
+import oracle
+from paper_2607_27735_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+TOL = 2e-3
+
+SHAPES = [  # (contexts, query heads, KV heads, head_dim, rows, page)
+    ([127, 128, 129, 255, 257, 1023, 1025], 8, 2, 128, 5, 0),
+    ([9, 4096, 9, 700, 2600], 32, 8, 128, 9, 16),               # one long sequence among short ones; T = n_q
+    ([1364, 1200, 1309, 332, 541, 404, 959, 601, 419, 663, 1292, 728], 8, 8, 128, 6, 0),  # a CTA per problem
+    ([1792, 1793, 3584, 3585, 7000, 512], 8, 2, 64, 7, 64),      # a part's capacity at 14 tiles, +- 1
+    ([300 + 17 * i for i in range(70)], 4, 2, 128, 3, 0),        # more sequences than are sorted
+]
+
+
+def make(ctx, hq, hkv, d, n_q, page, layers=1, seed=1):
+    cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=n_q, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, planted=4,
+                              batch=len(ctx), n_layers=layers, page_size=page, shuffled_pages=page > 0, seed=seed)
+    return inputs.make_case(cfg, device="cuda", ctx_override=list(ctx))
+
+
+def check(case, T, out_bf16=False):
+    out, lse, stats, ws = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, T, out_bf16=out_bf16)
+    assert binding.read_status(ws) == 0
+    assert binding.last_verify_impl() == binding.VERIFY_TCGEN05_CACHED
+    o_out, o_lse, o_stats = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, stats.shape[-1])
+    # bf16 output: half a step of 2^-8 of the largest value on top
+    bar = TOL + (o_out.abs().max().item() * 2.0 ** -8 if out_bf16 else 0.0)
+    assert (out.cpu().double() - o_out).abs().max().item() <= bar
+    assert (lse.cpu().double() - o_lse).abs().max().item() <= TOL
+    for b, t in enumerate(case.ctx_len.tolist()):
+        assert (stats[:, b, :, :t].cpu().double() - o_stats[:, b, :, :t]).abs().max().item() <= TOL
+    return out, lse, stats, ws
+
+
+@pytest.mark.parametrize("ctx,hq,hkv,d,n_q,page", SHAPES)
+@pytest.mark.parametrize("out_bf16", [False, True])
+def test_ragged_batches(ctx, hq, hkv, d, n_q, page, out_bf16):
+    check(make(ctx, hq, hkv, d, n_q, page), max(ctx), out_bf16)
+
+
+@pytest.mark.parametrize("slack", [0, 3000, 60000])
+def test_capacity_far_above_the_lengths(slack):
+    """The split is sized for the longest context the call allows; the lengths in device memory may be far below."""
+    ctx = [700, 3000, 150]
+    cap = max(ctx) + slack
+    case = make([cap] * 3, 32, 8, 128, 5, 0)
+    case = dataclasses.replace(case, ctx_len=torch.tensor(ctx, dtype=torch.int32, device="cuda"))
+    check(case, cap)
+
+
+def test_more_rounds_than_the_work_table():
+    check(make([4100, 3000, 5000, 4500], 32, 8, 128, 9, 0, layers=6), 5000)
+
+
+def test_back_to_back_passes_are_bit_identical():
+    """Nothing waits between the passes: partials, counters and score regions are used again by the next launch."""
+    for ctx, hq, hkv, n_q in (([2061, 1571, 2799, 3337, 2804, 1373, 4224, 1213, 2610, 1552], 16, 2, 5),
+                              ([851, 957, 1057, 1061, 1046, 1766], 16, 2, 8)):
+        a, b = make(ctx, hq, hkv, 128, n_q, 0, seed=1), make(ctx, hq, hkv, 128, n_q, 0, seed=2)
+        out, lse, stats, ws = check(a, max(ctx))
+        want = out.clone(), stats.clone()
+        for _ in range(25):
+            binding.spec_verify_attn(b.kv, b.q_verify, b.ctx_len, max(ctx), out=out, lse=lse, stats=stats, workspace=ws)
+            binding.spec_verify_attn(a.kv, a.q_verify, a.ctx_len, max(ctx), out=out, lse=lse, stats=stats, workspace=ws)
+            torch.cuda.synchronize()
+            assert torch.equal(out, want[0]) and torch.equal(stats, want[1])
+        assert binding.read_status(ws) == 0
