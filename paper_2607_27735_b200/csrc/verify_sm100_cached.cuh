@@ -774,58 +774,65 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const int lo = sg.rank * E4 / sg.n, hi = (sg.rank + 1) * E4 / sg.n;
             const float4* src = reinterpret_cast<const float4*>(
                 p.o_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R * kD);
-            // Sixteen loads in flight as four groups of four: with up to four partials the groups are four elements, 32
-            // apart, else they are sixteen partials of one element.
-            const bool few = sg.n <= 4;
-            const int ne = few ? 4 : 1;
             const int64_t out0 = ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D;
+            auto store = [&](int e, const float4& v) {
+                const int d = 4 * (e & (kD / 4 - 1));
+                if (d >= p.D) return;  // head_dim 64: the partial's upper columns are padding
+                const int64_t at = out0 + roff_s[e / (kD / 4)] + d;
+                if (p.a.out_bf16)
+                    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.a.out) + at) =
+                        make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+                else
+                    *reinterpret_cast<float4*>(p.a.out + at) = v;
+            };
+            if (sg.n <= 4) {  // few partials, many elements: three elements of every partial in flight
 #pragma unroll 1
-            for (int e0 = lo + tid; e0 < hi; e0 += 32 * ne) {
-                float4 acc[4];
+                for (int e0 = lo + tid; e0 < hi; e0 += 96) {
+                    float4 acc[3];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-                for (int k0 = 0; k0 < sg.n; k0 += 16) {
-                    float4 x[16];
+                    for (int u = 0; u < 3; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float4 x[4][3];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int left = few ? (e0 + 32 * u < hi ? sg.n : 0) : sg.n - k0 - 4 * u;  // partials of this group
-                        const float4* q = src + (few ? e0 + 32 * u : (k0 + 4 * u) * E4 + e0);
+                    for (int k = 0; k < 4; ++k)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            x[4 * u + k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (k < left) x[4 * u + k] = __ldcg(q);
-                            q += E4;
+                        for (int u = 0; u < 3; ++u) {
+                            x[k][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (k < sg.n && e0 + 32 * u < hi) x[k][u] = __ldcg(src + k * E4 + e0 + 32 * u);
+                        }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int u = 0; u < 3; ++u) {
+                            acc[u].x += x[k][u].x;
+                            acc[u].y += x[k][u].y;
+                            acc[u].z += x[k][u].z;
+                            acc[u].w += x[k][u].w;
+                        }
+#pragma unroll
+                    for (int u = 0; u < 3; ++u)
+                        if (e0 + 32 * u < hi) store(e0 + 32 * u, acc[u]);
+                }
+            } else {
+                for (int e = lo + tid; e < hi; e += 32) {
+                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k0 = 0; k0 < sg.n; k0 += 16) {  // batches of 16 independent loads
+                        float4 x[16];
+                        const float4* q = src + (int64_t)k0 * E4 + e;
+                        const int n_ld = sg.n - k0;
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) {
+                            x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (u < n_ld) x[u] = __ldcg(q + u * E4);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) {
+                            acc.x += x[u].x;
+                            acc.y += x[u].y;
+                            acc.z += x[u].z;
+                            acc.w += x[u].w;
                         }
                     }
-#pragma unroll
-                    for (int u = 0; u < 16; ++u) {
-                        acc[u >> 2].x += x[u].x;
-                        acc[u >> 2].y += x[u].y;
-                        acc[u >> 2].z += x[u].z;
-                        acc[u >> 2].w += x[u].w;
-                    }
-                }
-                if (!few) {
-#pragma unroll
-                    for (int u = 1; u < 4; ++u) {
-                        acc[0].x += acc[u].x;
-                        acc[0].y += acc[u].y;
-                        acc[0].z += acc[u].z;
-                        acc[0].w += acc[u].w;
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + 32 * u, d = 4 * (e & (kD / 4 - 1));
-                    if (u < ne && e < hi && d < p.D) {  // (head_dim 64: the partial's upper columns are padding)
-                        const int64_t at = out0 + roff_s[e / (kD / 4)] + d;
-                        if (p.a.out_bf16)
-                            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.a.out) + at) =
-                                make_uint2(pack_bf16(acc[u].x, acc[u].y), pack_bf16(acc[u].z, acc[u].w));
-                        else
-                            *reinterpret_cast<float4*>(p.a.out + at) = acc[u];
-                    }
+                    store(e, acc);
                 }
             }
             __syncwarp();
