@@ -1050,15 +1050,21 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     for (int i = 0; i < NH; ++i)
                         if (i < hidden) sc[i] = kNegBig;
                 }
-                // running max is refreshed only when some lane's score beats it by 2^8: one
-                // warp-uniform branch per tile, one ex2 per element otherwise
+                // The reference of a column is one for the whole warp, so that the sums of its lanes simply add up at the
+                // end: lane 0's first score, moved up to the tile's largest when some score is 2^8 above it (one
+                // warp-uniform branch per tile).  (A maximum over the lanes at the end of every unit cost 100
+                // cycles per column: 3.5 us per launch at 128 rows.)
+                if (c == 0) {
+#pragma unroll
+                    for (int i = 0; i < NH; ++i) m[i] = __shfl_sync(0xffffffffu, sc[i], 0);
+                }
                 bool need = false;
 #pragma unroll
                 for (int i = 0; i < NH; ++i) need |= sc[i] > m[i] + 8.f;
                 if (__any_sync(0xffffffffu, need)) {
 #pragma unroll
                     for (int i = 0; i < NH; ++i) {
-                        const float mn = fmaxf(m[i], sc[i]);
+                        const float mn = fmaxf(m[i], warp_max_all(sc[i]));
                         l[i] *= ex2(m[i] - mn);
                         m[i] = mn;
                     }
@@ -1069,13 +1075,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             if (!ok) break;
             // reduce (m, l) over the 32 key lanes of this warp, then over the 4 warps via smem
             {
-#pragma unroll
-                for (int i = 0; i < NH; ++i) {
-                    const float M = warp_max_all(m[i]);
-                    l[i] *= ex2(m[i] - M);
-                    m[i] = M;
-                }
-                if (lane == 0) {
+                if (lane == 0) {  // (the references are the same on all lanes)
 #pragma unroll
                     for (int i = 0; i < NH; i += 4)
                         *reinterpret_cast<float4*>(red_m + sw * NC + i) = make_float4(m[i], m[i + 1], m[i + 2], m[i + 3]);
