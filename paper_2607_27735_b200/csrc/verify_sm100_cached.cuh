@@ -969,22 +969,28 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(B.o_empty);
-            // no other CTA has a part of the problem: this is the output; else a partial
-            const bool alone = sg.n == 1, half = alone && p.a.out_bf16;
-            const int64_t out0 =
-                ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D;
-            char* dst = reinterpret_cast<char*>(alone ? p.a.out : p.o_part) +
-                        ((alone ? out0 : obase) + key_l) * (half ? 2 : 4);
-            const int R_key = alone && key_l >= p.D ? 0 : R;  // (head_dim 64: the upper half of the lanes is padding)
+            auto value = [&](int i) -> float {
+                const float fac = SC ? fac_s[c0 + i] * vsc : fac_s[c0 + i];
+                return (F8 ? fmaf(__uint_as_float(w[i]), 1.f / kLoExp, __uint_as_float(v[i]))
+                           : __uint_as_float(v[i]) + __uint_as_float(w[i])) * fac;
+            };
+            if (sg.n > 1) {
+                float* dst = p.o_part + obase + c0 * kD + key_l;
 #pragma unroll
-            for (int i = 0; i < NH; ++i) {
-                const int r = c0 + i;
-                if (r < R_key) {
-                    const float o = (F8 ? fmaf(__uint_as_float(w[i]), 1.f / kLoExp, __uint_as_float(v[i]))
-                                        : __uint_as_float(v[i]) + __uint_as_float(w[i])) * (SC ? fac_s[r] * vsc : fac_s[r]);
-                    const int off = alone ? roff_s[r] : r * kD;
-                    if (half) *reinterpret_cast<__nv_bfloat16*>(dst + 2 * off) = __float2bfloat16_rn(o);
-                    else *reinterpret_cast<float*>(dst + 4 * off) = o;
+                for (int i = 0; i < NH; ++i)
+                    if (c0 + i < R) dst[i * kD] = value(i);
+            } else if (key_l < p.D) {  // no other CTA has a part of the problem: this is the output
+                const int64_t out0 =
+                    ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D + key_l;
+                const bool half = p.a.out_bf16 != 0;
+                char* dst = reinterpret_cast<char*>(p.a.out) + out0 * (half ? 2 : 4);
+#pragma unroll
+                for (int i = 0; i < NH; ++i) {
+                    if (c0 + i < R) {
+                        const int off = roff_s[c0 + i];
+                        if (half) *reinterpret_cast<__nv_bfloat16*>(dst + 2 * off) = __float2bfloat16_rn(value(i));
+                        else *reinterpret_cast<float*>(dst + 4 * off) = value(i);
+                    }
                 }
             }
             __syncwarp();
@@ -1052,8 +1058,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 }
                 // The reference of a column is one for the whole warp, so that the sums of its lanes simply add up at the
                 // end: lane 0's first score, moved up to the tile's largest when some score is 2^8 above it (one
-                // warp-uniform branch per tile).  (A maximum over the lanes at the end of every unit cost 100
-                // cycles per column: 3.5 us per launch at 128 rows.)
+                // warp-uniform branch per tile).  (A maximum over the lanes at the end of every unit: 267 instead
+                // of 257 us at the 32B shape, 64 K, batch 4.)
                 if (c == 0) {
 #pragma unroll
                     for (int i = 0; i < NH; ++i) m[i] = __shfl_sync(0xffffffffu, sc[i], 0);
