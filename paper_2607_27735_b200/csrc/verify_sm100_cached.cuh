@@ -277,7 +277,7 @@ struct CBars {  // mbarrier addresses (shared space)
         pub_p1, pub_o, lse_ready, raw_full, raw_empty, q_ready;
 };
 
-// NC = score columns per softmax warpgroup, CG = number of such warpgroups (N = NC * CG):
+// NC = score columns per softmax warpgroup, CG = number of such warpgroups (R <= NC * CG <= N):
 // more, narrower warpgroups hide the latency of the serial softmax sections.
 // LP: the publisher warp combines the LSE partials (few CTAs per head); otherwise the softmax warps do.
 // PH: one Eq. 3 score per attention head (stats [.., n_q_heads, stride]) instead of per KV head,
@@ -382,6 +382,15 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         *reinterpret_cast<uint4*>(sgen + (s_q - sbase) + 16 * i) = make_uint4(0, 0, 0, 0);
     if (p.a.hist)
         for (int i = threadIdx.x; i < kScoreBins / 2; i += kBlock) hist_s[i] = 0u;
+    if (NC * CG < N) {  // row blocks of the P operand that no warpgroup has: zero once (hi and lo part of every buffer)
+        const int per = (N - NC * CG) / 8 * 128;  // 16-byte vectors of one part
+#pragma unroll 1
+        for (int i = threadIdx.x; i < 2 * p.p_bufs * per; i += kBlock) {
+            const int part = i / per, k = i - part * per, j = NC * CG / 8 + (k >> 7) + (part & 1) * (N / 8);
+            *reinterpret_cast<uint4*>(sgen + (s_p - sbase) + (part >> 1) * p_bytes + j * 2048 + (k & 127) * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
     if (p.D == 64) {  // the upper 64-wide half of every tile slot is never loaded: zero rows of V^T (and of K)
         for (int i = threadIdx.x; i < p.n_slots * 1024; i += kBlock)
             *reinterpret_cast<uint4*>(sgen + (s_slots - sbase) + (i >> 10) * kSlotBytes + 16384 + 16 * (i & 1023)) =
@@ -438,62 +447,42 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         const uint32_t box_bytes = box_rows * 128;
         const int halves = p.D / 64;  // 64-wide halves of the head dimension
         bool ok = true;
+        // A tile's boxes, one per lane (at most 16 boxes of 8 rows, for either half of the head dimension).  F8: the
+        // tile's bytes (128 per key) go to a raw stage, and the softmax warps expand them into a slot.
+        // The page table is read before the wait for a free slot: its latency (a trip to L2 per tile, which bounded
+        // the stream of 16-token pages) hides behind that wait.
         auto load_tile = [&](const CUtensorMap* map, const Work& sg, int tile) -> bool {
-            if (F8) {
-                // the tile's bytes (128 per key) go to a raw stage; the softmax warps expand them into a slot
-                const uint32_t r = ring, rph = ring_ph;
-                if (++ring == (uint32_t)p.n_raw) {
-                    ring = 0;
-                    ring_ph ^= 1;
-                }
-                bool got = true;
-                if (lane == 0) got = bar_wait(B.raw_empty + 8 * r, rph ^ 1, ctl);
-                if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
-                const int key0 = tile * kTile;
-                const int n_box = min(boxes, (sg.T - key0 + box_rows - 1) / box_rows);
-                if (lane == 0) mbar_expect_tx(B.raw_full + 8 * r, (uint32_t)n_box * box_bytes);
-                __syncwarp();
-                for (int bx = lane; bx < n_box; bx += 32) {
-                    const int pos = key0 + bx * box_rows;
-                    const int page = page_of(p.a.kv, pos), slot_in_page = pos - page * p.a.kv.page_size;
-                    int phys = p.a.kv.page_table ? __ldg(p.a.kv.page_table + (int64_t)sg.b * p.a.kv.max_pages + page)
-                                                 : sg.b * p.a.kv.max_pages + page;
-                    if (phys < 0 || phys >= p.n_pages) {
-                        set_status(p.status, SPEC_ERR_BAD_INDEX);
-                        phys = 0;
-                    }
-                    tma_load_5d(s_raw + r * 16384 + bx * box_bytes, map, B.raw_full + 8 * r, 0, slot_in_page, sg.h, phys,
-                                sg.layer, kEvictFirst);
-                }
-                __syncwarp();
-                return true;
-            }
-            const uint32_t s = ring, ph = ring_ph;
-            if (++ring == (uint32_t)p.n_slots) {
-                ring = 0;
-                ring_ph ^= 1;
-            }
-            bool got = true;
-            if (lane == 0) got = bar_wait(B.slot_empty + 8 * s, ph ^ 1, ctl);  // one lane polls
-            if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
-            // boxes of this tile that hold at least one key < T (pages past the context may not exist)
             const int key0 = tile * kTile;
+            // boxes that hold at least one key < T (pages past the context may not exist)
             const int n_box = min(boxes, (sg.T - key0 + box_rows - 1) / box_rows);
-            if (lane == 0) mbar_expect_tx(B.slot_full + 8 * s, (uint32_t)halves * n_box * box_bytes);
-            __syncwarp();
-            for (int i = lane; i < halves * n_box; i += 32) {
-                const int half = i >= n_box ? 1 : 0, bx = i - half * n_box;  // i < 2 * n_box
-                const int pos = key0 + bx * box_rows;
-                const int page = page_of(p.a.kv, pos), slot_in_page = pos - page * p.a.kv.page_size;
-                int phys = p.a.kv.page_table ? __ldg(p.a.kv.page_table + (int64_t)sg.b * p.a.kv.max_pages + page)
-                                             : sg.b * p.a.kv.max_pages + page;
+            const int n_ops = F8 ? n_box : halves * n_box;
+            const int half = !F8 && lane >= n_box ? 1 : 0, bx = lane - half * n_box;
+            const int pos = key0 + bx * box_rows;
+            const int page = page_of(p.a.kv, pos), slot_in_page = pos - page * p.a.kv.page_size;
+            int phys = 0;
+            if (lane < n_ops) {
+                phys = p.a.kv.page_table ? __ldg(p.a.kv.page_table + (int64_t)sg.b * p.a.kv.max_pages + page)
+                                         : sg.b * p.a.kv.max_pages + page;
                 if (phys < 0 || phys >= p.n_pages) {
                     set_status(p.status, SPEC_ERR_BAD_INDEX);
                     phys = 0;
                 }
-                const uint32_t dst = s_slots + s * kSlotBytes + half * 16384 + bx * box_bytes;
-                tma_load_5d(dst, map, B.slot_full + 8 * s, half * 64, slot_in_page, sg.h, phys, sg.layer, kEvictFirst);
             }
+            const uint32_t s = ring, ph = ring_ph;
+            if (++ring == (uint32_t)(F8 ? p.n_raw : p.n_slots)) {
+                ring = 0;
+                ring_ph ^= 1;
+            }
+            const uint32_t full = (F8 ? B.raw_full : B.slot_full) + 8 * s;
+            bool got = true;
+            if (lane == 0) {  // one lane polls
+                got = bar_wait((F8 ? B.raw_empty : B.slot_empty) + 8 * s, ph ^ 1, ctl);
+                if (got) mbar_expect_tx(full, (uint32_t)n_ops * box_bytes);
+            }
+            if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
+            if (lane < n_ops)
+                tma_load_5d((F8 ? s_raw + s * 16384 : s_slots + s * kSlotBytes + half * 16384) + bx * box_bytes, map, full,
+                            half * 64, slot_in_page, sg.h, phys, sg.layer, kEvictFirst);
             __syncwarp();
             return true;
         };
@@ -541,11 +530,13 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             struct Queue {
                 int u = -1, c = 0, n_t = 0;   // unit, its tile, its tiles
                 uint32_t slot = 0, ph = 0;    // ring position of the tile and the slot's phase
+                int at = 0;                   // the tile's number among all tiles, K and V
                 bool seek = true, done = false;
             } qq, pq;
             // slots of a unit: its K tiles, then its V tiles
             auto skip = [&](Queue& c, int n) {
                 c.slot += n;
+                c.at += n;
                 while (c.slot >= (uint32_t)p.n_slots) {
                     c.slot -= p.n_slots;
                     c.ph ^= 1;
@@ -572,6 +563,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             uint32_t pb = 0, pph = 0, pe = 0, o_phase = 0, q_phase = 0;
             bool ok = true;
             auto qk_ready = [&]() -> bool {
+                // A slot's phase only tells its last two fills apart, so the tile that had the slot before must have been
+                // used: with regions free for the next unit, K Q^T would otherwise take a V tile still in flight
+                // for its K tile.
+                if (qq.at >= pq.at + p.n_slots) return false;
                 if (qq.c == 0 && !mbar_test_wait(F8 ? B.q_ready : B.q_full, q_phase)) return false;
                 if (!mbar_test_wait(B.slot_full + 8 * qq.slot, qq.ph)) return false;
                 return mbar_test_wait(B.s_free + 8 * region, ((sfree_par >> region) & 1) ^ 1);
@@ -1483,6 +1478,12 @@ int launch_rows(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap&
     case n:                                                                                               \
         return lp ? launch_cfg<nc, cg, true, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream)        \
                   : launch_cfg<nc, cg, false, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream);
+    // 17 to 24 rows pad a quarter of the MMA's 32: three warpgroups of eight columns instead of four (16 chats of
+    // 0.6-6 K tokens: 57.5 -> 56.1 us per launch, five sequences of 4-30 K: 91.3 -> 88.4.  33 to 36 rows of 48 in
+    // three groups of twelve gave nothing: those launches are not bound by the softmax warps.)
+    if (fp.N == 32 && fp.R <= 24)
+        return lp ? launch_cfg<8, 3, true, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream)
+                  : launch_cfg<8, 3, false, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream);
     switch (fp.N) {  // (columns per warpgroup, warpgroups)
         SPEC_CASE(16, 8, 2)
         SPEC_CASE(32, 8, 4)

@@ -75,3 +75,20 @@ def test_back_to_back_passes_are_bit_identical():
             torch.cuda.synchronize()
             assert torch.equal(out, want[0]) and torch.equal(stats, want[1])
         assert binding.read_status(ws) == 0
+
+
+def test_two_rounds_on_fresh_tensors():
+    """Two rounds per team at five tiles per CTA and four K/V slots: the second round's K tiles come a whole turn of the
+    slot ring after the first one's V tiles, and the next K Q^T may start as soon as its score region is free."""
+    ctx, T = [20000], 20000
+    want = None
+    for it in range(150):
+        if it % 30 == 0:
+            case = make(ctx, 32, 8, 128, 9, 0, seed=1)
+        out, lse, stats, ws = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, T)
+        torch.cuda.synchronize()
+        assert binding.read_status(ws) == 0
+        if want is None:
+            want = out, lse, stats
+            check(case, T)
+        assert all(torch.equal(a, b) for a, b in zip((out, lse, stats), want))
