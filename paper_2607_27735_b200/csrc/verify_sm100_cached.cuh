@@ -255,13 +255,17 @@ __device__ __noinline__ void make_schedule(const FastParams& p, Sched& sc)
 __device__ __forceinline__ Work get_work(const Sched& sc, int unit) { return sc.work[unit % kWorkTab]; }
 
 // The waits of this kernel poll the abort flag and carry no clock of their own: whatever they wait for comes from the
-// MMA warp, whose idle timer is the watchdog of all of them, or follows a cross-CTA counter, whose wait is timed
-// (counter_wait).  A timer inlined at each of the thirty sites made the function 12 KB longer, and code that does not
-// fit the instruction cache is fetched again every unit.
+// MMA warp, whose idle timer watches over all of them, or follows a cross-CTA counter, whose wait is timed
+// (counter_wait).  A count of tries (a second and more: a try takes tens of cycles at least) ends them whatever
+// happens; the status is written at the end of the kernel.  A clock inlined at each of the thirty sites made the
+// function 12 KB longer, and code that does not fit the instruction cache is fetched again every unit.
+constexpr uint32_t kMaxTries = 1u << 27;
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const Ctl& c)
 {
-    while (!mbar_try_wait(bar, parity))
+    for (uint32_t n = 0; !mbar_try_wait(bar, parity);) {
         if (*c.abort_flag) return false;
+        if (++n > kMaxTries) *c.abort_flag = 1;
+    }
     return true;
 }
 // Barrier among the softmax warps, on an mbarrier so that the wait can be abandoned.
@@ -1412,6 +1416,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // ---- teardown ----
     tc_fence_before();
     __syncthreads();
+    if (*abort_flag && threadIdx.x == 0) set_status(p.status, SPEC_ERR_TIMEOUT);  // (unless the cause has been recorded)
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
