@@ -89,6 +89,20 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
         cached = best_hg != 0;
         // CTAs that the teams leave over join them
         if (cached && best_cph < nb) best_cph = nsm / best_hg < nb ? nsm / best_hg : nb;
+        // A single sequence: no more CTAs than its tiles per CTA need, so that the shares are even and fewer exchange
+        // partials (8 heads of 4 K: 18 -> 16 CTAs per head, 18.2 -> 17.1 us per launch; 2 heads of 111 K: 148 -> 128,
+        // 49.0 -> 45.0).
+        if (cached && kv.batch == 1) {
+            const int tpc = (nb + best_cph - 1) / best_cph;
+            best_cph = (nb + tpc - 1) / tpc;
+        }
+        // Short contexts of a batch ask for teams of a few CTAs, whose parts (4, 2, 1) fit the lengths less closely
+        // than those of a team of 24 (24, 12, 6, 3): 16 chats of 0.6-6 K tokens 54.0 -> 48.9 us per launch, 16
+        // sequences of 3 K 54.5 -> 50.5.  (Over an 8-bit cache, whose rounds cost more, 36.9 -> 40.8: not there.)
+        if (cached && best_cph < 8 && kv.batch >= 4 && nb >= 24 && nsm >= 24 && !kv.fp8) {
+            best_cph = 24;
+            best_hg = nsm / 24 < probs ? nsm / 24 : (int)probs;
+        }
     }
     if (!cached) {
         if (variant == 2 || kv.head_dim != kD || kv.fp8) return false;
