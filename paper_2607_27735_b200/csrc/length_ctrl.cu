@@ -24,7 +24,8 @@ namespace {
 // Every kernel of this file is launched with programmatic stream serialisation: its launch overlaps the end of the
 // kernel before it, whose results it waits for here.  The next kernel is let go only after that wait, so whatever
 // starts early under this kernel finds everything before this kernel complete.  (A round's scalar tail is a chain of
-// kernels of 2 us each: the gap between two of them costs as much as half a kernel.)
+// kernels of 2 us each: the gap between two of them costs as much as half a kernel.)  What an earlier kernel may have
+// written is read by ordinary loads, never through the read-only path, which the compiler could move ahead of the wait.
 __device__ __forceinline__ void stream_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -154,8 +155,8 @@ __device__ __forceinline__ void merge_lanes(Mst& acc, Arg& arg)
 // One cluster (gridDim.x CTAs) per row.  DT = 0: fp32 logits, 1: bf16 logits.  ENT: entropy[row];
 // ARG: token[row] = the smallest index of the largest logit.
 template <int DT, bool ENT, bool ARG>
-__global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict__ logits, int vocab, int64_t row_stride,
-                                                          float* __restrict__ entropy, int32_t* __restrict__ token)
+__global__ void __launch_bounds__(kEntThreads) row_kernel(const void* logits, int vocab, int64_t row_stride,
+                                                          float* entropy, int32_t* token)
 {
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ Mst warp_part[kEntThreads / 32];
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
 #pragma unroll
                 for (int j = 0; j < kUnroll; ++j)
                     if (g + j * kEntThreads < g1)
-                        w[j] = __ldg(reinterpret_cast<const uint4*>(base) + g + j * kEntThreads);
+                        w[j] = __ldcg(reinterpret_cast<const uint4*>(base) + g + j * kEntThreads);
 #pragma unroll
                 for (int j = 0; j < kUnroll; ++j)
                     if (g + j * kEntThreads < g1) fold_words<ENT, ARG>(acc, arg, w[j], (g + j * kEntThreads) * 8);
@@ -188,8 +189,8 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
 #pragma unroll
                 for (int j = 0; j < kUnroll; ++j)
                     if (g + j * kEntThreads < g1) {
-                        w[j][0] = __ldg(reinterpret_cast<const float4*>(base) + 2 * (g + j * kEntThreads));
-                        w[j][1] = __ldg(reinterpret_cast<const float4*>(base) + 2 * (g + j * kEntThreads) + 1);
+                        w[j][0] = __ldcg(reinterpret_cast<const float4*>(base) + 2 * (g + j * kEntThreads));
+                        w[j][1] = __ldcg(reinterpret_cast<const float4*>(base) + 2 * (g + j * kEntThreads) + 1);
                     }
 #pragma unroll
                 for (int j = 0; j < kUnroll; ++j)
@@ -248,8 +249,8 @@ __global__ void __launch_bounds__(kEntThreads) row_kernel(const void* __restrict
 // it equals the target's token for that position; one warp per sequence, 32 tokens at a time.
 constexpr int kAcceptWarps = 4;
 __global__ void __launch_bounds__(32 * kAcceptWarps)
-accept_kernel(const int32_t* __restrict__ target, const int32_t* __restrict__ draft, const int32_t* __restrict__ n_draft,
-              int batch, int k1, int32_t* __restrict__ n_accepted, int32_t* __restrict__ next_token)
+accept_kernel(const int32_t* target, const int32_t* draft, const int32_t* n_draft,
+              int batch, int k1, int32_t* n_accepted, int32_t* next_token)
 {
     const int b = blockIdx.x * kAcceptWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     stream_wait();
@@ -270,8 +271,8 @@ accept_kernel(const int32_t* __restrict__ target, const int32_t* __restrict__ dr
 }
 
 // Eq. "ema": state[0] <- beta state[0] + (1 - beta) mean(H_1..H_m), state[1] likewise with H_{m+1}..H_k
-__global__ void controller_update_kernel(float* state, const float* __restrict__ entropy, int k,
-                                         const int32_t* __restrict__ n_accepted, float beta)
+__global__ void controller_update_kernel(float* state, const float* entropy, int k,
+                                         const int32_t* n_accepted, float beta)
 {
     const int lane = threadIdx.x;
     stream_wait();
@@ -290,8 +291,8 @@ __global__ void controller_update_kernel(float* state, const float* __restrict__
 }
 
 // Eq. "prob" and Eq. "optimal_k"; ties go to the smaller candidate
-__global__ void controller_select_kernel(const float* __restrict__ state, const float* __restrict__ entropy, int n,
-                                         const int32_t* __restrict__ cand, int n_cand, float c_d, float c_v,
+__global__ void controller_select_kernel(const float* state, const float* entropy, int n,
+                                         const int32_t* cand, int n_cand, float c_d, float c_v,
                                          int32_t* k_star, float* p_out, float* score_out)
 {
     __shared__ float expected[kMaxDrafted];  // 1 + sum_{m <= k} prod_{i <= m} p_i at k = index + 1
@@ -352,9 +353,9 @@ __global__ void controller_select_kernel(const float* __restrict__ state, const 
 
 // Lengths of the next round, on the device: committed += accepted + 1 (the corrected token), the
 // verification context of a round with k drafted tokens, and the draft step lengths.
-__global__ void advance_lengths_kernel(int32_t* __restrict__ committed, const int32_t* __restrict__ n_accepted,
-                                       int batch, int k, int32_t* __restrict__ ctx_verify,
-                                       int32_t* __restrict__ cur_len, int max_len, int* __restrict__ status)
+__global__ void advance_lengths_kernel(int32_t* committed, const int32_t* n_accepted,
+                                       int batch, int k, int32_t* ctx_verify,
+                                       int32_t* cur_len, int max_len, int* status)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     stream_wait();

@@ -143,7 +143,7 @@ __device__ __forceinline__ void sweep(const uint32_t* __restrict__ st, int lo, i
     for (int base = lo + threadIdx.x; base < hi; base += 8 * kThreads) {
         uint32_t u[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) u[k] = base + k * kThreads < hi ? __ldg(st + base + k * kThreads) : 0u;
+        for (int k = 0; k < 8; ++k) u[k] = base + k * kThreads < hi ? __ldcg(st + base + k * kThreads) : 0u;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if (base + k * kThreads < hi) f(u[k], base + k * kThreads);
@@ -180,7 +180,7 @@ __device__ __noinline__ void select_by_sweeps(Shared& sh, const uint32_t* __rest
         int packed = 0;
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
-            u[k] = (i0 + k < hi) ? __ldg(st + i0 + k) : 0u;
+            u[k] = (i0 + k < hi) ? __ldcg(st + i0 + k) : 0u;
             if (i0 + k < hi) packed += u[k] > thr ? (1 << 16) : (u[k] == thr ? 1 : 0);
         }
         const int ex = block_exclusive_scan(sh, packed);
@@ -218,23 +218,27 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     const int64_t prob = blockIdx.x;
     const int b = (int)((prob / n_kv_heads) % batch);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int T = sel_len[b];
-    int32_t* out = indices + prob * k_total;
-    const uint32_t* st = reinterpret_cast<const uint32_t*>(stats + prob * stat_stride);
-    // counts handed over by the verification kernel: taken and cleared whatever happens below.  They cover
-    // positions [0, hist_len): usable if the candidate span lies inside
-    uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
-    const int HL = hg ? hist_len[b] : 0;
-    const bool have_hist = hg && T <= HL && T > k_total;
-    for (int i = tid; i < kBins; i += kThreads) {
-        sh.hist[i] = have_hist ? (int)hg[i] : 0;
-        if (hg) hg[i] = 0u;
-    }
+    // The launch may begin under the kernel before it (programmatic stream serialisation); everything that kernel
+    // leaves is read after this wait, and the next kernel is let go only then.
     for (int i = tid; i < kMapWords / 4; i += kThreads) reinterpret_cast<uint4*>(sh.bitmap)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
         sh.list_n = 0;
         sh.pair_n = 0;
         sh.max = 0u;
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int T = __ldcg(sel_len + b);  // (not through the read-only path, which could be moved ahead of the wait)
+    int32_t* out = indices + prob * k_total;
+    const uint32_t* st = reinterpret_cast<const uint32_t*>(stats + prob * stat_stride);
+    // counts handed over by the verification kernel: taken and cleared whatever happens below.  They cover
+    // positions [0, hist_len): usable if the candidate span lies inside
+    uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
+    const int HL = hg ? __ldcg(hist_len + b) : 0;
+    const bool have_hist = hg && T <= HL && T > k_total;
+    for (int i = tid; i < kBins; i += kThreads) {
+        sh.hist[i] = have_hist ? (int)hg[i] : 0;
+        if (hg) hg[i] = 0u;
     }
 
     if (T <= k_total) {  // everything fits: keep every position
@@ -274,7 +278,7 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
             __syncthreads();
             for (int i = tid; i < lo + (HL - hi); i += kThreads) {  // positions outside the span that were counted
                 const int pos = i < lo ? i : hi + (i - lo);
-                atomicSub(&sh.hist[__ldg(st + pos) >> 21], 1);
+                atomicSub(&sh.hist[__ldcg(st + pos) >> 21], 1);
             }
         } else {
             // 256 blocks of four vectors (64 bytes), evenly spread: eight scores per thread
@@ -333,13 +337,13 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
                 mx = max(mx, max(max(w.x, w.y), max(w.z, w.w)));
             }
             if (edge) {
-                const uint32_t u = __ldg(st + edge_pos);
+                const uint32_t u = __ldcg(st + edge_pos);
                 list[pad + edge_pos - lo] = u;
                 mx = max(mx, u);
             }
         } else {
             if (edge) {
-                const uint32_t u = __ldg(st + edge_pos);
+                const uint32_t u = __ldcg(st + edge_pos);
                 const int at = u >= floor_bits ? atomicAdd(&sh.list_n, 1) : cap;
                 if (at < cap) {
                     list[at] = u;
@@ -505,7 +509,7 @@ score_hist_kernel(const float* __restrict__ stats, int64_t stat_stride, int batc
     const int T = min(max(len[b], 0), max_len);
     const uint32_t* st = reinterpret_cast<const uint32_t*>(stats + prob * stat_stride);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < T; i += gridDim.x * blockDim.x)
-        atomicAdd(hist + prob * kBins + (__ldg(st + i) >> 21), 1u);
+        atomicAdd(hist + prob * kBins + (__ldcg(st + i) >> 21), 1u);
 }
 
 }  // namespace
@@ -527,11 +531,23 @@ int select_launch(const float* stats, int64_t stat_stride, int n_layers, int bat
     // no context is longer than a row of scores: short rows take less shared memory, and more CTAs share an SM
     const int64_t row = (stat_stride + 7) / 4 * 4;
     const int list_words = (int)(row < kListWords ? row : kListWords);
-    select_recall_kernel<<<(unsigned)probs, kThreads, (size_t)list_words * 4, stream>>>(
-        stats, stat_stride, batch, n_kv_heads, sel_len, k_sink, k_recent, k_total, list_words, indices, n_indices, hist,
-        hist_len);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)probs);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = (size_t)list_words * 4;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, select_recall_kernel, stats, stat_stride, batch, n_kv_heads, sel_len, k_sink, k_recent, k_total,
+                           list_words, indices, n_indices, hist, hist_len) != cudaSuccess) {
+        cudaGetLastError();
+        return SPEC_ERR_CUDA;
+    }
     count_launch(1);
-    return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+    return SPEC_OK;
 }
 
 int score_hist_launch(const float* stats, int64_t stat_stride, long probs, int batch, int heads, const int32_t* len,
