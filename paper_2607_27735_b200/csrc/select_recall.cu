@@ -231,11 +231,18 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     const int T = __ldcg(sel_len + b);  // (not through the read-only path, which could be moved ahead of the wait)
     int32_t* out = indices + prob * k_total;
     const uint32_t* st = reinterpret_cast<const uint32_t*>(stats + prob * stat_stride);
-    // counts handed over by the verification kernel: taken and cleared whatever happens below.  They cover
-    // positions [0, hist_len): usable if the candidate span lies inside
+    const int lo = k_sink, hi = T - k_recent;  // candidate span [lo, hi), holds > k_mid entries where T > k_total
+    const int k_mid = k_total - k_sink - k_recent;
+    const int span = hi - lo;
+    // Short spans, and spans of which a large part is kept, are list entries as they are.
+    const bool dense = span + 3 <= list_words && (span <= kDense || k_mid > span / 4);
+    bool fast = hi <= kMapWords * 32;
+    // Counts handed over by the verification kernel are cleared whatever happens below.  They cover positions
+    // [0, hist_len): usable if the candidate span lies inside.  Only the search for the floor takes them; every other
+    // form counts for itself and starts from zero.
     uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
     const int HL = hg ? __ldcg(hist_len + b) : 0;
-    const bool have_hist = hg && T <= HL && T > k_total;
+    const bool have_hist = hg && T <= HL && T > k_total && fast && !dense;
     for (int i = tid; i < kBins; i += kThreads) {
         sh.hist[i] = have_hist ? (int)hg[i] : 0;
         if (hg) hg[i] = 0u;
@@ -246,24 +253,18 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
         if (tid == 0) n_indices[prob] = T > 0 ? T : 0;
         return;
     }
-    const int lo = k_sink, hi = T - k_recent;  // candidate span [lo, hi), holds > k_mid entries
-    const int k_mid = k_total - k_sink - k_recent;
     for (int i = tid; i < k_sink; i += kThreads) out[i] = i;
     for (int i = tid; i < k_recent; i += kThreads) out[k_sink + k_mid + i] = hi + i;
     if (tid == 0) n_indices[prob] = k_total;
     if (k_mid == 0) return;
 
-    const int span = hi - lo;
     // whole 16-byte vectors of the span start at va; at most three scores at either end are left over
     const int va = lo + (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(st + lo) & 15)) >> 2 & 3);
     const int nv = hi > va ? (hi - va) >> 2 : 0;
     const uint4* vec = reinterpret_cast<const uint4*>(st + va);
     const int n_head = min(va, hi) - lo, n_end = max(hi - va - 4 * nv, 0);
     const int pad = (4 - (va - lo)) & 3;  // a dense list keeps position lo + i - pad at index i: va falls on 16 bytes
-    // Short spans, and spans of which a large part is kept, are list entries as they are.
-    const bool dense = span + 3 <= list_words && (span <= kDense || k_mid > span / 4);
     const int trips = (nv + kTrip - 1) / kTrip;
-    bool fast = hi <= kMapWords * 32;
     auto prefetch_trip = [&](int t) {
         const int v0 = t * kTrip;
         if (v0 < nv) prefetch_l2(vec + v0, (uint32_t)min(kTrip, nv - v0) * 16u);

@@ -98,3 +98,27 @@ def test_fused_histogram_over_an_8bit_cache(head_dim):
                                            score_hist=hist, hist_len=case.ctx_len)
         assert torch.equal(plain[0], fused[0]) and torch.equal(plain[1], fused[1])
         assert int(hist.abs().sum()) == 0
+
+
+# Forms of the selection that do not use the handed-over counts must not count on top of them: spans that end beyond the
+# position bitmap (131072), short spans and spans of which much is kept (the list is the whole span), with the
+# threshold among zeros or scores so small that the counts' bins lie above it.
+@pytest.mark.parametrize("T,k_total,kind", [(131072 + 64, 1024, "spread"), (131072 + 65, 1024, "spread"), (140000, 4096, "spread"),
+                                            (2000, 512, "zeros"), (2000, 512, "tiny"), (4164, 512, "zeros"),
+                                            (9000, 4000, "zeros"), (9000, 4000, "tiny"), (9000, 1000, "spread")])
+def test_counts_of_forms_that_count_for_themselves(T, k_total, kind):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    stats = torch.rand(1, 2, 2, T, generator=g, device="cuda") ** 6
+    if kind != "spread":  # a fifth of what the budget takes is positive
+        few = torch.rand(1, 2, 2, T, generator=g, device="cuda") < 0.2 * k_total / T
+        stats = torch.where(few, stats + 1e-3, torch.zeros_like(stats) if kind == "zeros" else 1e-30 * stats)
+    stats = stats.contiguous()
+    full = torch.tensor([T, T], dtype=torch.int32, device="cuda")
+    for sel in (full, full - 3):
+        hist = bins_of(stats, full).int().cuda()
+        idx, n = binding.spec_select_recall(stats, sel, 4, 64, k_total, score_hist=hist, hist_len=full)
+        plain = binding.spec_select_recall(stats, sel, 4, 64, k_total)
+        o_idx, o_n = oracle.select_recall(stats.cpu(), sel.cpu(), 4, 64, k_total)
+        assert torch.equal(plain[0].cpu(), o_idx) and torch.equal(plain[1].cpu(), o_n)
+        assert torch.equal(idx.cpu(), o_idx) and torch.equal(n.cpu(), o_n)
+        assert int(hist.abs().sum()) == 0
