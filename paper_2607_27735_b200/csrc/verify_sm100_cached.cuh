@@ -116,8 +116,14 @@ constexpr int kSortMax = 64;  // sequences, two per lane of the warp that sorts 
 // What a CTA does in one unit.  The first units are worked out in the prologue, by a thread each, and every role reads
 // them from shared memory: the arithmetic in each role's loop would be fetched from the instruction cache again every
 // unit.  Later units (launches over many layers) take the places of old ones: the publisher warp writes kWorkAhead
-// units ahead of its own and moves `limit`, the number of units that may be read.  The roles behind it are less than
-// four units off; the TMA and MMA warps, which skip units without work, do not pass the limit.
+// units ahead of its own and moves `limit`, the number of units that may be read.  An entry is neither read before it is
+// written nor overwritten before it is read:
+//  - the softmax warps keep step with the publisher: they start a unit after its arrival on `lse_ready` for the unit
+//    before, when kWorkAhead - 1 units beyond theirs are in the table (they look up to three ahead), and it passes a
+//    unit only after all of them have arrived on `pub_o` for it;
+//  - the TMA, MMA and reduction warps skip units in which they have nothing to do, so nothing ties them to the
+//    publisher: they do not pass `limit`, and say in `at` which unit they read next; the publisher waits for the
+//    slowest of them before it overwrites an entry.  (None of them can need the publisher for a unit that far back.)
 struct alignas(16) Work {
     uint16_t layer, b, h;
     uint16_t n, rank;  // CTAs of the problem (0: nothing to do in this unit), this one's number among them
@@ -134,6 +140,7 @@ struct Sched {
     Work work[kWorkTab];
     int n_units, sorted;
     volatile int limit;
+    volatile int at[3];         // next unit the TMA, MMA and reduction warps read (kept where n_units > kWorkTab)
     int unit0[kMaxClass + 1];   // first unit of a class
     int seq0[kMaxClass + 1];    // first sequence (in sorted order) of a class
     int len[kSortMax];          // as they come
@@ -246,6 +253,7 @@ __device__ __noinline__ void make_schedule(const FastParams& p, Sched& sc)
         sc.n_units = u;
         sc.sorted = sorted ? 1 : 0;
         sc.limit = min(u, kWorkTab);
+        sc.at[0] = sc.at[1] = sc.at[2] = 0;
     }
     __syncwarp();
     static_assert(kWorkTab == 32, "a unit per lane");
@@ -253,6 +261,21 @@ __device__ __noinline__ void make_schedule(const FastParams& p, Sched& sc)
 }
 
 __device__ __forceinline__ Work get_work(const Sched& sc, int unit) { return sc.work[unit % kWorkTab]; }
+// Waits until a word of the schedule is above `x` (bounded like every wait).
+__device__ __noinline__ bool wait_above(const volatile int& word, int x, const Ctl& c)
+{
+    const long long t0 = clock64();
+    while (word <= x) {
+        __nanosleep(200);
+        if (*c.abort_flag) return false;
+        if (clock64() - t0 > c.limit) {
+            report_timeout(c, 37);
+            return false;
+        }
+    }
+    __threadfence_block();
+    return true;
+}
 
 // The waits of this kernel poll the abort flag and carry no clock of their own: whatever they wait for comes from the
 // MMA warp, whose idle timer watches over all of them, or follows a cross-CTA counter, whose wait is timed
@@ -491,14 +514,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             return true;
         };
         for (int u = 0; u < U && ok; ++u) {
-            for (const long long t0 = clock64(); u >= sc.limit && ok;) {  // (see Sched; U <= kWorkTab: never)
-                __nanosleep(500);
-                if (*ctl.abort_flag || clock64() - t0 > ctl.limit) ok = false;
-            }
-            __syncwarp();
-            if (!__all_sync(0xffffffffu, ok)) {
-                ok = false;
-                break;
+            if (U > kWorkTab) {  // (see Sched)
+                ok = __all_sync(0xffffffffu, wait_above(sc.limit, u, ctl));
+                if (!ok) break;
+                if (lane == 0) sc.at[0] = u;
             }
             const Work sg = get_work(sc, u);
             if (!sg.valid()) continue;
@@ -549,7 +568,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             auto seek = [&](Queue& c, bool v) {  // on to the next unit with work, as far as the table goes
                 skip(c, v ? 0 : c.n_t);          // past the V tiles of the unit left behind
                 c.n_t = 0;
-                while (c.u + 1 < U && c.u + 1 < sc.limit) {
+                while (c.seek && c.u + 1 < U && c.u + 1 < sc.limit) {
+                    __threadfence_block();
                     ++c.u;
                     const Work sg = get_work(sc, c.u);
                     if (sg.valid()) {
@@ -557,10 +577,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                         c.c = 0;
                         c.seek = false;
                         if (v) skip(c, c.n_t);  // past the K tiles
-                        return;
                     }
                 }
-                c.done = c.u + 1 >= U;
+                if (U > kWorkTab) sc.at[1] = min(qq.u, pq.u) + 1;
+                c.done = c.seek && c.u + 1 >= U;
             };
             uint32_t sfree_par = 0;  // per cache region: parity of the next "region free" phase
             uint32_t region = 0;     // of the next K Q^T tile: regions are taken in turn, across units
@@ -669,12 +689,18 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         for (int unit = 0; unit < U && ok; ++unit) {
             const Work sg = get_work(sc, unit);
             const bool shared = sg.n > 1;  // a problem of one CTA has nothing to exchange
-            if (U > kWorkTab && lane == 0 && unit + kWorkAhead >= kWorkTab && unit + kWorkAhead < U) {
-                put_work(p, sc, unit + kWorkAhead);
-                __threadfence_block();
-                sc.limit = unit + kWorkAhead + 1;
+            if (U > kWorkTab && unit + kWorkAhead >= kWorkTab && unit + kWorkAhead < U) {
+                if (lane == 0) {  // the place of unit + kWorkAhead - kWorkTab, once everybody is past it
+                    for (int r = 0; r < 3 && ok; ++r) ok = wait_above(sc.at[r], unit + kWorkAhead - kWorkTab, ctl);
+                    if (ok) {
+                        put_work(p, sc, unit + kWorkAhead);
+                        __threadfence_block();
+                        sc.limit = unit + kWorkAhead + 1;
+                    }
+                }
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (!ok) break;
             }
-            if (U > kWorkTab) __syncwarp();
             int* c_p1 = p.counters + unit * p.n_sid + sg.sid;
             int* c_o = c_p1 + p.n_units * p.n_sid;
             if (unit >= kRing - 1) {
@@ -763,6 +789,11 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         const int tid = lane;
         bool ok = true;
         for (int unit = 0; unit < U && ok; ++unit) {
+            if (U > kWorkTab) {  // (see Sched)
+                ok = __all_sync(0xffffffffu, wait_above(sc.limit, unit, ctl));
+                if (!ok) break;
+                if (lane == 0) sc.at[2] = unit;
+            }
             const Work sg = get_work(sc, unit);
             if (sg.n <= 1) continue;  // (a problem of one CTA: the softmax warps store the output)
             int* c_o = p.counters + (p.n_units + unit) * p.n_sid + sg.sid;

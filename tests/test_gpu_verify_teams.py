@@ -9,6 +9,7 @@ import torch
 
 import oracle
 from paper_2607_27735_b200 import binding, inputs
+from verify_schedule import TABLE, schedule
 
 pytestmark = pytest.mark.gpu
 TOL = 2e-3
@@ -58,8 +59,30 @@ def test_capacity_far_above_the_lengths(slack):
     check(case, cap)
 
 
-def test_more_rounds_than_the_work_table():
+def test_several_rounds_per_team():
     check(make([4100, 3000, 5000, 4500], 32, 8, 128, 9, 0, layers=6), 5000)
+
+
+# More units than the work table holds.  "stale": a CTA has nothing to exchange for a stretch of units in which it would
+# find, 32 units back, an entry of a problem that it shared (whole teams before parts that leave the last CTA of a team idle;
+# with more than 64 sequences, which keep their order, short sequences after long ones).
+ROUNDS = [  # (contexts, query heads, KV heads, rows, layers, stale)
+    ([16000, 8000, 8000, 8000], 4, 1, 16, 64, True),
+    ([3072] * 8 + [100 + i % 29 for i in range(60)] + [2900] * 4, 8, 8, 5, 1, True),
+    ([30000], 4, 1, 16, 100, True),  # whole teams, the last round not full
+    ([300, 200, 40], 8, 8, 3, 200, False),  # a CTA per problem
+]
+
+
+@pytest.mark.parametrize("ctx,hq,hkv,n_q,layers,stale", ROUNDS)
+def test_more_rounds_than_the_work_table(ctx, hq, hkv, n_q, layers, stale):
+    case = make(ctx, hq, hkv, 128, n_q, 0, layers=layers)
+    plan = binding.describe_plan(binding.WS_VERIFY, binding._kv_struct(case.kv), n_q, max(ctx))
+    work = schedule(plan[1], plan[2], plan[5], ctx, layers * hkv)
+    assert len(work[0]) > TABLE
+    assert stale == any(mine[u][0] <= 1 and mine[u - TABLE][0] > 1 for mine in work for u in range(TABLE, len(mine)))
+    for _ in range(2):  # the second pass finds the counters as the first one left them
+        check(case, max(ctx))
 
 
 def test_back_to_back_passes_are_bit_identical():
