@@ -176,6 +176,26 @@ bool want_args(Py_ssize_t n, Py_ssize_t want)
     return false;
 }
 
+// The call itself, without the interpreter lock: a launch that waits for room in a full queue must not stop the other
+// Python threads.  What needs the lock happens before; the caller's arguments keep the tensors alive meanwhile.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    Unlocked() = default;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+    Unlocked(const Unlocked&) = delete;
+    Unlocked& operator=(const Unlocked&) = delete;
+};
+template <typename F>
+PyObject* unlocked(F f)
+{
+    int rc = 0;
+    {
+        Unlocked u;
+        rc = f();
+    }
+    return PyLong_FromLong(rc);
+}
+
 // A C++ exception (a stream query on a machine without a driver) becomes a Python one.
 template <typename F>
 PyObject* guarded(F f)
@@ -224,10 +244,13 @@ PyObject* verify(PyObject*, PyObject* const* a, Py_ssize_t n)
         }
         const at::Tensor* ws = tensor_of(a[9], "workspace");
         if (!ws) return nullptr;
-        return PyLong_FromLong(spec_verify_attn_hist(
-            &s, q, (int32_t)tq.size(2), static_cast<const int32_t*>(ctx), max_ctx, window, static_cast<float*>(out),
-            static_cast<float*>(lse), static_cast<float*>(stats), stride, ws->data_ptr(), (size_t)ws->numel(),
-            (uint32_t)flags, static_cast<uint32_t*>(hist), stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_verify_attn_hist(
+                &s, q, (int32_t)tq.size(2), static_cast<const int32_t*>(ctx), max_ctx, window, static_cast<float*>(out),
+                static_cast<float*>(lse), static_cast<float*>(stats), stride, ws->data_ptr(), (size_t)ws->numel(),
+                (uint32_t)flags, static_cast<uint32_t*>(hist), st);
+        });
     });
 }
 
@@ -249,10 +272,13 @@ PyObject* select(PyObject*, PyObject* const* a, Py_ssize_t n)
             PyErr_SetString(PyExc_ValueError, "stats: expected [layers, batch, heads, stride]");
             return nullptr;
         }
-        return PyLong_FromLong(spec_select_recall_hist(
-            static_cast<const float*>(stats), t.size(3), (int32_t)t.size(0), (int32_t)t.size(1), (int32_t)t.size(2),
-            static_cast<const int32_t*>(len), sink, recent, total, static_cast<int32_t*>(idx), static_cast<int32_t*>(cnt),
-            static_cast<uint32_t*>(hist), static_cast<const int32_t*>(hlen), nullptr, 0, stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_select_recall_hist(
+                static_cast<const float*>(stats), t.size(3), (int32_t)t.size(0), (int32_t)t.size(1), (int32_t)t.size(2),
+                static_cast<const int32_t*>(len), sink, recent, total, static_cast<int32_t*>(idx), static_cast<int32_t*>(cnt),
+                static_cast<uint32_t*>(hist), static_cast<const int32_t*>(hlen), nullptr, 0, st);
+        });
     });
 }
 
@@ -280,10 +306,13 @@ PyObject* draft(PyObject*, PyObject* const* a, Py_ssize_t n)
         }
         const at::Tensor* ws = tensor_of(a[9], "workspace");
         if (!ws) return nullptr;
-        return PyLong_FromLong(spec_sparse_draft_attn_ex(
-            &s, q, static_cast<const int32_t*>(idx), static_cast<const int32_t*>(cnt), (int32_t)ti.size(3),
-            static_cast<const int32_t*>(ts), static_cast<const int32_t*>(cl), max_tail, static_cast<float*>(out),
-            static_cast<float*>(lse), ws->data_ptr(), (size_t)ws->numel(), (uint32_t)flags, stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_sparse_draft_attn_ex(
+                &s, q, static_cast<const int32_t*>(idx), static_cast<const int32_t*>(cnt), (int32_t)ti.size(3),
+                static_cast<const int32_t*>(ts), static_cast<const int32_t*>(cl), max_tail, static_cast<float*>(out),
+                static_cast<float*>(lse), ws->data_ptr(), (size_t)ws->numel(), (uint32_t)flags, st);
+        });
     });
 }
 
@@ -316,10 +345,13 @@ PyObject* rows(PyObject*, PyObject* const* a, Py_ssize_t n)
         const int32_t dt = t->scalar_type() == at::kBFloat16 ? 1 : 0, r = (int32_t)t->size(0), v = (int32_t)t->size(1);
         // a single row's stride says nothing
         const int64_t stride = (a[1] != Py_None || r <= 1) ? std::max(t->stride(0), t->size(1)) : t->stride(0);
-        return PyLong_FromLong(a[1] == Py_None
-                                   ? spec_token_entropy(t->data_ptr(), dt, r, v, stride, static_cast<float*>(entropy), stream())
-                                   : spec_token_argmax(t->data_ptr(), dt, r, v, stride, static_cast<int32_t*>(token),
-                                                       static_cast<float*>(entropy), stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return a[1] == Py_None
+                       ? spec_token_entropy(t->data_ptr(), dt, r, v, stride, static_cast<float*>(entropy), st)
+                       : spec_token_argmax(t->data_ptr(), dt, r, v, stride, static_cast<int32_t*>(token),
+                                           static_cast<float*>(entropy), st);
+        });
     });
 }
 
@@ -335,10 +367,13 @@ PyObject* accept(PyObject*, PyObject* const* a, Py_ssize_t n)
             !dev_ptr(a[4], at::kInt, "n_accepted", &acc) || !dev_ptr(a[5], at::kInt, "next_token", &next))
             return nullptr;
         const int32_t vocab = (int32_t)t->size(2);
-        return PyLong_FromLong(spec_accept_greedy(
-            t->data_ptr(), t->scalar_type() == at::kBFloat16 ? 1 : 0, (int32_t)t->size(0), (int32_t)t->size(1), vocab, vocab,
-            static_cast<const int32_t*>(draft_p), static_cast<const int32_t*>(nd), static_cast<int32_t*>(target),
-            static_cast<int32_t*>(acc), static_cast<int32_t*>(next), stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_accept_greedy(
+                t->data_ptr(), t->scalar_type() == at::kBFloat16 ? 1 : 0, (int32_t)t->size(0), (int32_t)t->size(1), vocab, vocab,
+                static_cast<const int32_t*>(draft_p), static_cast<const int32_t*>(nd), static_cast<int32_t*>(target),
+                static_cast<int32_t*>(acc), static_cast<int32_t*>(next), st);
+        });
     });
 }
 
@@ -359,9 +394,12 @@ PyObject* advance(PyObject*, PyObject* const* a, Py_ssize_t n)
         }
         if (!dev_ptr_or_none(a[3], at::kInt, "ctx_verify", &ctx) || !dev_ptr_or_none(a[4], at::kInt, "cur_len", &cur))
             return nullptr;
-        return PyLong_FromLong(spec_advance_lengths(
-            static_cast<int32_t*>(committed), static_cast<const int32_t*>(acc), (int32_t)THPVariable_Unpack(a[0]).numel(), k,
-            max_len, ws, static_cast<int32_t*>(ctx), static_cast<int32_t*>(cur), stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_advance_lengths(
+                static_cast<int32_t*>(committed), static_cast<const int32_t*>(acc), (int32_t)THPVariable_Unpack(a[0]).numel(), k,
+                max_len, ws, static_cast<int32_t*>(ctx), static_cast<int32_t*>(cur), st);
+        });
     });
 }
 
@@ -375,9 +413,12 @@ PyObject* controller_update(PyObject*, PyObject* const* a, Py_ssize_t n)
         if (!dev_ptr(a[0], at::kFloat, "state", &state) || !dev_ptr(a[1], at::kFloat, "entropy", &entropy) ||
             !dev_ptr(a[2], at::kInt, "n_accepted", &acc) || !to_f32(a[3], &beta))
             return nullptr;
-        return PyLong_FromLong(spec_controller_update(static_cast<float*>(state), static_cast<const float*>(entropy),
-                                                      (int32_t)THPVariable_Unpack(a[1]).numel(),
-                                                      static_cast<const int32_t*>(acc), beta, stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_controller_update(static_cast<float*>(state), static_cast<const float*>(entropy),
+                                                          (int32_t)THPVariable_Unpack(a[1]).numel(),
+                                                          static_cast<const int32_t*>(acc), beta, st);
+        });
     });
 }
 
@@ -393,10 +434,13 @@ PyObject* controller_select(PyObject*, PyObject* const* a, Py_ssize_t n)
             !dev_ptr(a[5], at::kInt, "k_star", &k_star) || !dev_ptr(a[6], at::kFloat, "p", &p) ||
             !dev_ptr(a[7], at::kFloat, "score", &score))
             return nullptr;
-        return PyLong_FromLong(spec_controller_select(
-            static_cast<const float*>(state), static_cast<const float*>(entropy), (int32_t)THPVariable_Unpack(a[1]).numel(),
-            static_cast<const int32_t*>(cand), (int32_t)THPVariable_Unpack(a[2]).numel(), c_d, c_v,
-            static_cast<int32_t*>(k_star), static_cast<float*>(p), static_cast<float*>(score), stream()));
+        void* const st = stream();
+        return unlocked([&] {
+            return spec_controller_select(
+                static_cast<const float*>(state), static_cast<const float*>(entropy), (int32_t)THPVariable_Unpack(a[1]).numel(),
+                static_cast<const int32_t*>(cand), (int32_t)THPVariable_Unpack(a[2]).numel(), c_d, c_v,
+                static_cast<int32_t*>(k_star), static_cast<float*>(p), static_cast<float*>(score), st);
+        });
     });
 }
 

@@ -1,0 +1,42 @@
+"""The Python module of the native calls does not hold up other threads."""
+import threading
+import time
+
+import pytest
+import torch
+
+from paper_2607_27735_b200 import binding
+
+
+@pytest.mark.gpu
+def test_a_launch_that_waits_for_room_leaves_other_threads_running():
+    state = torch.tensor([1.0, 4.0], device="cuda")
+    entropy = torch.rand(8, device="cuda")
+    m = torch.tensor([3], dtype=torch.int32, device="cuda")
+    binding.spec_controller_update(state, entropy, m, 0.9)
+    torch.cuda.synchronize()
+    gaps, stop = [], threading.Event()
+
+    def tick():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.002)
+            now = time.perf_counter()
+            gaps.append(now - last)
+            last = now
+
+    t = threading.Thread(target=tick)
+    t.start()
+    try:
+        torch.cuda._sleep(1_000_000_000)  # half a second on the device; the launches behind it fill the queue
+        longest = 0.0
+        for _ in range(6000):
+            t0 = time.perf_counter()
+            binding.spec_controller_update(state, entropy, m, 0.9)
+            longest = max(longest, time.perf_counter() - t0)
+        torch.cuda.synchronize()
+    finally:
+        stop.set()
+        t.join()
+    assert longest > 0.1, "no launch had to wait: the test shows nothing"
+    assert max(gaps) < 0.5 * longest
