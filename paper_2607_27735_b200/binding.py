@@ -338,7 +338,7 @@ def spec_advance_lengths(committed, n_accepted, k, ctx_verify=None, cur_len=None
     """committed += n_accepted + 1 on the device (``n_accepted=None``: unchanged), then the lengths of the
     next round: ``ctx_verify`` [batch] and ``cur_len`` [k, batch] (both optional, int32).  ``max_len`` > 0
     holds a sequence whose next round would not fit the cache and records that in ``workspace``."""
-    rc = (_native or _nat()).advance(committed, n_accepted, k, ctx_verify, cur_len, max_len, workspace)
+    rc = (_native or _nat()).advance(committed, n_accepted, k, ctx_verify, cur_len, int(max_len), workspace)
     if rc != 0:
         raise SpecError(rc, "spec_advance_lengths")
     return committed

@@ -1,4 +1,4 @@
-"""The Python module of the native calls does not hold up other threads."""
+"""The Python module of the native calls: other threads run meanwhile, and arguments are taken as before it existed."""
 import threading
 import time
 
@@ -40,3 +40,10 @@ def test_a_launch_that_waits_for_room_leaves_other_threads_running():
         t.join()
     assert longest > 0.1, "no launch had to wait: the test shows nothing"
     assert max(gaps) < 0.5 * longest
+
+
+@pytest.mark.gpu
+def test_the_bound_of_the_lengths_may_be_a_float():
+    committed = torch.tensor([50, 995], dtype=torch.int32, device="cuda")
+    binding.spec_advance_lengths(committed, None, 8, max_len=1000.0)
+    assert committed.tolist() == [50, 991]
