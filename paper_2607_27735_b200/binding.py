@@ -16,6 +16,8 @@ import os
 
 import torch
 
+from .build import native_abi
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libspec_attn.so")
 
@@ -78,6 +80,9 @@ def _nat():
             from . import _spec_native
         except ImportError as e:
             raise ImportError("_spec_native is missing: run `python -m paper_2607_27735_b200.build`") from e
+        if _spec_native.abi != native_abi():
+            raise ImportError(f"_spec_native was built for {_spec_native.abi}, this is {native_abi()}: "
+                              "run `python -m paper_2607_27735_b200.build`")
         _native = _spec_native
     return _native
 

@@ -47,6 +47,23 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def native_abi() -> str:
+    """What the Python module is compiled against, as text the module carries: it uses torch's C++ interface, so a
+    module built beside another torch or interpreter must not be loaded."""
+    import torch
+
+    return f"torch {torch.__version__} python {sys.version_info[0]}.{sys.version_info[1]}"
+
+
+def _native_current() -> bool:
+    """Whether the built module is newer than its sources and compiled against this torch and interpreter."""
+    if not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < max(
+            os.path.getmtime(NATIVE_SRC), os.path.getmtime(os.path.join(ROOT, "include", "spec_attn.h"))):
+        return False
+    with open(NATIVE, "rb") as f:
+        return native_abi().encode() + b"\0" in f.read()
+
+
 def _native_obj(verbose: bool) -> str:
     """Object file of the Python module (torch's headers make it the slowest host file: compiled beside the kernels)."""
     import torch
@@ -56,7 +73,7 @@ def _native_obj(verbose: bool) -> str:
     inc = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], os.path.join(ROOT, "include"),
            os.path.join(cpp_extension.CUDA_HOME or "/usr/local/cuda", "include")]
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           *(f"-I{p}" for p in inc), "-c", NATIVE_SRC, "-o", obj]
+           f'-DSPEC_NATIVE_ABI="{native_abi()}"', *(f"-I{p}" for p in inc), "-c", NATIVE_SRC, "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
@@ -76,8 +93,7 @@ def _link_native(obj: str) -> None:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     lib_old = force or not os.path.exists(LIB) or os.path.getmtime(LIB) < _newest_dep()
-    native_old = force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < max(
-        os.path.getmtime(NATIVE_SRC), os.path.getmtime(os.path.join(ROOT, "include", "spec_attn.h")))
+    native_old = force or not _native_current()
     os.makedirs(OBJ, exist_ok=True)
     with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
         native = ex.submit(_native_obj, verbose) if native_old else None

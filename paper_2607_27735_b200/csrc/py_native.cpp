@@ -457,5 +457,10 @@ PyMODINIT_FUNC PyInit__spec_native(void)
 {
     for (int i = 0; i < N_NAMES; ++i)
         if (!(g_names[i] = PyUnicode_InternFromString(kNames[i]))) return nullptr;
-    return PyModule_Create(&kModule);
+    PyObject* m = PyModule_Create(&kModule);
+    if (m && PyModule_AddStringConstant(m, "abi", SPEC_NATIVE_ABI) != 0) {  // see build.py
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
 }

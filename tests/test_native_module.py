@@ -1,11 +1,22 @@
-"""The Python module of the native calls: other threads run meanwhile, and arguments are taken as before it existed."""
+"""The Python module of the native calls: built against the torch it is loaded beside, other threads run meanwhile, and
+arguments are taken as before it existed."""
 import threading
 import time
 
 import pytest
 import torch
 
-from paper_2607_27735_b200 import binding
+from paper_2607_27735_b200 import binding, build
+
+
+def test_module_of_another_torch_is_rebuilt_and_not_loaded(monkeypatch):
+    assert build._native_current()
+    assert binding._nat().abi == build.native_abi()
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    assert not build._native_current()  # by content, whatever its date
+    monkeypatch.setattr(binding, "_native", None)
+    with pytest.raises(ImportError, match="0.0.0"):
+        binding._nat()
 
 
 @pytest.mark.gpu
