@@ -1,6 +1,7 @@
 // Recall selection of Eq. 4: sink + TopK over the middle span + recent, per (layer, sequence,
 // KV head).  One CTA per problem.  The scores are sums of probabilities (finite, >= 0), so the
-// fp32 bit pattern orders like the value and selection works on bit patterns: integer work only.
+// fp32 bit pattern orders like the value and selection works on bit patterns: integer work only.  (Any other pattern a
+// caller leaves there, a sign bit or a NaN, is ordered as the unsigned number it is.)
 //
 // The scores are read ONCE.  A strided sample of 4096 of them gives a floor that the K_mid-th largest lies
 // above with a wide margin (6 sigma); one sweep of 16-byte loads collects what reaches the floor (a few
@@ -118,6 +119,13 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 __device__ __forceinline__ int sample_bin(uint32_t u)
 {
     return u <= kSampleBase ? 0 : min((int)((u - kSampleBase) >> kSampleShift), kBins - 1);
+}
+
+// Takes one off where u < floor, unsigned as the comparison that stores (two instructions: the borrow of u - floor; adding
+// up comparisons made the sweep of 131 K scores 4 % longer).
+__device__ __forceinline__ void less_below(int& count, uint32_t u, uint32_t floor)
+{
+    asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\tsubc.u32 %0, %0, 0;\n\t}" : "+r"(count) : "r"(u), "r"(floor));
 }
 
 // Where u >= floor: stores u and its position in the list slot at shared address `at` (positions `off` bytes further) and
@@ -364,11 +372,14 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
                 const int base = t * kTrip + tid;
                 load(x, base + kTrip);
                 if (tid == 0) prefetch_trip(t + 4);
-                int mine = 4 * kV;  // hits: less the signs of (score - floor), without a branch
+                int mine = 4 * kV;  // hits
 #pragma unroll
-                for (int k = 0; k < kV; ++k)  // (scores past the end read as 0 and the floor is above 0)
-                    mine -= (int)(((w[k].x - floor_bits) >> 31) + ((w[k].y - floor_bits) >> 31) +
-                                  ((w[k].z - floor_bits) >> 31) + ((w[k].w - floor_bits) >> 31));
+                for (int k = 0; k < kV; ++k) {  // (scores past the end read as 0 and the floor is above 0)
+                    less_below(mine, w[k].x, floor_bits);
+                    less_below(mine, w[k].y, floor_bits);
+                    less_below(mine, w[k].z, floor_bits);
+                    less_below(mine, w[k].w, floor_bits);
+                }
                 int inc = mine;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -409,8 +420,8 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
 
     // ---- the threshold on the list: bins over its own range, refined until the threshold's bin is small ----
     const int i0 = dense ? pad : 0, i1 = i0 + n_list;  // list entries
-    uint32_t bin_lo = floor_bits, width = 0xffffffffu;  // the threshold lies in [bin_lo, bin_lo + width)
-    int need = k_mid;                                   // entries to take from there
+    uint32_t bin_lo = floor_bits, last = 0xffffffffu;  // the threshold lies in [bin_lo, bin_lo + last]
+    int need = k_mid;                                  // entries to take from there
     auto each_entry = [&](auto f) {  // f(bits, list index), four neighbouring entries per thread and trip
 #pragma unroll 1
         for (int i = 4 * tid; i < i1; i += 4 * kThreads) {
@@ -427,13 +438,13 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
         for (;;) {
             each_entry([&](uint32_t u, int) {
                 const uint32_t d = u - bin_lo;
-                if (d < width) atomicAdd(&sh.hist[d >> shift], 1);
+                if (d <= last) atomicAdd(&sh.hist[d >> shift], 1);
             });
             __syncthreads();
             find_bucket(sh, need);
             need -= sh.above;
             bin_lo += (uint32_t)sh.bucket << shift;
-            width = 1u << shift;
+            last = (1u << shift) - 1u;
             if (sh.count <= kPair) break;
             if (shift == 0) {  // more than a thousand equal scores at the threshold
                 fast = false;
@@ -452,10 +463,9 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     uint32_t* pu = reinterpret_cast<uint32_t*>(sh.hist);
     int* pp = sh.hist + kPair;
     each_entry([&](uint32_t u, int i) {
-        const uint32_t d = u - bin_lo;
-        if ((int)d < 0) return;  // below the bin (scores and their differences stay below 2^31)
+        if (u < bin_lo) return;
         const int pos = dense ? lo + i - pad : lpos[i];
-        if (d >= width) {
+        if (u - bin_lo > last) {
             atomicOr(&sh.bitmap[pos >> 5], 1u << (pos & 31));
         } else {
             const int at = atomicAdd(&sh.pair_n, 1);

@@ -49,3 +49,25 @@ def test_distributions(T, kind):
         stats.scatter_(-1, where, kth.expand(1, 2, 2, 700).contiguous())
     sel_len = torch.tensor([T, T - 7], dtype=torch.int32, device="cuda")
     check(stats.contiguous(), sel_len, 4, 64, 1000)
+
+
+@pytest.mark.parametrize("T", [3000, 9000, 33333, 140000])
+@pytest.mark.parametrize("kind", ["any", "some_negative", "nan", "minus_zero"])
+def test_any_bit_pattern_is_ordered_as_an_unsigned_number(T, kind):
+    """Scores are sums of probabilities; what else may lie in the buffer changes nothing but the order."""
+    g = torch.Generator(device="cuda").manual_seed(T)
+    n = (1, 1, 2, T)
+    bits = torch.rand(n, generator=g, device="cuda").view(torch.int32)
+    odd = {"any": torch.randint(-2 ** 31, 2 ** 31, n, generator=g, device="cuda", dtype=torch.int64).int(),
+           "some_negative": (-torch.rand(n, generator=g, device="cuda")).view(torch.int32),
+           "nan": torch.full(n, -1, dtype=torch.int32, device="cuda"),
+           "minus_zero": torch.full(n, -2 ** 31, dtype=torch.int32, device="cuda")}[kind]
+    share = 1.0 if kind == "any" else 0.03
+    bits = torch.where(torch.rand(n, generator=g, device="cuda") < share, odd, bits)
+    sel_len = torch.tensor([T], dtype=torch.int32, device="cuda")
+    idx, cnt = binding.spec_select_recall(bits.view(torch.float32), sel_len, 4, 64, 1000)
+    order = (bits.long() & 0xFFFFFFFF)[..., 4:T - 64] * 2 ** 18 + torch.arange(T - 68, 0, -1, device="cuda")
+    mid = order.topk(932, dim=-1).indices.sort(dim=-1).values + 4
+    want = torch.cat([torch.arange(4, device="cuda").expand(1, 1, 2, 4), mid,
+                      torch.arange(T - 64, T, device="cuda").expand(1, 1, 2, 64)], dim=-1).int()
+    assert torch.equal(idx, want) and bool((cnt == 1000).all())
