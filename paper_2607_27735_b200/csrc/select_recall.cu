@@ -103,11 +103,13 @@ __device__ __noinline__ bool find_bucket(Shared& sh, int want)
     return sh.total >= want;
 }
 
-// 16 bytes of scores; volatile, so that a load written ahead of other work is also issued ahead of it
+// 16 bytes of scores; volatile, so that a load written ahead of other work is also issued ahead of it, and behind the
+// wait for the kernel before.  Not through the read-only path: that kernel may still be writing them when this one starts.
 __device__ __forceinline__ uint4 load_vec(const uint4* p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 // asks L2 for `bytes` (a multiple of 16) from a 16-byte aligned address; nothing waits for it
