@@ -35,11 +35,10 @@ struct FastParams {
     int cls_subs[kMaxClass];          // parts of a team
     uint32_t cls_mul[kMaxClass];      // division by cls_size (see div_by)
     int32_t cls_sh[kMaxClass];
-    int n_sid;                        // parts of all teams in the finest class
     int n_counters;                   // ints to zero at the end, the "CTAs finished" word being the one after them
-    int* counters;                    // two-sweep: [2][n_units * HG]: P1 partials done, O partials done; score cache:
-                                      // [3][n_units * n_sid], the third: reductions done; then one
-                                      // "CTAs finished" word.  All zero between calls.
+    int* counters;                    // [2][problems]: P1 partials done (two-sweep: by unit and head; score cache: by
+                                      // problem, and above the CTAs of the problem, reductions done), O partials
+                                      // done; then one "CTAs finished" word.  All zero between calls.
     float2* ml_part;                  // [kRing][CTAs][R]
     float* o_part;                    // [kRing][CTAs][R][kD] (columns >= head_dim unused)
     int* status;

@@ -32,7 +32,7 @@ EncodeTiledFn encode_fn()
 struct Plan {
     bool cached;
     int HG, cph, n_units, N, n_slots, p_bufs, box_rows, boxes, n_cache, n_raw;
-    int n_cls, cls_size[kMaxClass], cls_subs[kMaxClass], n_sid, n_counters;
+    int n_cls, cls_size[kMaxClass], cls_subs[kMaxClass], n_counters;
     size_t smem_bytes;
     size_t ctr_off, ctr_bytes, ml_off, o_off, total;
 };
@@ -137,9 +137,7 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
         pl->cls_subs[f] = pl->cph / pl->cls_size[f];
         pl->n_cls = f + 1;
     }
-    pl->n_sid = pl->HG * pl->cls_subs[pl->n_cls - 1];
-    // score cache: every class may end in a round that is not full
-    pl->n_counters = cached ? 3 * (pl->n_units + kMaxClass) * pl->n_sid : 2 * pl->n_units * pl->HG;
+    pl->n_counters = (int)(2 * lb * kv.n_kv_heads);
     pl->N = N;
     pl->box_rows = box_rows;
     pl->boxes = kTile / box_rows;
@@ -304,12 +302,10 @@ __global__ void add_stats_kernel(float* stats, int64_t stat_stride, const float*
 
 }  // namespace
 
-// A team has at most 15 parts (cph / (cph >> 3)) and the parts of all teams are at most one per SM, so the counters
-// of a plan, 3 (units + kMaxClass) parts, stay below this whatever the split.
+// Two counters per problem whatever the split, and one for the CTAs that have finished.
 size_t verify_counter_bytes(const KvView& kv)
 {
-    const size_t probs = (size_t)kv.n_layers * kv.batch * kv.n_kv_heads;
-    return (3 * (16 * probs + (kMaxClass + 1) * (size_t)sm_count()) + 1) * sizeof(int);
+    return (2 * (size_t)kv.n_layers * kv.batch * kv.n_kv_heads + 1) * sizeof(int);
 }
 
 bool verify_sm100_supported(const KvView& kv, int n_q, int variant)
@@ -448,10 +444,9 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         fp.cls_subs[f] = pl.cls_subs[f];
         set_divisor(&fp.cls_mul[f], &fp.cls_sh[f], pl.cls_size[f]);
     }
-    fp.n_sid = pl.n_sid;
     fp.n_counters = pl.n_counters;
     set_divisor(&fp, 3, a.kv.n_q_heads / a.kv.n_kv_heads);
-    fp.n_units = pl.cached ? pl.n_units + kMaxClass : pl.n_units;
+    fp.n_units = pl.n_units;
     fp.N = pl.N;
     fp.R = a.n_q * G;
     fp.G = G;

@@ -127,9 +127,8 @@ constexpr int kSortMax = 64;  // sequences, two per lane of the warp that sorts 
 struct alignas(16) Work {
     uint16_t layer, b, h;
     uint16_t n, rank;  // CTAs of the problem (0: nothing to do in this unit), this one's number among them
-    uint16_t sid;      // the part's number: index of its counters
     uint16_t cta0;     // first CTA of the part
-    uint16_t pad;
+    uint16_t pad[2];
     int T, t0, t1, prob;
     __device__ bool valid() const { return n != 0; }
 };
@@ -186,9 +185,7 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     w.h = (uint16_t)h;
     w.n = (uint16_t)(valid ? n : 0);
     w.rank = (uint16_t)rank;
-    w.sid = (uint16_t)slot;
     w.cta0 = (uint16_t)(team * p.cph + sub * size);
-    w.pad = 0;
     w.prob = (layer * p.a.kv.batch + b) * p.a.kv.n_kv_heads + h;
     sc.work[unit % kWorkTab] = w;
 }
@@ -701,15 +698,15 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                 if (!ok) break;
             }
-            int* c_p1 = p.counters + unit * p.n_sid + sg.sid;
-            int* c_o = c_p1 + p.n_units * p.n_sid;
+            int* c_p1 = p.counters + sg.prob;
+            int* c_o = c_p1 + p.n_counters / 2;
             if (unit >= kRing - 1) {
                 // the partials' places are used again by the next unit: their readers must be done (they have been
                 // for two units, as a rule)
                 const Work old = get_work(sc, unit - (kRing - 1));
                 if (old.n > 1) {
                     if (lane == 0)
-                        ok = counter_wait(p.counters + (2 * p.n_units + unit - (kRing - 1)) * p.n_sid + old.sid, old.n, ctl, 36);
+                        ok = counter_wait(p.counters + old.prob, 2 * old.n, ctl, 36);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                     if (!ok) break;
                 }
@@ -796,7 +793,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             }
             const Work sg = get_work(sc, unit);
             if (sg.n <= 1) continue;  // (a problem of one CTA: the softmax warps store the output)
-            int* c_o = p.counters + (p.n_units + unit) * p.n_sid + sg.sid;
+            int* c_p1 = p.counters + sg.prob;
+            int* c_o = c_p1 + p.n_counters / 2;
             if (lane == 0) ok = counter_wait(c_o, sg.n, ctl, 30);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
@@ -868,7 +866,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             __syncwarp();
             if (lane == 0 && unit + kRing - 1 < U) {  // the partials have been read: their places may be used again
                 __threadfence();
-                atomicAdd(c_o + p.n_units * p.n_sid, 1);
+                atomicAdd(c_p1, 1);  // (every CTA of the problem has added its one before: c_o was complete)
             }
         }
     } else {
@@ -1272,7 +1270,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 ok = bar_wait(B.lse_ready, unit & 1, ctl);
                 if (!ok) break;
                 if (!LP && sg.n > 1) {  // many CTAs per head: too many partials for one warp, all softmax threads fold them
-                    if (lane == 0) ok = counter_wait(p.counters + unit * p.n_sid + sg.sid, sg.n, ctl, 33);
+                    if (lane == 0) ok = counter_wait(p.counters + sg.prob, sg.n, ctl, 33);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;  // lane 0's acquire, then warp-wide
                     if (!ok) break;
                     const float2* src = p.ml_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R;
