@@ -22,7 +22,7 @@ def taken(kv, n_q, ctx):
 
 def test_counters_leave_the_partials_their_room():
     # 56 rows on 144 CTAs: 3840 bytes are left for counters
-    assert taken(kv_struct(1, 1, 32, 8, 128, 4096), 14, 4096)
+    assert taken(kv_struct(1, 1, 32, 8, 128, 2048), 14, 2048)
     assert taken(kv_struct(1, 1, 64, 16, 128, 2048), 14, 2048)
 
 
