@@ -110,11 +110,21 @@ static KvView bf16_twin(const KvView& kv)
 
 // Workspace of a verification call over an 8-bit cache: [0, base) as for any call (base = the larger of the
 // generic kernels' and the tensor-core kernels' needs on the bf16 twin), then the twin's K and V.
-static size_t fp8_verify_base(const KvView& kv, int n_q, int max_ctx_len)
+static size_t fp8_verify_base(const KvView& kv, int n_q, int max_ctx_len, int max_ctas = 0)
 {
     const size_t g = verify_generic_workspace(kv, n_q, max_ctx_len);
-    const size_t f = verify_sm100_workspace(bf16_twin(kv), n_q, max_ctx_len);
+    const size_t f = verify_sm100_workspace(bf16_twin(kv), n_q, max_ctx_len, max_ctas);
     return ((g > f ? g : f) + 255) & ~(size_t)255;
+}
+
+static size_t verify_workspace(const KvView& kv, int n_q, int max_ctx_len, int max_ctas)
+{
+    // 8-bit cache: room for its bf16 copy behind the usual workspace (4 bytes per cache element of the view)
+    if (kv.fp8 && kv_expand_supported(kv))
+        return fp8_verify_base(kv, n_q, max_ctx_len, max_ctas) + 4 * (size_t)kv_expand_elems(kv);
+    const size_t g = verify_generic_workspace(kv, n_q, max_ctx_len);
+    const size_t f = verify_sm100_workspace(kv, n_q, max_ctx_len, max_ctas);
+    return g > f ? g : f;
 }
 
 static int sm100_variant(int impl)
@@ -122,33 +132,9 @@ static int sm100_variant(int impl)
     return impl == SPEC_VERIFY_TCGEN05_TWOSWEEP ? 1 : (impl == SPEC_VERIFY_TCGEN05_CACHED ? 2 : 0);
 }
 
-}  // namespace spec
-
-using namespace spec;
-
-extern "C" {
-
-int spec_verify_attn(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
-                     int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
-                     int64_t stat_stride, void* workspace, size_t workspace_bytes, void* cuda_stream)
-{
-    return spec_verify_attn_ex(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace,
-                               workspace_bytes, 0u, cuda_stream);
-}
-
-int spec_verify_attn_ex(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
-                        int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
-                        int64_t stat_stride, void* workspace, size_t workspace_bytes, uint32_t flags,
-                        void* cuda_stream)
-{
-    return spec_verify_attn_hist(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace,
-                                 workspace_bytes, flags, nullptr, cuda_stream);
-}
-
-int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
-                          int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
-                          int64_t stat_stride, void* workspace, size_t workspace_bytes, uint32_t flags,
-                          uint32_t* score_hist, void* cuda_stream)
+int verify_call(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len, int32_t max_ctx_len,
+                int32_t stat_window, float* out, float* lse, float* stats, int64_t stat_stride, void* workspace,
+                size_t workspace_bytes, uint32_t flags, uint32_t* score_hist, int max_ctas, void* cuda_stream)
 {
     if (flags & ~(uint32_t)(SPEC_VERIFY_ACCUMULATE_STATS | SPEC_VERIFY_STATS_PER_QUERY_HEAD | SPEC_VERIFY_OUT_BF16 |
                             SPEC_VERIFY_STATS_GROUP_MAX))
@@ -181,6 +167,7 @@ int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const
     a.stat_per_head = (flags & SPEC_VERIFY_STATS_PER_QUERY_HEAD) ? 1 : 0;
     a.stat_group_max = (flags & SPEC_VERIFY_STATS_GROUP_MAX) ? 1 : 0;
     a.out_bf16 = (flags & SPEC_VERIFY_OUT_BF16) ? 1 : 0;
+    a.max_ctas = max_ctas;
     a.hist = score_hist;  // the score-cache kernel counts in its statistic pass; the others get a sweep afterwards
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const long hist_probs = (long)kv->n_layers * kv->batch * (a.stat_per_head ? kv->n_q_heads : kv->n_kv_heads);
@@ -196,7 +183,7 @@ int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const
         verify_sm100_can_run(a, sm100_variant(impl))) {
         fast_ok = true;
     } else if (a.kv.fp8 && impl != SPEC_VERIFY_GENERIC && kv_expand_supported(a.kv)) {
-        const size_t base = fp8_verify_base(a.kv, n_q, max_ctx_len);
+        const size_t base = fp8_verify_base(a.kv, n_q, max_ctx_len, max_ctas);
         const size_t elems = (size_t)kv_expand_elems(a.kv);
         if (workspace_bytes >= base + 4 * elems) {
             __nv_bfloat16* k16 = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(workspace) + base);
@@ -236,6 +223,53 @@ int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const
     if (rc3 != SPEC_OK || !score_hist) return rc3;
     return score_hist_launch(stats, stat_stride, hist_probs, kv->batch, hist_heads, ctx_len, max_ctx_len, score_hist,
                              stream);
+}
+
+int verify_ctas_within(const spec_kv_t* kv, int32_t n_q, int32_t max_ctx_len, size_t bytes)
+{
+    KvView v;
+    if (make_view(kv, &v) != SPEC_OK || n_q < 1 || n_q > 32 || max_ctx_len < n_q) return SPEC_ERR_INVALID_ARG;
+    const bool expand = v.fp8 && kv_expand_supported(v);
+    const size_t g = verify_generic_workspace(v, n_q, max_ctx_len);
+    const size_t f = verify_sm100_even_workspace(expand ? bf16_twin(v) : v, n_q, max_ctx_len);
+    size_t need = g > f ? g : f;
+    if (expand) need = ((need + 255) & ~(size_t)255) + 4 * (size_t)kv_expand_elems(v);
+    if (need > bytes) return SPEC_ERR_WORKSPACE_TOO_SMALL;
+    int ctas = sm_count();
+    while (ctas > 1 && verify_workspace(v, n_q, max_ctx_len, ctas) > bytes) --ctas;
+    return ctas;
+}
+
+}  // namespace spec
+
+using namespace spec;
+
+extern "C" {
+
+int spec_verify_attn(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
+                     int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
+                     int64_t stat_stride, void* workspace, size_t workspace_bytes, void* cuda_stream)
+{
+    return spec_verify_attn_ex(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace,
+                               workspace_bytes, 0u, cuda_stream);
+}
+
+int spec_verify_attn_ex(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
+                        int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
+                        int64_t stat_stride, void* workspace, size_t workspace_bytes, uint32_t flags,
+                        void* cuda_stream)
+{
+    return spec_verify_attn_hist(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace,
+                                 workspace_bytes, flags, nullptr, cuda_stream);
+}
+
+int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const int32_t* ctx_len,
+                          int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
+                          int64_t stat_stride, void* workspace, size_t workspace_bytes, uint32_t flags,
+                          uint32_t* score_hist, void* cuda_stream)
+{
+    return verify_call(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, workspace, workspace_bytes,
+                       flags, score_hist, 0, cuda_stream);
 }
 
 int spec_select_recall(const float* stats, int64_t stat_stride, int32_t n_layers, int32_t batch,
@@ -320,12 +354,7 @@ size_t spec_workspace_bytes(int which, const spec_kv_t* kv, int32_t n_q, int32_t
     if (make_view(kv, &v) != SPEC_OK) return 0;
     if (which == SPEC_WS_VERIFY) {
         if (n_q < 1 || n_q > 32 || max_ctx_len < n_q) return 0;
-        // 8-bit cache: room for its bf16 copy behind the usual workspace (4 bytes per cache element of the view)
-        if (v.fp8 && kv_expand_supported(v))
-            return fp8_verify_base(v, n_q, max_ctx_len) + 4 * (size_t)kv_expand_elems(v);
-        size_t g = verify_generic_workspace(v, n_q, max_ctx_len);
-        size_t f = verify_sm100_workspace(v, n_q, max_ctx_len);
-        return g > f ? g : f;
+        return verify_workspace(v, n_q, max_ctx_len, 0);
     }
     if (which == SPEC_WS_DRAFT) {
         if (k_total < 1) return 0;

@@ -127,6 +127,7 @@ struct VerifyArgs {
     int stat_per_head;    // stats is [layers, batch, n_q_heads, stride]: one score per attention head
     int stat_group_max;   // stats is per KV head, but the group's per-head scores are folded by max instead of sum
     int out_bf16;         // `out` points to bf16 elements (round to nearest even) instead of fp32
+    int max_ctas;         // > 0: the tensor-core kernels use at most that many CTAs (the workspace holds no more partials)
     uint32_t* hist;       // not null: += counts of the final scores' top 11 bits, [problems][kScoreBins]
 };
 

@@ -50,9 +50,8 @@ int spec_verify_attn_noalloc(const spec_kv_t* kv, const void* q, int32_t n_q, co
                              int32_t max_ctx_len, int32_t stat_window, float* out, float* lse, float* stats,
                              int64_t stat_stride, void* cuda_stream)
 {
-    const size_t need = spec_workspace_bytes(SPEC_WS_VERIFY, kv, n_q, max_ctx_len, 1);
-    if (need == 0) return SPEC_ERR_INVALID_ARG;
-    if (need > kStaticScratchBytes) return SPEC_ERR_WORKSPACE_TOO_SMALL;  // shape too large for the built-in scratch
+    const int ctas = spec::verify_ctas_within(kv, n_q, max_ctx_len, kStaticScratchBytes);
+    if (ctas < 0) return ctas;
     void* scratch = nullptr;
     const int rc = scratch_address(&scratch);
     if (rc != SPEC_OK) return rc;
@@ -64,12 +63,12 @@ int spec_verify_attn_noalloc(const spec_kv_t* kv, const void* q, int32_t n_q, co
     shape.batch = kv->batch;
     shape.n_kv_heads = kv->n_kv_heads;
     size_t head = spec::verify_counter_bytes(shape);
-    if (spec::kStatusBytes + head > need) head = need > spec::kStatusBytes ? need - spec::kStatusBytes : 0;
-    if (head > 0 && cudaMemsetAsync(static_cast<char*>(scratch) + spec::kStatusBytes, 0, head,
-                                    static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
+    if (head > kStaticScratchBytes - spec::kStatusBytes) head = kStaticScratchBytes - spec::kStatusBytes;
+    if (cudaMemsetAsync(static_cast<char*>(scratch) + spec::kStatusBytes, 0, head,
+                        static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return SPEC_ERR_CUDA;
-    return spec_verify_attn(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, scratch,
-                            kStaticScratchBytes, cuda_stream);
+    return spec::verify_call(kv, q, n_q, ctx_len, max_ctx_len, stat_window, out, lse, stats, stat_stride, scratch,
+                             kStaticScratchBytes, 0u, nullptr, ctas, cuda_stream);
 }
 
 int spec_noalloc_read_status(void* cuda_stream)

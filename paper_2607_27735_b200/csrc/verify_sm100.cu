@@ -1,6 +1,7 @@
 // Host side of the sm_100a verification path: shape checks, the work plan (how KV heads are
 // grouped into units and split over the CTAs), TMA tensor maps, and the choice between the
 // score-cache kernel (K and V read once) and the two-sweep kernel (any context length).
+#include <climits>
 #include <cstdlib>
 
 #include "sm100_common.cuh"
@@ -34,7 +35,7 @@ struct Plan {
     int HG, cph, n_units, N, n_slots, p_bufs, box_rows, boxes, n_cache, n_raw;
     int n_cls, cls_size[kMaxClass], cls_subs[kMaxClass], n_counters;
     size_t smem_bytes;
-    size_t ctr_off, ctr_bytes, ml_off, o_off, total;
+    size_t ctr_off, ml_off, o_off, total;
 };
 
 int box_rows_for(int page_size)
@@ -44,8 +45,59 @@ int box_rows_for(int page_size)
     return 0;
 }
 
-// variant: 0 = prefer the score-cache kernel, 1 = two-sweep only, 2 = score-cache only
-bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl)
+// Score tiles the tensor-memory cache holds next to the output accumulator.
+int cache_tiles(int N)
+{
+    const int n = (kTmemCols - 2 * N) / N;
+    return n > 32 ? 32 : n;
+}
+
+// Heads of a sequence that are worked on at once when every one gets the same share of the SMs (a divisor of the KV heads;
+// 0: a head's share exceeds `tiles` key tiles however it is cut).  from_l2: K is swept a second time.
+int best_head_group(const KvView& kv, int max_ctx_len, int nsm, int tiles, bool from_l2)
+{
+    const int nb = (max_ctx_len + kTile - 1) / kTile;
+    int best_hg = 0;
+    double best = -1.0;
+    for (int hg = 1; hg <= kv.n_kv_heads; ++hg) {
+        if (kv.n_kv_heads % hg) continue;
+        const int cph = nsm / hg;
+        if (cph < 1) continue;
+        const int tpc = (nb + cph - 1) / cph;
+        if (tpc > tiles) continue;
+        double score = (double)nb * hg / ((double)nsm * tpc);  // fraction of CTA-tile slots doing work
+        if (from_l2) {
+            const double k_mib = (double)hg * max_ctx_len * 256.0 / (1 << 20);
+            if (k_mib > 40.0) score -= 0.3;  // the unit's K must stay L2-resident
+            if ((long)kv.n_layers * kv.batch * (kv.n_kv_heads / hg) < 2) score -= 0.1;  // a single unit cannot be pipelined
+        }
+        score += 0.001 * hg;  // ties: fewer partials per head
+        if (score > best) {
+            best = score;
+            best_hg = hg;
+        }
+    }
+    return best_hg;
+}
+
+// Workspace of a call whose partials come from `ctas` CTAs with R rows each.
+size_t workspace_layout(const KvView& kv, int R, int ctas, size_t* ctr_off, size_t* ml_off, size_t* o_off)
+{
+    size_t off = kStatusBytes;
+    *ctr_off = off;
+    off += verify_counter_bytes(kv);
+    off = (off + 255) & ~(size_t)255;
+    *ml_off = off;
+    off += (size_t)kRing * ctas * R * sizeof(float2);
+    off = (off + 255) & ~(size_t)255;
+    *o_off = off;
+    off += (size_t)kRing * ctas * R * kD * sizeof(float);
+    return (off + 255) & ~(size_t)255;
+}
+
+// variant: 0 = prefer the score-cache kernel, 1 = two-sweep only, 2 = score-cache only.  max_ctas > 0: on at most that
+// many CTAs (a caller whose workspace holds no more partials).
+bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl, int max_ctas = 0)
 {
     const int G = kv.n_q_heads / kv.n_kv_heads, R = n_q * G;
     pl->n_raw = 0;
@@ -55,12 +107,11 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     if (!(kv.head_dim == kD || (kv.head_dim == 64 && variant != 1)) || R > 128 || G > 256 || n_q > 256) return false;
     const int box_rows = box_rows_for(kv.page_size);
     if (box_rows == 0) return false;
-    const int nsm = sm_count();
+    const int nsm = max_ctas > 0 && max_ctas < sm_count() ? max_ctas : sm_count();
     const int N = (R + 15) / 16 * 16;
     const int nb = (max_ctx_len + kTile - 1) / kTile;
     const long lb = (long)kv.n_layers * kv.batch;
-    int n_cache = (kTmemCols - 2 * N) / N;
-    if (n_cache > 32) n_cache = 32;
+    const int n_cache = cache_tiles(N);
 
     int best_hg = 0;
     bool cached = false;
@@ -106,22 +157,7 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     }
     if (!cached) {
         if (variant == 2 || kv.head_dim != kD || kv.fp8) return false;
-        double best = -1.0;
-        for (int hg = 1; hg <= kv.n_kv_heads; ++hg) {
-            if (kv.n_kv_heads % hg) continue;
-            const int cph = nsm / hg;
-            if (cph < 1) continue;
-            const int tpc = (nb + cph - 1) / cph;
-            double score = (double)nb * hg / ((double)nsm * tpc);  // fraction of CTA-tile slots doing work
-            const double k_mib = (double)hg * max_ctx_len * 256.0 / (1 << 20);
-            if (k_mib > 40.0) score -= 0.3;                         // the unit's K must stay L2-resident
-            if (lb * (kv.n_kv_heads / hg) < 2) score -= 0.1;        // a single unit cannot be pipelined
-            score += 0.001 * hg;                                    // ties: fewer partials per head
-            if (score > best) {
-                best = score;
-                best_hg = hg;
-            }
-        }
+        best_hg = best_head_group(kv, max_ctx_len, nsm, INT_MAX, true);
         if (best_hg == 0) return false;
     }
     pl->cached = cached;
@@ -190,17 +226,7 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     if (slots < 3) return false;
     pl->n_slots = slots;
     pl->smem_bytes = fixed + (size_t)slots * kSlotBytes;
-    size_t off = kStatusBytes;
-    pl->ctr_off = off;
-    pl->ctr_bytes = verify_counter_bytes(kv);
-    off += pl->ctr_bytes;
-    off = (off + 255) & ~(size_t)255;
-    pl->ml_off = off;
-    off += (size_t)kRing * pl->HG * pl->cph * R * sizeof(float2);
-    off = (off + 255) & ~(size_t)255;
-    pl->o_off = off;
-    off += (size_t)kRing * pl->HG * pl->cph * R * kD * sizeof(float);
-    pl->total = (off + 255) & ~(size_t)255;
+    pl->total = workspace_layout(kv, R, pl->HG * pl->cph, &pl->ctr_off, &pl->ml_off, &pl->o_off);
     return true;
 }
 
@@ -267,15 +293,16 @@ struct SplitPlan {
     int64_t stat_stride;
 };
 
-bool make_split_plan(const KvView& kv, int n_q, int max_ctx_len, SplitPlan* sp)
+bool make_split_plan(const KvView& kv, int n_q, int max_ctx_len, SplitPlan* sp, int max_ctas = 0)
 {
     if (kv.n_layers * kv.batch != 1 || n_q < 2) return false;
     Plan full;
-    if (make_plan(kv, n_q, max_ctx_len, 2, &full)) return false;  // fits in one pass
+    if (make_plan(kv, n_q, max_ctx_len, 2, &full, max_ctas)) return false;  // fits in one pass
     sp->nA = (n_q + 1) / 2;
     sp->nB = n_q - sp->nA;
     Plan pa, pb;
-    if (!make_plan(kv, sp->nA, max_ctx_len, 2, &pa) || !make_plan(kv, sp->nB, max_ctx_len, 2, &pb)) return false;
+    if (!make_plan(kv, sp->nA, max_ctx_len, 2, &pa, max_ctas) || !make_plan(kv, sp->nB, max_ctx_len, 2, &pb, max_ctas))
+        return false;
     sp->main_bytes = pa.total > pb.total ? pa.total : pb.total;
     sp->ctx_off = sp->main_bytes;
     sp->stat_off = sp->ctx_off + 256;
@@ -328,16 +355,39 @@ void verify_sm100_describe(const KvView& kv, int n_q, int max_ctx_len, int32_t o
     for (int i = 0; i < 8; ++i) out[i] = v[i];
 }
 
-size_t verify_sm100_workspace(const KvView& kv, int n_q, int max_ctx_len)
+size_t verify_sm100_workspace(const KvView& kv, int n_q, int max_ctx_len, int max_ctas)
 {
     // the same bytes serve either variant: take the larger of the two plans
     size_t best = 0;
     for (int variant = 1; variant <= 2; ++variant) {
         Plan pl;
-        if (make_plan(kv, n_q, max_ctx_len, variant, &pl) && pl.total > best) best = pl.total;
+        if (make_plan(kv, n_q, max_ctx_len, variant, &pl, max_ctas) && pl.total > best) best = pl.total;
     }
     SplitPlan sp;
-    if (make_split_plan(kv, n_q, max_ctx_len, &sp) && sp.total > best) best = sp.total;
+    if (make_split_plan(kv, n_q, max_ctx_len, &sp, max_ctas) && sp.total > best) best = sp.total;
+    return best;
+}
+
+size_t verify_sm100_even_workspace(const KvView& kv, int n_q, int max_ctx_len)
+{
+    const int nsm = sm_count(), G = kv.n_q_heads / kv.n_kv_heads;
+    size_t best = 0, ctr, ml, o;
+    auto cached = [&](int rows) -> size_t {  // rows that the score cache can hold
+        const int R = rows * G;
+        const int hg = best_head_group(kv, max_ctx_len, nsm, cache_tiles((R + 15) / 16 * 16), false);
+        return hg ? workspace_layout(kv, R, hg * (nsm / hg), &ctr, &ml, &o) : 0;
+    };
+    Plan pl;
+    if (make_plan(kv, n_q, max_ctx_len, 1, &pl)) best = workspace_layout(kv, n_q * G, pl.HG * pl.cph, &ctr, &ml, &o);
+    if (make_plan(kv, n_q, max_ctx_len, 2, &pl)) {
+        const size_t b = cached(n_q);
+        return b > best ? b : best;
+    }
+    SplitPlan sp;
+    if (make_split_plan(kv, n_q, max_ctx_len, &sp)) {
+        const size_t b = cached(sp.nA) + (sp.total - sp.main_bytes);  // (nA >= nB)
+        if (b > best) best = b;
+    }
     return best;
 }
 
@@ -349,13 +399,13 @@ bool verify_sm100_can_run(const VerifyArgs& a, int variant)
     if (a.stat_per_head || a.stat_group_max) {
         const int G = a.kv.n_q_heads / a.kv.n_kv_heads;
         Plan pl;
-        if (variant == 1 || G > 8 || !make_plan(a.kv, a.n_q, a.max_ctx_len, 2, &pl)) return false;
+        if (variant == 1 || G > 8 || !make_plan(a.kv, a.n_q, a.max_ctx_len, 2, &pl, a.max_ctas)) return false;
         variant = 2;
     }
     SplitPlan sp;
-    if (variant == 0 && make_split_plan(a.kv, a.n_q, a.max_ctx_len, &sp)) return a.workspace_bytes >= sp.total;
+    if (variant == 0 && make_split_plan(a.kv, a.n_q, a.max_ctx_len, &sp, a.max_ctas)) return a.workspace_bytes >= sp.total;
     Plan pl;
-    if (!make_plan(a.kv, a.n_q, a.max_ctx_len, variant, &pl)) return false;
+    if (!make_plan(a.kv, a.n_q, a.max_ctx_len, variant, &pl, a.max_ctas)) return false;
     if ((a.kv.k_scale || a.kv.v_scale) && !pl.cached) return false;
     return a.workspace_bytes >= pl.total;
 }
@@ -369,12 +419,12 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         // everything else goes to the generic kernels
         const int G = a.kv.n_q_heads / a.kv.n_kv_heads;
         Plan pl;
-        if (variant == 1 || G > 8 || !make_plan(a.kv, a.n_q, a.max_ctx_len, 2, &pl))
+        if (variant == 1 || G > 8 || !make_plan(a.kv, a.n_q, a.max_ctx_len, 2, &pl, a.max_ctas))
             return SPEC_ERR_UNSUPPORTED_SHAPE;
         variant = 2;
     }
     SplitPlan sp;
-    if (variant == 0 && make_split_plan(a.kv, a.n_q, a.max_ctx_len, &sp)) {
+    if (variant == 0 && make_split_plan(a.kv, a.n_q, a.max_ctx_len, &sp, a.max_ctas)) {
         if (a.workspace_bytes < sp.total) return SPEC_ERR_WORKSPACE_TOO_SMALL;
         char* ws = static_cast<char*>(a.workspace);
         int32_t* ctx_a = reinterpret_cast<int32_t*>(ws + sp.ctx_off);
@@ -412,7 +462,7 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         return SPEC_OK;
     }
     Plan pl;
-    if (!make_plan(a.kv, a.n_q, a.max_ctx_len, variant, &pl)) return SPEC_ERR_UNSUPPORTED_SHAPE;
+    if (!make_plan(a.kv, a.n_q, a.max_ctx_len, variant, &pl, a.max_ctas)) return SPEC_ERR_UNSUPPORTED_SHAPE;
     // per-(layer, KV head) scales (an 8-bit cache expanded to bf16): only the score-cache kernel applies them
     if ((a.kv.k_scale || a.kv.v_scale) && !pl.cached) return SPEC_ERR_UNSUPPORTED_SHAPE;
     if (a.workspace_bytes < pl.total) return SPEC_ERR_WORKSPACE_TOO_SMALL;

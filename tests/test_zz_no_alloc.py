@@ -57,3 +57,20 @@ def test_noalloc_refuses_shapes_beyond_the_built_in_scratch():
         binding.spec_verify_attn_noalloc(case.kv, case.q_verify, case.ctx_len, 4096)
     assert e.value.code == -3
     assert binding.launch_count() == before
+
+
+def test_noalloc_runs_on_fewer_ctas_where_the_scratch_asks_for_it():
+    """56 rows: the scratch holds the partials of 144 CTAs, this batch's own split would use 147."""
+    lens = [896, 300, 57, 640, 777]
+    cfg = inputs.small_config(ctx=(57, 896), n_q=14, batch=5, n_q_heads=64, n_kv_heads=16, planted=0, q_mode="iid", q_std=0.09)
+    case = inputs.make_case(cfg, device="cuda", ctx_override=lens)
+    T = 896
+    plan = binding.describe_plan(binding.WS_VERIFY, binding._kv_struct(case.kv), 14, T)
+    assert 4 * plan[1] * plan[2] * 56 * (512 + 8) > binding.noalloc_scratch_bytes()
+    o_out, o_lse, o_stats = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, 896)
+    out, lse, stats = binding.spec_verify_attn_noalloc(case.kv, case.q_verify, case.ctx_len, T)
+    assert binding.noalloc_read_status() == 0
+    assert (out.cpu().double() - o_out).abs().max().item() <= TOL
+    assert (lse.cpu().double() - o_lse).abs().max().item() <= TOL
+    for b, t in enumerate(case.ctx_len.tolist()):
+        assert (stats[:, b, :, :t].cpu().double() - o_stats[:, b, :, :t]).abs().max().item() <= TOL
