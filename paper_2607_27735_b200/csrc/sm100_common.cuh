@@ -35,6 +35,7 @@ struct FastParams {
     int cls_subs[kMaxClass];          // parts of a team
     uint32_t cls_mul[kMaxClass];      // division by cls_size (see div_by)
     int32_t cls_sh[kMaxClass];
+    int one_round;                    // a single sequence, no more heads (over all layers) than teams
     int n_counters;                   // ints to zero at the end, the "CTAs finished" word being the one after them
     int* counters;                    // [2][problems]: P1 partials done (two-sweep: by unit and head; score cache: by
                                       // problem, and above the CTAs of the problem, reductions done), O partials

@@ -494,6 +494,7 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         fp.cls_subs[f] = pl.cls_subs[f];
         set_divisor(&fp.cls_mul[f], &fp.cls_sh[f], pl.cls_size[f]);
     }
+    fp.one_round = pl.cached && a.kv.batch == 1 && a.kv.n_layers * a.kv.n_kv_heads <= pl.HG;
     fp.n_counters = pl.n_counters;
     set_divisor(&fp, 3, a.kv.n_q_heads / a.kv.n_kv_heads);
     fp.n_units = pl.n_units;

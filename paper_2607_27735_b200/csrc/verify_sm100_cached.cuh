@@ -257,6 +257,35 @@ __device__ __noinline__ void make_schedule(const FastParams& p, Sched& sc)
     if (lane < u) put_work(p, sc, lane);
 }
 
+// The schedule of a single sequence whose heads are one round of whole teams (a call per layer of a long context): a unit
+// that follows from the length.  The general form takes 5 k cycles from the start of a CTA, most of them first
+// instruction fetches, and such a call has nothing to hide them behind: 2 rows over 2 K 14.9 us per launch with it.
+__device__ __forceinline__ void one_unit(const FastParams& p, Sched& sc)
+{
+    int raw;
+    Work w;
+    w.T = read_len(p, 0, &raw);
+    const int team = fast_div(p, 2, blockIdx.x), rank = blockIdx.x - team * p.cph;
+    const int layer = fast_div(p, 1, team), h = team - layer * p.a.kv.n_kv_heads;
+    const int nb = (w.T + kTile - 1) / kTile, n = min(p.cph, nb);
+    const bool valid = rank < n;
+    w.t0 = !valid ? 0 : (n < p.cph ? rank : fast_div(p, 2, rank * nb));
+    w.t1 = !valid ? 0 : (n < p.cph ? rank + 1 : fast_div(p, 2, (rank + 1) * nb));
+    w.layer = (uint16_t)layer;
+    w.b = 0;
+    w.h = (uint16_t)h;
+    w.n = (uint16_t)(valid ? n : 0);
+    w.rank = (uint16_t)rank;
+    w.cta0 = (uint16_t)(team * p.cph);
+    w.prob = team;
+    if ((threadIdx.x & 31) == 0) {
+        if (raw != w.T) set_status(p.status, SPEC_ERR_BAD_INDEX);
+        sc.work[0] = w;
+        sc.n_units = 1;
+        sc.limit = 1;
+    }
+}
+
 __device__ __forceinline__ Work get_work(const Sched& sc, int unit) { return sc.work[unit % kWorkTab]; }
 // Waits until a word of the schedule is above `x` (bounded like every wait).
 __device__ __noinline__ bool wait_above(const volatile int& word, int x, const Ctl& c)
@@ -432,7 +461,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // The schedule is made from the lengths as they are now, before the launch's dependency is resolved (the kernel
     // before may still be writing them: they are read again and compared after the wait below): its latencies and
     // first instruction fetches then hide behind the previous launch's end.
-    if (warp == 0) make_schedule(p, sc);
+    if (warp == 0 && !p.one_round) make_schedule(p, sc);
     if (warp == 3 && lane < 3)
         asm volatile("prefetch.tensormap [%0];" ::"l"(lane == 0 ? &tm_k : (lane == 1 ? &tm_v : &tm_q)) : "memory");
     if (warp == 1) {
@@ -448,7 +477,9 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
-    if (warp == 0) {
+    if (warp == 0 && p.one_round) {
+        one_unit(p, sc);
+    } else if (warp == 0) {
         // the schedule stands if the lengths are what they were when it was made; lengths out of range are reported
         const bool sorted = p.a.kv.batch <= kSortMax;
         bool same = sorted;
