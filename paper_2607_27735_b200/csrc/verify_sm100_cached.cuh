@@ -125,12 +125,11 @@ constexpr int kSortMax = 64;  // sequences, two per lane of the warp that sorts 
 //    publisher: they do not pass `limit`, and say in `at` which unit they read next; the publisher waits for the
 //    slowest of them before it overwrites an entry.  (None of them can need the publisher for a unit that far back.)
 struct alignas(16) Work {
-    uint16_t layer, b, h;
+    int layer, b, h;
     uint16_t n, rank;  // CTAs of the problem (0: nothing to do in this unit), this one's number among them
-    uint16_t cta0;     // first CTA of the part
-    uint16_t pad[2];
     int T, t0, t1, prob;
     __device__ bool valid() const { return n != 0; }
+    __device__ int cta0() const { return blockIdx.x - rank; }  // first CTA of the part
 };
 static_assert(sizeof(Work) == 32, "two vector loads");
 constexpr int kWorkTab = 32;    // units in the table
@@ -180,12 +179,11 @@ __device__ __noinline__ void put_work(const FastParams& p, Sched& sc, int unit)
     // shares of nb / n tiles; n < size means a tile each
     w.t0 = !valid ? 0 : (n < size ? rank : div_by(p.cls_mul[f], p.cls_sh[f], rank * nb));
     w.t1 = !valid ? 0 : (n < size ? rank + 1 : div_by(p.cls_mul[f], p.cls_sh[f], (rank + 1) * nb));
-    w.layer = (uint16_t)layer;
-    w.b = (uint16_t)b;
-    w.h = (uint16_t)h;
+    w.layer = layer;
+    w.b = b;
+    w.h = h;
     w.n = (uint16_t)(valid ? n : 0);
     w.rank = (uint16_t)rank;
-    w.cta0 = (uint16_t)(team * p.cph + sub * size);
     w.prob = (layer * p.a.kv.batch + b) * p.a.kv.n_kv_heads + h;
     sc.work[unit % kWorkTab] = w;
 }
@@ -271,12 +269,11 @@ __device__ __forceinline__ void one_unit(const FastParams& p, Sched& sc)
     const bool valid = rank < n;
     w.t0 = !valid ? 0 : (n < p.cph ? rank : fast_div(p, 2, rank * nb));
     w.t1 = !valid ? 0 : (n < p.cph ? rank + 1 : fast_div(p, 2, (rank + 1) * nb));
-    w.layer = (uint16_t)layer;
+    w.layer = layer;
     w.b = 0;
-    w.h = (uint16_t)h;
+    w.h = h;
     w.n = (uint16_t)(valid ? n : 0);
     w.rank = (uint16_t)rank;
-    w.cta0 = (uint16_t)(team * p.cph);
     w.prob = team;
     if ((threadIdx.x & 31) == 0) {
         if (raw != w.T) set_status(p.status, SPEC_ERR_BAD_INDEX);
@@ -756,7 +753,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 if (lane == 0) ok = counter_wait(c_p1, sg.n, ctl, 31);
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;  // lane 0's acquire, then warp-wide
                 if (!ok) break;
-                const float2* src = p.ml_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R;
+                const float2* src = p.ml_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0()) * R;
                 // two lanes per row, 16 rows per pass: each lane folds every other partial, 20 loads in flight
                 const int sub = lane & 1;
                 for (int r0 = 0; r0 < R; r0 += 16) {
@@ -832,7 +829,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const int E4 = R * kD / 4;
             const int lo = sg.rank * E4 / sg.n, hi = (sg.rank + 1) * E4 / sg.n;
             const float4* src = reinterpret_cast<const float4*>(
-                p.o_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R * kD);
+                p.o_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0()) * R * kD);
             const int64_t out0 = ((int64_t)sg.layer * p.a.kv.batch + sg.b) * p.a.n_q * p.a.kv.n_q_heads * p.D + sg.h * G * p.D;
             auto store = [&](int e, const float4& v) {
                 const int d = 4 * (e & (kD / 4 - 1));
@@ -1304,7 +1301,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     if (lane == 0) ok = counter_wait(p.counters + sg.prob, sg.n, ctl, 33);
                     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;  // lane 0's acquire, then warp-wide
                     if (!ok) break;
-                    const float2* src = p.ml_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0) * R;
+                    const float2* src = p.ml_part + ((int64_t)(unit % kRing) * gridDim.x + sg.cta0()) * R;
                     // tpr threads of one warp share a row: each folds every tpr-th partial, then shuffles
                     int tpr = 32;
                     while (tpr * R > 128 * CG) tpr >>= 1;

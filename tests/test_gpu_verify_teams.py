@@ -115,3 +115,25 @@ def test_two_rounds_on_fresh_tensors():
             want = out, lse, stats
             check(case, T)
         assert all(torch.equal(a, b) for a, b in zip((out, lse, stats), want))
+
+
+def test_more_sequences_than_sixteen_bits_count():
+    """65600 sequences of at most 16 tokens, one head: the last 64 are not their namesakes 65536 below."""
+    B, n_q, D = 65600, 2, 64
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").bfloat16()
+    kv = inputs.KVCache(k=rand(1, B, 1, 16, D), v=rand(1, B, 1, 16, D), layer_stride=B * 16 * D, page_stride=16 * D,
+                        head_stride=16 * D, slot_stride=D, n_layers=1, page_size=16, page_table=None, max_pages=1, batch=B,
+                        n_q_heads=1, n_kv_heads=1, head_dim=D)
+    q = rand(1, B, n_q, 1, D)
+    lens = torch.randint(n_q, 17, (B,), generator=g, device="cuda", dtype=torch.int32)
+    out, lse, stats, ws = binding.spec_verify_attn(kv, q, lens, 16)
+    assert binding.read_status(ws) == 0 and binding.last_verify_impl() == binding.VERIFY_TCGEN05_CACHED
+    s = torch.einsum("bqd,bkd->bqk", q[0, :, :, 0].double(), kv.k[0, :, 0].double()) / D ** 0.5
+    last = lens[:, None].long() - n_q + torch.arange(n_q, device="cuda")
+    s = s.masked_fill(torch.arange(16, device="cuda") > last[..., None], -float("inf"))
+    p = s.softmax(-1)
+    assert (out[0, :, :, 0].double() - p @ kv.v[0, :, 0].double()).abs().max().item() <= TOL
+    assert (lse[0, :, :, 0].double() - s.logsumexp(-1)).abs().max().item() <= TOL
+    seen = torch.arange(16, device="cuda") < lens[:, None]
+    assert ((stats[0, :, 0, :16].double() - p.sum(1)) * seen).abs().max().item() <= TOL
