@@ -226,7 +226,8 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     if (slots < 3) return false;
     pl->n_slots = slots;
     pl->smem_bytes = fixed + (size_t)slots * kSlotBytes;
-    pl->total = workspace_layout(kv, R, pl->HG * pl->cph, &pl->ctr_off, &pl->ml_off, &pl->o_off);
+    // room for every CTA, whatever the split: what a split for a long context leaves out one for a shorter may use
+    pl->total = workspace_layout(kv, R, nsm, &pl->ctr_off, &pl->ml_off, &pl->o_off);
     return true;
 }
 
@@ -357,11 +358,11 @@ void verify_sm100_describe(const KvView& kv, int n_q, int max_ctx_len, int32_t o
 
 size_t verify_sm100_workspace(const KvView& kv, int n_q, int max_ctx_len, int max_ctas)
 {
-    // the same bytes serve either variant: take the larger of the two plans
+    // the same bytes serve either variant and every shorter context, with or without the rows in two passes
     size_t best = 0;
-    for (int variant = 1; variant <= 2; ++variant) {
+    for (int ctx : {max_ctx_len, max_ctas > 0 ? max_ctx_len : kTile}) {
         Plan pl;
-        if (make_plan(kv, n_q, max_ctx_len, variant, &pl, max_ctas) && pl.total > best) best = pl.total;
+        if (make_plan(kv, n_q, ctx, 0, &pl, max_ctas) && pl.total > best) best = pl.total;
     }
     SplitPlan sp;
     if (make_split_plan(kv, n_q, max_ctx_len, &sp, max_ctas) && sp.total > best) best = sp.total;

@@ -3,6 +3,8 @@ is pure host arithmetic on the cache description and the SM count (148 assumed w
 its invariants are checked here: every CTA fits one wave, a CTA's share of a head fits the
 tensor-memory cache, shares cover the key list, and the shapes the score-cache kernel cannot take
 fall back as documented."""
+import ctypes
+
 import pytest
 
 from paper_2607_27735_b200 import binding
@@ -102,3 +104,14 @@ def test_describe_plan_rejects_bad_arguments():
         binding.describe_plan(binding.WS_VERIFY, kv, 0, 4096)
     with pytest.raises(binding.SpecError):
         binding.describe_plan(binding.WS_SELECT, kv, 1, 4096)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("layers,batch,hq,hkv,n_q", [(1, 1, 8, 2, 5), (1, 1, 32, 8, 17), (1, 4, 32, 8, 9), (4, 3, 16, 2, 2), (1, 1, 64, 8, 16)])
+def test_a_workspace_for_a_long_context_serves_every_shorter_one(d, layers, batch, hq, hkv, n_q):
+    lib, need = binding.load(), []
+    lens = [128, 200, 512, 1000, 2048, 4096, 9000, 10240, 20000, 32768, 65536, 131072, 300000]
+    for ctx in lens:
+        kv = kv_struct(layers, batch, hq, hkv, d, (lens[-1] + 127) // 128 * 128)
+        need.append(lib.spec_workspace_bytes(binding.WS_VERIFY, ctypes.byref(kv), n_q, ctx, 1))
+    assert need == sorted(need)
