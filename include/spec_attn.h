@@ -185,9 +185,8 @@ int spec_verify_attn_ex(const spec_kv_t* kv, const void* q, int32_t n_q, const i
                         uint32_t flags, void* cuda_stream);
 
 /*
- * spec_verify_attn_ex that also hands the selection its first radix pass (Eq. 4 picks the largest
- * scores; the selection kernel finds the K-th largest by a radix select on the scores' fp32 bit
- * patterns, whose first pass is a histogram of the top 11 bits).  score_hist: uint32
+ * spec_verify_attn_ex that also counts the scores by the top 11 bits of their fp32 patterns, the
+ * first pass of a radix select (Eq. 4 picks the largest scores).  score_hist: uint32
  * [n_layers, batch, heads, 2048] (heads = n_kv_heads, or n_q_heads with
  * SPEC_VERIFY_STATS_PER_QUERY_HEAD), ZERO-FILLED once after allocation; this call ADDS, for every
  * score stats[.., i] it writes (i < ctx_len[b]), one count to bin (bit pattern >> 21) of the
@@ -208,7 +207,8 @@ int spec_verify_attn_hist(const spec_kv_t* kv, const void* q, int32_t n_q, const
  *                   [k_sink, T'-k_recent) with the largest stats (equal stats: the lower
  *                   position wins) U recent [T'-k_recent, T'); n = k_total.
  * Output ascending, padded with -1.  stats must be finite and >= 0 (they are sums of
- * probabilities), which makes the fp32 bit pattern order-isomorphic to the value; the result
+ * probabilities), which makes the fp32 bit pattern order-isomorphic to the value (any other
+ * pattern is ordered as the unsigned number it is); the result
  * is a pure function of the stats bits, so it is reproducible bit for bit.
  *
  *   stats     fp32 [n_layers, batch, n_kv_heads, stat_stride]
@@ -223,13 +223,12 @@ int spec_select_recall(const float* stats, int64_t stat_stride, int32_t n_layers
                        void* workspace, size_t workspace_bytes, void* cuda_stream);
 
 /*
- * spec_select_recall fed with the counts of spec_verify_attn_hist.  score_hist: uint32
+ * spec_select_recall that takes back the counts of spec_verify_attn_hist.  score_hist: uint32
  * [n_layers, batch, n_kv_heads, 2048] as that call left it; hist_len: int32 [batch], the ctx_len of
- * that call (the counts cover positions [0, hist_len[b]) of stats).  The kernel removes the
- * positions outside the candidate span from the counts, skips its own first sweep over the
- * scores, and writes zeros back to score_hist.  The result is the same, bit for bit, as
- * spec_select_recall on the same stats.  A sequence with sel_len[b] > hist_len[b] falls back to
- * the full sweep.  score_hist and hist_len are both NULL (= spec_select_recall) or both given.
+ * that call.  The kernel writes zeros back to score_hist.  It does not use the counts: its own
+ * sample of the scores costs less than loading them.  The result is the same, bit for bit, as
+ * spec_select_recall on the same stats.  score_hist and hist_len are both NULL
+ * (= spec_select_recall) or both given.
  */
 int spec_select_recall_hist(const float* stats, int64_t stat_stride, int32_t n_layers, int32_t batch,
                             int32_t n_kv_heads, const int32_t* sel_len, int32_t k_sink,

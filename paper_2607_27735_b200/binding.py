@@ -187,7 +187,7 @@ def spec_verify_attn(kv, q, ctx_len, max_ctx_len, stat_window=16, out=None, lse=
                      out_bf16=False, score_hist=None, group_max=False):
     """Verification attention + Eq. 3 statistic; returns ``(out, lse, stats, workspace)``.
     ``score_hist`` (uint32-as-int32 ``[L, B, heads, 2048]``, zero before the first use) receives the
-    selection's first radix pass (spec_verify_attn_hist).
+    counts of the scores' top 11 bits (spec_verify_attn_hist).
     ``accumulate`` adds this call's statistic to the given ``stats``; ``per_head`` keeps one score per
     attention head (``stats`` is ``[L, B, n_q_heads, stride]``); both go through spec_verify_attn_ex."""
     if stat_stride is None:

@@ -8,18 +8,20 @@
 // percent: score and position) in shared memory; the threshold is found on that list by a histogram of
 // (bits - floor) scaled to the list's own range, refined until its bin is small, whose entries are ranked
 // pair by pair (larger score, then lower position).  Chosen positions become bits of a position bitmap, which is
-// read off in order.  A span that fits the list needs no sample (every score is a list entry).  Where this
-// fails (a sample that misleads, hundreds of equal scores at the threshold, a budget above the list, contexts
-// above the bitmap's 128 K) one sweep per radix digit and an ordered compaction do it.
+// read off in order, window by window where the context exceeds the bitmap's 128 K.  A span that fits the list needs no
+// sample (every score is a list entry); hundreds of equal scores at the threshold, or a threshold of zero, are ranked in
+// the bitmap.  Where this fails (a sample that misleads, a budget above the list) one sweep per radix digit and an
+// ordered compaction do it.
 //
 // What bounds it: HBM at many long problems, else the chain of memory latencies, block barriers and first
 // instruction fetches (about 8 us; code that runs once stays rolled and shared).  256 problems (32 layers x
 // 8 heads) of 131 K scores: 105 -> 47 us; of 32 K: 35 -> 20 us.  The two sweeps of
 // histogram and collection that this replaced waited for every load and read the scores twice.
 //
-// The first radix digit's histogram (top 11 bits) may arrive from the verification kernel, which counts
-// every score it writes: the positions outside the candidate span are taken out again here, the bin of the
-// K_mid-th largest is the floor, no sample is taken, and the counts are cleared for the next round.
+// Counts of the scores' top 11 bits may arrive from the verification kernel, which counts every score it writes.  They
+// are cleared for the next round and not used: as a floor a bin of theirs (an eighth of an octave) is coarser than the
+// sample's, and loading it, taking the positions outside the span out again and the longer list cost more than the
+// sample saves (us with / without, the clearing included: 8 problems of 6 K 9.6 / 8.5, 256 of 6 K 18.5 / 12.1, 256 of 131 K 45.8 / 43.3).
 #include <atomic>
 
 #include "spec_common.cuh"
@@ -36,11 +38,12 @@ constexpr int kItems = 16;         // consecutive candidates per thread in the c
 constexpr int kListWords = 20480;  // list: 10240 entries (score, position), or 20480 scores in order: 80 KB
 constexpr int kDense = 4096;       // spans up to here are list entries as they are (eight per thread)
 constexpr int kPair = 512;         // entries ranked pair by pair (they reuse the histogram's storage)
-static_assert(2 * kPair <= kBins, "score and position of each");
+static_assert(3 * kPair <= kBins, "score, position and choice of each");
 constexpr int kSample = 4096;      // eight per thread: a relative error of the floor's rank of 8 % at 3 % kept
 constexpr int kV = 4;              // vectors per thread and trip of the sweep; the next trip's are in flight meanwhile
 constexpr int kTrip = kV * kThreads;           // vectors per trip
-constexpr int kMapWords = 4096;                // position bitmap: contexts up to 128 K keys
+constexpr int kMapWords = 4096;                // position bitmap: 128 K keys at a time
+constexpr int kWindow = 32 * kMapWords;
 // Bins of the sample's histogram: an exponent and five bits, 32 to the octave, for the 64 octaves below 2^16 (a
 // score is a sum of at most some hundred probabilities); smaller scores share the last one.
 constexpr int kSampleShift = 18;
@@ -160,6 +163,144 @@ __device__ __forceinline__ void sweep(const uint32_t* __restrict__ st, int lo, i
     }
 }
 
+// Entries [i0, i1) of the list, for the functions that stand outside the kernel: position(i) of entry i.
+struct List {
+    const uint32_t* u;
+    const int* pos;  // null: a dense list, where entry i is position i + shift
+    int i0, i1, shift;
+    __device__ int position(int i) const { return pos ? pos[i] : i + shift; }
+};
+
+// Floor of a span longer than a window, to 16 bits below the octave, from a sample that grows with it (4096 of every 256 K
+// scores), so that the rank wanted lies 4 sigma above the expected one and 5 below the list's end at every length
+// (a budget of 4096 over 1 M scores: 1015 us for 8 problems when one in four lists overflowed, 144 so).  0: the list
+// cannot hold enough.
+__device__ __noinline__ uint32_t floor_of_long_span(Shared& sh, const uint4* vec, int nv, int span, int k_mid, int cap)
+{
+    const int rounds = (span >> 18) + 1;
+    const float expect = (float)k_mid * rounds * kSample / span, room = (float)cap * rounds * kSample / span;
+    const int want = (int)min(expect + 6.f * sqrtf(expect) + 8.f, room - 5.f * sqrtf(room));
+    if ((float)want < expect + 4.f * sqrtf(expect)) return 0u;
+    auto each_sample = [&](auto f) {
+#pragma unroll 1
+        for (int r = 0; r < 2 * rounds; ++r) {
+            const int64_t k = (threadIdx.x >> 2) + r * (kThreads / 4);
+            const uint4 v = load_vec(vec + (int)(k * (nv - 4) / (rounds * (kSample / 16) - 1)) + (threadIdx.x & 3));
+            f(v.x);
+            f(v.y);
+            f(v.z);
+            f(v.w);
+        }
+    };
+    __syncthreads();
+    each_sample([&](uint32_t u) { atomicAdd(&sh.hist[sample_bin(u)], 1); });
+    __syncthreads();
+    if (!find_bucket(sh, want)) return 0u;
+    if (sh.bucket == 0) return 1u;  // every score but the zeros, if the list holds them
+    const int bin = sh.bucket, rest = want - sh.above;
+    each_sample([&](uint32_t u) {
+        if (sample_bin(u) == bin) atomicAdd(&sh.hist[(u >> (kSampleShift - 11)) & 2047u], 1);
+    });
+    __syncthreads();
+    find_bucket(sh, rest);
+    return kSampleBase + ((uint32_t)bin << kSampleShift) + ((uint32_t)sh.bucket << (kSampleShift - 11));
+}
+
+// The lowest n bits of m.
+__device__ __forceinline__ uint32_t lowest(uint32_t m, int n)
+{
+    for (int drop = n > 0 ? __popc(m) - n : 0; drop > 0; --drop) m &= ~(0x80000000u >> __clz((int)m));
+    return n > 0 ? m : 0u;
+}
+
+// The index set of a context above one window, with many equal scores at the threshold, or with a threshold of zero:
+// entries above [bin_lo, bin_lo + last], and the best `need` inside (last = 0: the first `need`, whose number does not
+// matter; bin_lo = 0 as well: the list holds every score but the zeros, and the first `need` positions of [lo, hi) that
+// it lacks are added).  The bitmap is clear and the histogram free.
+__device__ __noinline__ void write_windows(Shared& sh, const List l, uint32_t bin_lo, uint32_t last, int need, int lo, int hi,
+                                           int* out)
+{
+    const int tid = threadIdx.x;
+    const bool zeros = bin_lo == 0u && last == 0u && l.pos, equal = last == 0u && !zeros;
+    constexpr int kWpt = kMapWords / kThreads;  // bitmap words per thread, consecutive ones
+    uint32_t* bits = sh.bitmap + kWpt * tid;
+    auto count = [&]() {
+        int cnt = 0;
+        for (int k = 0; k < kWpt; ++k) cnt += __popc(bits[k]);
+        return cnt;
+    };
+    uint32_t* pu = reinterpret_cast<uint32_t*>(sh.hist);
+    int *pp = sh.hist + kPair, *pc = sh.hist + 2 * kPair;  // inside the bin: score, position; chosen: position, or -1
+    for (int i = l.i0 + tid; i < l.i1; i += kThreads) {
+        const uint32_t u = l.u[i];
+        if (last && u >= bin_lo && u - bin_lo <= last) {
+            const int at = atomicAdd(&sh.pair_n, 1);
+            pu[at] = u;
+            pp[at] = l.position(i);
+        }
+    }
+    __syncthreads();
+    const int np = sh.pair_n;
+    for (int e = tid; e < np; e += kThreads) {
+        int rank = 0;
+        for (int j = 0; j < np; ++j) rank += (pu[j] > pu[e]) | ((pu[j] == pu[e]) & (pp[j] < pp[e]));
+        pc[e] = rank < need ? pp[e] : -1;
+    }
+#pragma unroll 1
+    for (int w0 = 0; w0 < hi; w0 += kWindow) {
+        auto mark = [&](int pos) {
+            const uint32_t d = (uint32_t)(pos - w0);
+            if (pos >= 0 && d < (uint32_t)kWindow) atomicOr(&sh.bitmap[d >> 5], 1u << (d & 31));
+        };
+        __syncthreads();
+        if (equal) {  // the first `need` of them, in the order of positions
+            for (int i = l.i0 + tid; i < l.i1; i += kThreads)
+                if (l.u[i] == bin_lo) mark(l.position(i));
+            __syncthreads();
+            int keep = need - block_exclusive_scan(sh, count());
+            for (int k = 0; k < kWpt; ++k) {
+                const int n = __popc(bits[k]);
+                bits[k] = lowest(bits[k], keep);
+                keep -= n;
+            }
+            __syncthreads();
+            need -= min(need, sh.total);
+        }
+        for (int i = l.i0 + tid; i < l.i1; i += kThreads)
+            if (l.u[i] >= bin_lo && l.u[i] - bin_lo > last) mark(l.position(i));
+        for (int e = tid; e < np; e += kThreads) mark(pc[e]);
+        __syncthreads();
+        if (zeros) {
+            auto absent = [&](int k) {  // positions of [lo, hi) without a bit in a word
+                const int pos0 = w0 + 32 * (kWpt * tid + k);
+                uint32_t m = ~bits[k];
+                if (pos0 < lo) m &= lo - pos0 < 32 ? 0xffffffffu << (lo - pos0) : 0u;
+                if (hi - pos0 < 32) m &= hi > pos0 ? (1u << (hi - pos0)) - 1u : 0u;
+                return m;
+            };
+            int n = 0;
+            for (int k = 0; k < kWpt; ++k) n += __popc(absent(k));
+            int keep = need - block_exclusive_scan(sh, n);
+            for (int k = 0; k < kWpt; ++k) {
+                const uint32_t m = absent(k);
+                bits[k] |= lowest(m, keep);
+                keep -= __popc(m);
+            }
+            __syncthreads();
+            need -= min(need, sh.total);
+        }
+        int at = block_exclusive_scan(sh, count());
+        for (int k = 0; k < kWpt; ++k) {
+            const int pos0 = w0 + 32 * (kWpt * tid + k) - 1;
+            for (uint32_t m = bits[k]; m; m &= m - 1) out[at++] = pos0 + __ffs((int)m);
+            bits[k] = 0u;
+        }
+        __syncthreads();
+        out += sh.total;
+        if (hi - w0 <= kWindow) break;  // (w0 + kWindow may pass 2^31)
+    }
+}
+
 // Slow path: one sweep per radix digit, then an ordered compaction.  The histogram is clear.
 __device__ __noinline__ void select_by_sweeps(Shared& sh, const uint32_t* __restrict__ st, int lo, int hi, int k_mid,
                                               int32_t* __restrict__ out)
@@ -217,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int batch, int n_kv_heads,
                      const int32_t* __restrict__ sel_len, int k_sink, int k_recent, int k_total, int list_words,
                      int32_t* __restrict__ indices, int32_t* __restrict__ n_indices,
-                     uint32_t* __restrict__ hist_g, const int32_t* __restrict__ hist_len)
+                     uint32_t* __restrict__ hist_g)
 {
     __shared__ __align__(16) Shared sh;
     extern __shared__ __align__(16) uint32_t dyn_smem[];
@@ -246,16 +387,10 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     const int span = hi - lo;
     // Short spans, and spans of which a large part is kept, are list entries as they are.
     const bool dense = span + 3 <= list_words && (span <= kDense || k_mid > span / 4);
-    bool fast = hi <= kMapWords * 32;
-    // Counts handed over by the verification kernel are cleared whatever happens below.  They cover positions
-    // [0, hist_len): usable if the candidate span lies inside.  Only the search for the floor takes them; every other
-    // form counts for itself and starts from zero.
-    uint32_t* hg = hist_g ? hist_g + prob * kBins : nullptr;
-    const int HL = hg ? __ldcg(hist_len + b) : 0;
-    const bool have_hist = hg && T <= HL && T > k_total && fast && !dense;
+    bool fast = true;
     for (int i = tid; i < kBins; i += kThreads) {
-        sh.hist[i] = have_hist ? (int)hg[i] : 0;
-        if (hg) hg[i] = 0u;
+        sh.hist[i] = 0;
+        if (hist_g) hist_g[prob * kBins + i] = 0u;
     }
 
     if (T <= k_total) {  // everything fits: keep every position
@@ -282,53 +417,39 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
 
     // ---- the floor ----
     uint32_t floor_bits = 0;
-    if (fast && !dense) {
-        int want = k_mid;
-        uint32_t u[8];
-        if (have_hist) {
-            __syncthreads();
-            for (int i = tid; i < lo + (HL - hi); i += kThreads) {  // positions outside the span that were counted
-                const int pos = i < lo ? i : hi + (i - lo);
-                atomicSub(&sh.hist[__ldcg(st + pos) >> 21], 1);
-            }
-        } else {
-            // 256 blocks of four vectors (64 bytes), evenly spread: eight scores per thread
-            uint4 s[2];
+    if (!dense && hi > kWindow) {
+        floor_bits = floor_of_long_span(sh, vec, nv, span, k_mid, cap);
+        fast = floor_bits != 0u;
+        if (tid < 4) prefetch_trip(tid);
+    } else if (!dense) {
+        // 256 blocks of four vectors (64 bytes), evenly spread: eight scores per thread
+        uint4 s[2];
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int k = (tid >> 2) + r * (kThreads / 4);
-                s[r] = load_vec(vec + (int)((int64_t)k * (nv - 4) / (kSample / 16 - 1)) + (tid & 3));
-            }
-            // rank in the sample: the expected one plus 6 sigma (neighbours may be alike), within what the list holds
-            const float r = (float)k_mid * kSample / span;
-            want = min((int)(r + 6.f * sqrtf(r) + 8.f), (int)(0.9f * cap * kSample / span));
-            u[0] = s[0].x; u[1] = s[0].y; u[2] = s[0].z; u[3] = s[0].w;
-            u[4] = s[1].x; u[5] = s[1].y; u[6] = s[1].z; u[7] = s[1].w;
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < 8; ++k) atomicAdd(&sh.hist[sample_bin(u[k])], 1);
+        for (int r = 0; r < 2; ++r) {
+            const int k = (tid >> 2) + r * (kThreads / 4);
+            s[r] = load_vec(vec + (int)((int64_t)k * (nv - 4) / (kSample / 16 - 1)) + (tid & 3));
         }
+        // rank in the sample: the expected one plus 6 sigma (neighbours may be alike), within what the list holds
+        const float r = (float)k_mid * kSample / span;
+        const int want = min((int)(r + 6.f * sqrtf(r) + 8.f), (int)(0.9f * cap * kSample / span));
+        const uint32_t u[8] = {s[0].x, s[0].y, s[0].z, s[0].w, s[1].x, s[1].y, s[1].z, s[1].w};
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) atomicAdd(&sh.hist[sample_bin(u[k])], 1);
         // The span is asked into L2 four trips (128 KB) ahead of the sweep: a trip waits for L2 and not for HBM.
         if (tid < 4) prefetch_trip(tid);
         __syncthreads();
         fast = find_bucket(sh, want);
         const uint32_t bin = (uint32_t)sh.bucket;
-        if (have_hist) {
-            floor_bits = bin << 21;
-            fast = fast && sh.above + sh.count <= cap;
-        } else {
-            floor_bits = kSampleBase + (bin << kSampleShift);
-            if (bin == 0u) {
-                floor_bits = 0u;
-            } else if (fast && sh.count * 4 > want) {  // flat scores, for which 2 % is a coarse step: eleven more bits
-                const int rest = want - sh.above;
+        floor_bits = bin ? kSampleBase + (bin << kSampleShift) : 0u;
+        if (bin && fast && sh.count * 4 > want) {  // flat scores, for which 2 % is a coarse step: eleven more bits
+            const int rest = want - sh.above;
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (sample_bin(u[k]) == (int)bin) atomicAdd(&sh.hist[(u[k] >> (kSampleShift - 11)) & 2047u], 1);
-                __syncthreads();
-                find_bucket(sh, rest);
-                floor_bits |= (uint32_t)sh.bucket << (kSampleShift - 11);
-            }
+            for (int k = 0; k < 8; ++k)
+                if (sample_bin(u[k]) == (int)bin) atomicAdd(&sh.hist[(u[k] >> (kSampleShift - 11)) & 2047u], 1);
+            __syncthreads();
+            find_bucket(sh, rest);
+            floor_bits |= (uint32_t)sh.bucket << (kSampleShift - 11);
         }
         floor_bits = max(floor_bits, 1u);  // (zero scores stay out: if they are needed the list is too short)
     }
@@ -417,6 +538,10 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
         if (lane == 0) atomicMax(&sh.max, mx);
         __syncthreads();
         n_list = dense ? span : sh.list_n;
+        if (floor_bits == 1u && n_list < k_mid && n_list <= cap && !dense) {  // everything but the zeros is in the list: the rest are zeros
+            write_windows(sh, List{list, lpos, 0, n_list, 0}, 0u, 0u, k_mid - n_list, lo, hi, out + k_sink);
+            return;
+        }
         fast = n_list >= k_mid && (dense || n_list <= cap);
     }
 
@@ -448,10 +573,7 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
             bin_lo += (uint32_t)sh.bucket << shift;
             last = (1u << shift) - 1u;
             if (sh.count <= kPair) break;
-            if (shift == 0) {  // more than a thousand equal scores at the threshold
-                fast = false;
-                break;
-            }
+            if (shift == 0) break;  // more than kPair equal scores at the threshold
             shift = max(0, shift - 11);
             __syncthreads();  // (sh.bucket and its fellows are read before the next search writes them)
         }
@@ -459,6 +581,10 @@ select_recall_kernel(const float* __restrict__ stats, int64_t stat_stride, int b
     }
     if (!fast) {
         select_by_sweeps(sh, st, lo, hi, k_mid, out + k_sink);
+        return;
+    }
+    if (hi > kWindow || sh.count > kPair) {
+        write_windows(sh, List{list, dense ? nullptr : lpos, i0, i1, lo - pad}, bin_lo, last, need, lo, hi, out + k_sink);
         return;
     }
     // above the bin: chosen; inside: set aside and ranked pair by pair
@@ -529,7 +655,7 @@ score_hist_kernel(const float* __restrict__ stats, int64_t stat_stride, int batc
 
 int select_launch(const float* stats, int64_t stat_stride, int n_layers, int batch, int n_kv_heads,
                   const int32_t* sel_len, int k_sink, int k_recent, int k_total, int32_t* indices,
-                  int32_t* n_indices, uint32_t* hist, const int32_t* hist_len, cudaStream_t stream)
+                  int32_t* n_indices, uint32_t* hist, cudaStream_t stream)
 {
     const long probs = (long)n_layers * batch * n_kv_heads;
     static std::atomic<bool> opted_in[64] = {};  // per device: the kernel's dynamic shared memory exceeds the default limit
@@ -555,7 +681,7 @@ int select_launch(const float* stats, int64_t stat_stride, int n_layers, int bat
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, select_recall_kernel, stats, stat_stride, batch, n_kv_heads, sel_len, k_sink, k_recent, k_total,
-                           list_words, indices, n_indices, hist, hist_len) != cudaSuccess) {
+                           list_words, indices, n_indices, hist) != cudaSuccess) {
         cudaGetLastError();
         return SPEC_ERR_CUDA;
     }

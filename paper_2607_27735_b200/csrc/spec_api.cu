@@ -294,7 +294,7 @@ int spec_select_recall_hist(const float* stats, int64_t stat_stride, int32_t n_l
     if (k_sink < 0 || k_recent < 0 || k_total < 1 || k_sink + (int64_t)k_recent > k_total)
         return SPEC_ERR_INVALID_ARG;
     return select_launch(stats, stat_stride, n_layers, batch, n_kv_heads, sel_len, k_sink, k_recent,
-                         k_total, indices, n_indices, score_hist, hist_len, static_cast<cudaStream_t>(cuda_stream));
+                         k_total, indices, n_indices, score_hist, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int spec_sparse_draft_attn(const spec_kv_t* kv, const void* q, const int32_t* indices,

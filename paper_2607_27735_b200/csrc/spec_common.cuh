@@ -153,7 +153,7 @@ int verify_generic_launch(const VerifyArgs& a, cudaStream_t stream);
 
 int select_launch(const float* stats, int64_t stat_stride, int n_layers, int batch, int n_kv_heads,
                   const int32_t* sel_len, int k_sink, int k_recent, int k_total, int32_t* indices,
-                  int32_t* n_indices, uint32_t* hist, const int32_t* hist_len, cudaStream_t stream);
+                  int32_t* n_indices, uint32_t* hist, cudaStream_t stream);
 // counts the top 11 bits of stats[prob][0 : len[b]) into hist[prob][kScoreBins] (kernels that do not fuse it)
 int score_hist_launch(const float* stats, int64_t stat_stride, long probs, int batch, int heads, const int32_t* len,
                       int max_len, uint32_t* hist, cudaStream_t stream);

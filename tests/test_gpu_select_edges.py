@@ -71,3 +71,36 @@ def test_any_bit_pattern_is_ordered_as_an_unsigned_number(T, kind):
     want = torch.cat([torch.arange(4, device="cuda").expand(1, 1, 2, 4), mid,
                       torch.arange(T - 64, T, device="cuda").expand(1, 1, 2, 64)], dim=-1).int()
     assert torch.equal(idx, want) and bool((cnt == 1000).all())
+
+
+# the position bitmap holds 131072 positions: spans that end around a multiple of it, large scores in one window only, equal
+# scores at the threshold in all of them, and lengths whose sample grows
+@pytest.mark.parametrize("T,k_total", [(131072 + 63, 1024), (131072 + 64, 1024), (131072 + 65, 4096), (262144 + 64, 4096),
+                                       (262144 + 65, 2048), (300001, 4096), (1048576 + 4, 4096), (3000001, 4096)])
+@pytest.mark.parametrize("where", ["anywhere", "first", "last", "ties", "flat", "zeros"])
+def test_contexts_of_several_windows(T, k_total, where):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    stats = torch.rand(1, 1, 2, T, generator=g, device="cuda") ** 8
+    if where in ("first", "last"):
+        stats[..., slice(4, 5000) if where == "first" else slice(T - 5064, T - 64)] += 1.0
+    elif where == "ties":
+        tie = torch.rand(1, 1, 2, T, generator=g, device="cuda") < 1.2 * k_total / T
+        stats = torch.where(tie, torch.full_like(stats, 0.999), 0.99 * stats)
+    elif where == "flat":
+        stats = 0.5 + 1e-5 * stats
+    elif where == "zeros":  # fewer positive scores than the budget takes
+        few = torch.rand(1, 1, 2, T, generator=g, device="cuda") < 0.3 * k_total / T
+        stats = torch.where(few, stats + 1e-3, torch.zeros_like(stats))
+    check(stats.contiguous(), torch.tensor([T], dtype=torch.int32, device="cuda"), 4, 64, k_total)
+
+
+@pytest.mark.parametrize("n_equal", [512, 513, 2000])
+@pytest.mark.parametrize("T", [3000, 9000, 33333])
+def test_the_lowest_of_equal_scores(T, n_equal):
+    """The threshold among n_equal equal scores, up to which the pairwise ranking goes or does not."""
+    g = torch.Generator(device="cuda").manual_seed(T + n_equal)
+    stats = torch.rand(1, 1, 3, T, generator=g, device="cuda") * 0.5
+    at = torch.rand(1, 1, 3, T, generator=g, device="cuda").argsort(dim=-1)
+    stats.scatter_(-1, at[..., :n_equal], 0.75)
+    stats.scatter_(-1, at[..., n_equal:n_equal + 300], 0.9)
+    check(stats, torch.tensor([T], dtype=torch.int32, device="cuda"), 4, 64, 800)
