@@ -27,7 +27,14 @@ struct FastParams {
     int n_slots, p_bufs;
     int n_raw;                        // 8-bit cache read directly: raw 16 KB stages in front of the operand slots (else 0)
     int D;                            // head_dim: 128, or 64 (score-cache kernel only)
-    int box_rows, boxes;              // TMA boxes per 64-wide half of a tile
+    int box_rows, boxes;              // TMA boxes per 64-wide half of a tile, or (whole_rows) per tile
+    // Score-cache kernel: how a tile lies in its slot.  whole_rows: a box holds whole 256-byte rows, the two 1 KB halves of
+    // eight rows side by side; its place in the cache is layer * row_layer + page * row_page + head * row_head.  Else
+    // (head_dim 64, 8-bit) a box holds one 64-wide half of its rows, the halves of a tile 16 KB apart.  The copy unit
+    // takes 100-150 cycles over a box however small it is, so that with the two halves apart 16-token pages (16 boxes of 2 KB
+    // per tile) were bound by it: eight sequences of 9-66 K took 345 us, 241 on 64-token pages; with whole rows 272 and 246.
+    int whole_rows, half_bytes, group_bytes;  // bytes from half to half and from eight rows to the next eight
+    int row_layer, row_page, row_head;
     float scale_log2;
     // score-cache kernel: HG teams of cph CTAs; sequences short enough run on a team's parts (see Sched)
     int n_cls;                        // classes in use
@@ -178,10 +185,10 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 
-// K-major operand, 128-byte swizzle: rows of 128 B, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr)
+// K-major operand, 128-byte swizzle: rows of 128 B, 8-row groups `group` bytes apart.
+__device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, uint32_t group = 1024)
 {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | (1ull << 16) | ((uint64_t)(group >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 // MN-major operand without swizzle: 8x8 core matrices of 128 contiguous bytes, K groups 128 B
 // apart (leading offset), 8-row MN blocks 2048 B apart (stride offset).
@@ -189,11 +196,12 @@ __device__ __forceinline__ uint64_t desc_mnmajor_nosw(uint32_t saddr)
 {
     return (uint64_t)((saddr >> 4) & 0x3FFF) | (8ull << 16) | (128ull << 32) | (1ull << 46);
 }
-// MN-major operand, 128-byte swizzle: 64-element MN blocks 16 KiB apart (leading offset),
-// 8-row K groups 1024 B apart (stride offset).
-__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t saddr)
+// MN-major operand, 128-byte swizzle: 64-element MN blocks `half` bytes apart (leading offset),
+// 8-row K groups `group` bytes apart (stride offset).
+__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t saddr, uint32_t half = 16384, uint32_t group = 1024)
 {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | (1024ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(half >> 4) << 16) | ((uint64_t)(group >> 4) << 32) | (1ull << 46) |
+           (2ull << 61);
 }
 
 // ---------------------------------------------------------------------------------------------

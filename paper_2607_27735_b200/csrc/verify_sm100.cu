@@ -3,6 +3,7 @@
 // score-cache kernel (K and V read once) and the two-sweep kernel (any context length).
 #include <climits>
 #include <cstdlib>
+#include <numeric>
 
 #include "sm100_common.cuh"
 #include "verify_sm100.cuh"
@@ -249,6 +250,34 @@ bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_p
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The cache as rows of two 64-wide halves: dimensions (64, 8 rows, half, groups of 8 rows in a page, (layer, page, head)).
+// One box then brings whole rows, the halves of eight of them as two swizzled 1 KB blocks side by side.  The last
+// dimension counts in the greatest common divisor of the three strides.
+// False where a row cannot be numbered in 31 bits (and for head_dim 64): the caller takes the other map.
+bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn || kv.head_dim != kD) return false;
+    const int64_t st[3] = {kv.n_layers > 1 ? kv.layer_stride : 0, n_pages > 1 ? kv.page_stride : 0,
+                           kv.n_kv_heads > 1 ? kv.head_stride : 0};
+    const int64_t n[3] = {kv.n_layers, n_pages, kv.n_kv_heads};
+    int64_t unit = 0, last = 0;
+    for (int64_t s : st) unit = std::gcd(unit, s);
+    if (unit == 0) unit = 8;
+    for (int i = 0; i < 3; ++i) last += st[i] / unit * (n[i] - 1);
+    if (last >= INT_MAX || kv.slot_stride >= 1ll << 35 || unit >= 1ll << 38) return false;
+    fp->row_layer = (int)(st[0] / unit);
+    fp->row_page = (int)(st[1] / unit);
+    fp->row_head = (int)(st[2] / unit);
+    const cuuint64_t dims[5] = {64, 8, 2, (cuuint64_t)kv.page_size / 8, (cuuint64_t)last + 1};
+    const cuuint64_t strides[4] = {(cuuint64_t)kv.slot_stride * 2, 128, (cuuint64_t)kv.slot_stride * 16, (cuuint64_t)unit * 2};
+    const cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)box_rows / 8, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // 8-bit cache: a box is box_rows whole rows of 128 bytes, unswizzled (the softmax warps expand it)
 bool encode_kv_map_u8(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows)
 {
@@ -470,17 +499,23 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
     const int G = a.kv.n_q_heads / a.kv.n_kv_heads;
     const int n_pages = a.kv.n_pages;
     CUtensorMap tk, tv, tq;
+    FastParams fp;
+    fp.whole_rows = 0;
     if (a.kv.fp8) {
         if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows) ||
             !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows))
             return SPEC_ERR_CUDA;
+    } else if (pl.cached && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
+               encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
+        fp.whole_rows = 1;
     } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows) ||
                !encode_kv_map(&tv, a.kv.v, a.kv, n_pages, pl.box_rows)) {
         return SPEC_ERR_CUDA;
     }
     if (!encode_q_map(&tq, a.q, a.kv, a.n_q, G)) return SPEC_ERR_CUDA;
     char* ws = static_cast<char*>(a.workspace);
-    FastParams fp;
+    fp.half_bytes = fp.whole_rows ? 1024 : 16384;
+    fp.group_bytes = fp.whole_rows ? 2048 : 1024;
     fp.a = a;
     fp.HG = pl.HG;
     fp.NHG = pl.cached ? 1 : a.kv.n_kv_heads / pl.HG;

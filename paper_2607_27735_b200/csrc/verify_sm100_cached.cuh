@@ -499,10 +499,12 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         // =========================== TMA producer ===========================
         uint32_t ring = 0, ring_ph = 0, qn = 0;  // next slot (F8: raw stage), its phase; Q buffers filled
         const int boxes = p.boxes, box_rows = p.box_rows;
-        const uint32_t box_bytes = box_rows * 128;
+        const bool whole = !F8 && p.whole_rows;
+        const uint32_t box_bytes = box_rows * (whole ? 256 : 128);
         const int halves = p.D / 64;  // 64-wide halves of the head dimension
         bool ok = true;
-        // A tile's boxes, one per lane (at most 16 boxes of 8 rows, for either half of the head dimension).  F8: the
+        // A tile's boxes, one per lane: at most 16 of 8 whole rows, or that many for either half of the head dimension.
+        // F8: the
         // tile's bytes (128 per key) go to a raw stage, and the softmax warps expand them into a slot.
         // The page table is read before the wait for a free slot: its latency (a trip to L2 per tile, which bounded
         // the stream of 16-token pages) hides behind that wait.
@@ -510,8 +512,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const int key0 = tile * kTile;
             // boxes that hold at least one key < T (pages past the context may not exist)
             const int n_box = min(boxes, (sg.T - key0 + box_rows - 1) / box_rows);
-            const int n_ops = F8 ? n_box : halves * n_box;
-            const int half = !F8 && lane >= n_box ? 1 : 0, bx = lane - half * n_box;
+            const int n_ops = F8 || whole ? n_box : halves * n_box;
+            const int half = !F8 && !whole && lane >= n_box ? 1 : 0, bx = lane - half * n_box;
             const int pos = key0 + bx * box_rows;
             const int page = page_of(p.a.kv, pos), slot_in_page = pos - page * p.a.kv.page_size;
             int phys = 0;
@@ -535,7 +537,11 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 if (got) mbar_expect_tx(full, (uint32_t)n_ops * box_bytes);
             }
             if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
-            if (lane < n_ops)
+            if (whole) {
+                if (lane < n_ops)
+                    tma_load_5d(s_slots + s * kSlotBytes + bx * box_bytes, map, full, 0, 0, 0, slot_in_page >> 3,
+                                sg.layer * p.row_layer + phys * p.row_page + sg.h * p.row_head, kEvictFirst);
+            } else if (lane < n_ops)
                 tma_load_5d((F8 ? s_raw + s * 16384 : s_slots + s * kSlotBytes + half * 16384) + bx * box_bytes, map, full,
                             half * 64, slot_in_page, sg.h, phys, sg.layer, kEvictFirst);
             __syncwarp();
@@ -576,6 +582,12 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             // O^T += V^T [P_hi | P_lo]^T : A = V^T and B = P^T both MN-major, N = 2 * rows
             const uint32_t idesc_pv = (1u << 4) | ab_fmt | (1u << 15) | (1u << 16) |
                                       ((uint32_t)((2 * N) >> 3) << 17) | ((128u >> 4) << 24);
+            // Descriptors of slot 0's tiles (a place further on in shared memory only adds to them), the step to a row's
+            // other half and by 16 keys.  (Worked out anew for every product from the layout, which is not known at
+            // compile time, a launch of the 8B shape took 42.4 us instead of 39.1.)
+            const uint64_t k_desc = desc_kmajor(s_slots, p.group_bytes);
+            const uint64_t v_desc = desc_mnmajor(s_slots, p.half_bytes, p.group_bytes);
+            const uint32_t k_half = p.half_bytes >> 4, v_step = p.group_bytes >> 3;
             // Two independent queues, issued in whichever order their inputs become ready: the
             // QK^T tiles of unit u+1 may overtake the P V tiles of unit u that still wait for P.
             struct Queue {
@@ -626,12 +638,12 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             auto issue_qk = [&]() {
                 sfree_par ^= 1u << region;
                 tc_fence_after();
-                const uint32_t k_addr = s_slots + qq.slot * kSlotBytes;
+                const uint64_t k_tile = k_desc + qq.slot * (kSlotBytes >> 4);
                 const uint32_t d_s = tmem_base + col_s + region * N;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     if (ks * 16 < p.D) {  // head_dim 64: the first four 16-wide steps
-                        const uint64_t a = desc_kmajor(k_addr + (ks >> 2) * 16384 + (ks & 3) * 32);
+                        const uint64_t a = k_tile + ((ks >> 2) * k_half + (ks & 3) * 2);
                         const uint64_t b = desc_kmajor(s_q + (ks >> 2) * (N * 128) + (ks & 3) * 32);
                         tc_mma(d_s, a, b, idesc_qk, ks ? 1u : 0u);
                     }
@@ -653,12 +665,12 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             };
             auto issue_pv = [&]() {
                 tc_fence_after();
-                const uint32_t v_addr = s_slots + pq.slot * kSlotBytes;
+                const uint64_t v_tile = v_desc + pq.slot * (kSlotBytes >> 4);
                 const uint32_t p_addr = s_p + pb * p_bytes;
                 const uint32_t d_o = tmem_base + col_o;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t a = desc_mnmajor(v_addr + ks * 2048);
+                    const uint64_t a = v_tile + ks * v_step;
                     const uint64_t b = desc_mnmajor_nosw(p_addr + ks * 256);
                     tc_mma(d_o, a, b, idesc_pv, (pq.c == 0 && ks == 0) ? 0u : 1u);
                 }
@@ -1281,7 +1293,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                             ok = bar_wait(B.slot_full + 8 * vs, vsph, ctl);
                             if (!ok) break;
                             if (key >= sg.T && wg < 2) {  // warpgroups 0 and 1 clear one 64-wide half each
-                                uint8_t* vrow = sgen + (s_slots - sbase) + vs * kSlotBytes + wg * 16384 + key_l * 128;
+                                uint8_t* vrow = sgen + (s_slots - sbase) + vs * kSlotBytes + wg * p.half_bytes +
+                                                (key_l >> 3) * p.group_bytes + (key_l & 7) * 128;
 #pragma unroll
                                 for (int ch = 0; ch < 8; ++ch) *reinterpret_cast<uint4*>(vrow + 16 * ch) = make_uint4(0, 0, 0, 0);
                             }

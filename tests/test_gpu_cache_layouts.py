@@ -1,0 +1,50 @@
+"""Verification over the same keys and values laid out in memory in different ways: what the copies of a tile are built from
+is the strides' greatest common divisor, so heads outside pages, heads between rows, padded rows, layers inside
+pages and pages of 8 to 128 tokens have to give the bits that the dense order gives (the arithmetic behind the copies is
+the same)."""
+import dataclasses
+
+import pytest
+import torch
+
+import oracle
+from paper_2607_27735_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+TOL = 2e-3
+L, H, D, N_Q = 2, 2, 128, 5
+
+
+def laid_out(kv, order, pad):
+    """``kv`` ([layer, page, head, slot, D]) with its first four axes stored in ``order`` and ``pad`` elements behind each row."""
+    axes = [kv.n_layers, kv.k.shape[1], H, kv.page_size]
+    strides, step = [0] * 4, D + pad
+    for a in reversed(order):
+        strides[a] = step
+        step *= axes[a]
+    def store(x):
+        flat = torch.full((step + D,), 7.0, device=x.device, dtype=x.dtype)
+        flat.as_strided(axes + [D], strides + [1]).copy_(x)
+        return flat
+    return dataclasses.replace(kv, k=store(kv.k), v=store(kv.v), layer_stride=strides[0], page_stride=strides[1],
+                               head_stride=strides[2], slot_stride=strides[3], n_pages=kv.k.shape[1])
+
+
+@pytest.mark.parametrize("page", [8, 16, 64, 128])
+@pytest.mark.parametrize("ctx", [[700, 129, 128], [9]])
+def test_every_order_gives_the_bits_of_the_dense_one(page, ctx):
+    cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=N_Q, n_q_heads=4 * H, n_kv_heads=H, head_dim=D, planted=4,
+                              batch=len(ctx), n_layers=L, page_size=page, shuffled_pages=True, seed=5)
+    case = inputs.make_case(cfg, device="cuda", ctx_override=ctx)
+    T = max(ctx)
+    ref = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, T)
+    assert binding.read_status(ref[3]) == 0
+    o_out, o_lse, _ = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, ref[2].shape[-1])
+    assert (ref[0].cpu().double() - o_out).abs().max().item() <= TOL
+    assert (ref[1].cpu().double() - o_lse).abs().max().item() <= TOL
+    for order, pad in (((0, 1, 2, 3), 8), ((0, 1, 3, 2), 0), ((2, 0, 1, 3), 0), ((1, 0, 2, 3), 24), ((3, 2, 1, 0), 0), ((0, 2, 1, 3), 8)):
+        out, lse, stats, ws = binding.spec_verify_attn(laid_out(case.kv, order, pad), case.q_verify, case.ctx_len, T)
+        assert binding.read_status(ws) == 0
+        assert torch.equal(out, ref[0]) and torch.equal(lse, ref[1])
+        for b, t in enumerate(ctx):
+            assert torch.equal(stats[:, b, :, :t], ref[2][:, b, :, :t])
