@@ -50,12 +50,6 @@ __device__ __forceinline__ void mma_f16_16816(float (&d)[4], uint32_t a0, uint32
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// two e4m3 bytes (the low 16 bits of `two`) as a packed fp16 pair: exact
-__device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two)
-{
-    const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(two & 0xffffu), __NV_E4M3);
-    return (uint32_t)h.x | ((uint32_t)h.y << 16);
-}
 __device__ __forceinline__ uint32_t pack_f16(float x, float y)
 {
     const __half2 v = __floats2half2_rn(x, y);
@@ -196,9 +190,8 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
         waited = true;
     }
     // A fragments of Q (heads x d): the thread holds head grp at d = 16 ks + 2 quad + {0, 1} and + {8, 9}.
-    // F8: the K fragment of a step comes from ONE 4-byte load (d = 16 ks + 4 quad + 0..3), so the step's
-    // sixteen d's are visited in that order and Q follows it: d = 16 ks + 4 quad + {0, 1} and + {2, 3},
-    // as fp16.
+    // F8: a thread takes a quarter of a K row in 16-byte loads, four bytes of it per step, so a step's sixteen d's are
+    // D / 4 * quad + 4 ks + 0..3 and Q follows that order: + {0, 1} and + {2, 3}, as fp16.
     // keys_on_rows (see below): Q is the B operand and its eight columns are the heads 0, 0, 1, 1, 2, 2, 3, 3
     const bool keys_on_rows = G <= 4;
     const int qh = keys_on_rows ? grp >> 1 : grp;  // the head whose row this thread's fragments come from
@@ -206,14 +199,21 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
     {
         const int64_t row = ((int64_t)layer * a.kv.batch + b) * a.kv.n_q_heads + h * G + qh;
         const uint32_t* qrow = reinterpret_cast<const uint32_t*>(a.q + row * D);
+        if (F8) {
+            uint4 w[KS / 2];
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            if (F8) {
-                const uint32_t w0 = qh < G ? __ldg(qrow + ks * 8 + 2 * quad) : 0u;
-                const uint32_t w1 = qh < G ? __ldg(qrow + ks * 8 + 2 * quad + 1) : 0u;
-                qa[ks][0] = pack_f16(bf16_lo(w0), bf16_hi(w0));
-                qa[ks][1] = pack_f16(bf16_lo(w1), bf16_hi(w1));
-            } else {
+            for (int i = 0; i < KS / 2; ++i)
+                w[i] = qh < G ? __ldg(reinterpret_cast<const uint4*>(qrow + quad * (D / 8)) + i) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int i = 0; i < KS / 2; ++i) {
+                qa[2 * i][0] = pack_f16(bf16_lo(w[i].x), bf16_hi(w[i].x));
+                qa[2 * i][1] = pack_f16(bf16_lo(w[i].y), bf16_hi(w[i].y));
+                qa[2 * i + 1][0] = pack_f16(bf16_lo(w[i].z), bf16_hi(w[i].z));
+                qa[2 * i + 1][1] = pack_f16(bf16_lo(w[i].w), bf16_hi(w[i].w));
+            }
+        } else {
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
                 qa[ks][0] = qh < G ? __ldg(qrow + ks * 8 + quad) : 0u;
                 qa[ks][1] = qh < G ? __ldg(qrow + ks * 8 + 4 + quad) : 0u;
             }
@@ -226,23 +226,35 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
 #pragma unroll
     for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
 
+    // F8: this thread's quarter of K rows grp and grp + 8 of a chunk (four bytes per step)
+    auto load_quarter = [&](const uint8_t* ksm, uint32_t (&k0)[KS], uint32_t (&k1)[KS]) {
+        const uint8_t* kp = ksm + grp * ROWB + quad * (D / 4);
+#pragma unroll
+        for (int i = 0; i < KS; i += 4) {
+            const uint4 a = *reinterpret_cast<const uint4*>(kp + 4 * i), b = *reinterpret_cast<const uint4*>(kp + 8 * ROWB + 4 * i);
+            k0[i] = a.x, k0[i + 1] = a.y, k0[i + 2] = a.z, k0[i + 3] = a.w;
+            k1[i] = b.x, k1[i + 1] = b.y, k1[i + 2] = b.z, k1[i + 3] = b.w;
+        }
+    };
     // S = Q K^T of the chunk in a stage: keys 0..7 and 8..15 are the two 8-wide column blocks
     auto qk = [&](const uint8_t* ksm, float (&s0)[4], float (&s1)[4]) {
         {
             float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};  // four accumulation chains
             if (F8) {
-                // key grp (and grp + 8), bytes 16 ks + 4 quad .. + 3: one load per key block and step
-                const uint8_t* kp = ksm + grp * ROWB + 4 * quad;
+                // keys grp and grp + 8
+                uint32_t k0[KS], k1[KS];
+                load_quarter(ksm, k0, k1);
 #pragma unroll
                 for (int ks = 0; ks < KS; ks += 2) {
-                    const uint32_t k00 = *reinterpret_cast<const uint32_t*>(kp + ks * 16);
-                    const uint32_t k01 = *reinterpret_cast<const uint32_t*>(kp + 8 * ROWB + ks * 16);
-                    const uint32_t k10 = *reinterpret_cast<const uint32_t*>(kp + ks * 16 + 16);
-                    const uint32_t k11 = *reinterpret_cast<const uint32_t*>(kp + 8 * ROWB + ks * 16 + 16);
-                    mma_f16_16816(s0, qa[ks][0], 0u, qa[ks][1], 0u, e4m3x2_to_f16x2(k00), e4m3x2_to_f16x2(k00 >> 16));
-                    mma_f16_16816(s1, qa[ks][0], 0u, qa[ks][1], 0u, e4m3x2_to_f16x2(k01), e4m3x2_to_f16x2(k01 >> 16));
-                    mma_f16_16816(t0, qa[ks + 1][0], 0u, qa[ks + 1][1], 0u, e4m3x2_to_f16x2(k10), e4m3x2_to_f16x2(k10 >> 16));
-                    mma_f16_16816(t1, qa[ks + 1][0], 0u, qa[ks + 1][1], 0u, e4m3x2_to_f16x2(k11), e4m3x2_to_f16x2(k11 >> 16));
+                    uint32_t a[8];
+                    e4m3x4_to_f16x4(k0[ks], a[0], a[1]);
+                    e4m3x4_to_f16x4(k1[ks], a[2], a[3]);
+                    e4m3x4_to_f16x4(k0[ks + 1], a[4], a[5]);
+                    e4m3x4_to_f16x4(k1[ks + 1], a[6], a[7]);
+                    mma_f16_16816(s0, qa[ks][0], 0u, qa[ks][1], 0u, a[0], a[1]);
+                    mma_f16_16816(s1, qa[ks][0], 0u, qa[ks][1], 0u, a[2], a[3]);
+                    mma_f16_16816(t0, qa[ks + 1][0], 0u, qa[ks + 1][1], 0u, a[4], a[5]);
+                    mma_f16_16816(t1, qa[ks + 1][0], 0u, qa[ks + 1][1], 0u, a[6], a[7]);
                 }
             } else {
                 const uint8_t* kp = ksm + ((lane & 7) + ((lane >> 4) & 1) * 8) * ROWB + ((lane >> 3) & 1) * 16;
@@ -301,14 +313,13 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
             for (int j = 0; j < D / 32; ++j) {
                 uint32_t vf[4];
                 ldmatrix_x4_trans(vf, vp + j * 32);
-                mma_f16_16816(o[4 * j + 0], ah0, al0, ah1, al1, e4m3x2_to_f16x2(__byte_perm(vf[0], 0u, 0x4420)),
-                              e4m3x2_to_f16x2(__byte_perm(vf[1], 0u, 0x4420)));
-                mma_f16_16816(o[4 * j + 1], ah0, al0, ah1, al1, e4m3x2_to_f16x2(__byte_perm(vf[0], 0u, 0x4431)),
-                              e4m3x2_to_f16x2(__byte_perm(vf[1], 0u, 0x4431)));
-                mma_f16_16816(o[4 * j + 2], ah0, al0, ah1, al1, e4m3x2_to_f16x2(__byte_perm(vf[2], 0u, 0x4420)),
-                              e4m3x2_to_f16x2(__byte_perm(vf[3], 0u, 0x4420)));
-                mma_f16_16816(o[4 * j + 3], ah0, al0, ah1, al1, e4m3x2_to_f16x2(__byte_perm(vf[2], 0u, 0x4431)),
-                              e4m3x2_to_f16x2(__byte_perm(vf[3], 0u, 0x4431)));
+                uint32_t e[4], f[4];  // even d, odd d
+#pragma unroll
+                for (int i = 0; i < 4; ++i) e4m3x4_to_f16x4(__byte_perm(vf[i], 0u, 0x3120), e[i], f[i]);
+                mma_f16_16816(o[4 * j + 0], ah0, al0, ah1, al1, e[0], e[1]);
+                mma_f16_16816(o[4 * j + 1], ah0, al0, ah1, al1, f[0], f[1]);
+                mma_f16_16816(o[4 * j + 2], ah0, al0, ah1, al1, e[2], e[3]);
+                mma_f16_16816(o[4 * j + 3], ah0, al0, ah1, al1, f[2], f[3]);
             }
         } else {
             const uint8_t* vp = vsm + ((lane & 7) + ((lane >> 3) & 1) * 8) * ROWB + ((lane >> 4) & 1) * 16;
@@ -337,19 +348,18 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
         auto tr_qk = [&](const uint8_t* ksm, float (&st)[2]) {
             float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};  // two accumulation chains
             if (F8) {
-                // rows grp and grp + 8, bytes 16 ks + 4 quad .. + 3: one 4-byte load per row and step gives the
-                // row's two fragment registers (the step's sixteen d's are visited in that order, as Q's are)
-                const uint8_t* kp = ksm + grp * ROWB + 4 * quad;
+                // rows grp and grp + 8
+                uint32_t k0[KS], k1[KS];
+                load_quarter(ksm, k0, k1);
 #pragma unroll
                 for (int ks = 0; ks < KS; ks += 2) {
-                    const uint32_t k00 = *reinterpret_cast<const uint32_t*>(kp + ks * 16);
-                    const uint32_t k01 = *reinterpret_cast<const uint32_t*>(kp + 8 * ROWB + ks * 16);
-                    const uint32_t k10 = *reinterpret_cast<const uint32_t*>(kp + ks * 16 + 16);
-                    const uint32_t k11 = *reinterpret_cast<const uint32_t*>(kp + 8 * ROWB + ks * 16 + 16);
-                    mma_f16_16816(c0, e4m3x2_to_f16x2(k00), e4m3x2_to_f16x2(k01), e4m3x2_to_f16x2(k00 >> 16),
-                                  e4m3x2_to_f16x2(k01 >> 16), qa[ks][0], qa[ks][1]);
-                    mma_f16_16816(c1, e4m3x2_to_f16x2(k10), e4m3x2_to_f16x2(k11), e4m3x2_to_f16x2(k10 >> 16),
-                                  e4m3x2_to_f16x2(k11 >> 16), qa[ks + 1][0], qa[ks + 1][1]);
+                    uint32_t a[8];
+                    e4m3x4_to_f16x4(k0[ks], a[0], a[2]);
+                    e4m3x4_to_f16x4(k1[ks], a[1], a[3]);
+                    e4m3x4_to_f16x4(k0[ks + 1], a[4], a[6]);
+                    e4m3x4_to_f16x4(k1[ks + 1], a[5], a[7]);
+                    mma_f16_16816(c0, a[0], a[1], a[2], a[3], qa[ks][0], qa[ks][1]);
+                    mma_f16_16816(c1, a[4], a[5], a[6], a[7], qa[ks + 1][0], qa[ks + 1][1]);
                 }
             } else {
                 const uint8_t* kp = ksm + ((lane & 7) + ((lane >> 3) & 1) * 8) * ROWB + (lane >> 4) * 16;
@@ -396,14 +406,11 @@ draft_stream_kernel(DraftArgs a, StreamShape shp, int* __restrict__ status)
                 for (int j = 0; j < D / 32; ++j) {
                     uint32_t vf[4];  // keys 0..7 x bytes 0..15, keys 0..7 x bytes 16..31, keys 8..15 x the same
                     ldmatrix_x4_trans(vf, vp + j * 32);
-                    mma_f16_16816(ot[2 * j], e4m3x2_to_f16x2(__byte_perm(vf[0], 0u, 0x4420)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[0], 0u, 0x4431)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[2], 0u, 0x4420)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[2], 0u, 0x4431)), b0, b1);
-                    mma_f16_16816(ot[2 * j + 1], e4m3x2_to_f16x2(__byte_perm(vf[1], 0u, 0x4420)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[1], 0u, 0x4431)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[3], 0u, 0x4420)),
-                                  e4m3x2_to_f16x2(__byte_perm(vf[3], 0u, 0x4431)), b0, b1);
+                    uint32_t e[4], f[4];  // even d, odd d
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) e4m3x4_to_f16x4(__byte_perm(vf[i], 0u, 0x3120), e[i], f[i]);
+                    mma_f16_16816(ot[2 * j], e[0], f[0], e[2], f[2], b0, b1);
+                    mma_f16_16816(ot[2 * j + 1], e[1], f[1], e[3], f[3], b0, b1);
                 }
             } else {
 #pragma unroll

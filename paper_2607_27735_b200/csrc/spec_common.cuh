@@ -69,6 +69,18 @@ __device__ __forceinline__ int64_t kv_row_offset(const KvView& kv, int layer, in
            slot * kv.slot_stride;
 }
 
+// Four e4m3 bytes as two packed fp16 pairs (bytes 0, 1 and bytes 2, 3): exact, subnormals included.
+// One instruction per pair, which picks its half of the register itself: 68 elements per clock of an SM.  (The intrinsic
+// returns its two halves apart; putting them together took more instructions than the conversion, and the draft kernel
+// over an 8-bit cache 8.4 us instead of 6.5 per call of eight ragged sequences.  By integer instructions - the byte's low
+// seven bits shifted into bits 7..13 of an fp16 give the value times 2^-8 - 25 elements per clock.)
+__device__ __forceinline__ void e4m3x4_to_f16x4(uint32_t w, uint32_t& lo, uint32_t& hi)
+{
+    asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tcvt.rn.f16x2.e4m3x2 %0, a;\n\tcvt.rn.f16x2.e4m3x2 %1, b;\n\t}"
+        : "=r"(lo), "=r"(hi)
+        : "r"(w));
+}
+
 // Two e4m3 bytes (low byte first) as two floats: exact (cvt to fp16 holds every e4m3 value).
 __device__ __forceinline__ float2 e4m3x2_to_float2(uint16_t two)
 {

@@ -94,17 +94,6 @@ __device__ __forceinline__ void sum_step(float (&l)[NHT], int lane, int& col)
     }
 }
 
-// Four e4m3 bytes as two packed fp16 pairs (bytes 0, 1 and bytes 2, 3): exact, subnormals included.
-// (The same by integer instructions - the byte's low seven bits shifted into bits 7..13 of an fp16 give the
-// value times 2^-8 - measured slower: the softmax warps are bound by instruction issue, and that takes four
-// instructions per pair instead of one.)
-__device__ __forceinline__ void e4m3x4_to_f16x4(uint32_t w, uint32_t& lo, uint32_t& hi)
-{
-    asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tcvt.rn.f16x2.e4m3x2 %0, a;\n\tcvt.rn.f16x2.e4m3x2 %1, b;\n\t}"
-        : "=r"(lo), "=r"(hi)
-        : "r"(w));
-}
-
 // Which problem a CTA works on in which unit.  A problem is one KV head of one (layer, sequence).  Teams of cph CTAs are
 // sized for the longest context the call allows; a sequence whose share still fits the score cache on a half,
 // a quarter or an eighth of a team runs on such a part, several problems side by side: a round costs a fixed
