@@ -48,3 +48,16 @@ def test_every_order_gives_the_bits_of_the_dense_one(page, ctx):
         assert torch.equal(out, ref[0]) and torch.equal(lse, ref[1])
         for b, t in enumerate(ctx):
             assert torch.equal(stats[:, b, :, :t], ref[2][:, b, :, :t])
+
+
+def test_rows_beyond_31_bits_take_the_other_map():
+    """A pool whose rows cannot be numbered in 31 bits (it is only said to be that large; the pages in use are the same): tiles
+    are copied half by half into the other layout, which gives the same bits."""
+    cfg = inputs.small_config(ctx=(700, 700), n_q=N_Q, n_q_heads=4 * H, n_kv_heads=H, head_dim=D, planted=4, n_layers=L,
+                              page_size=16, shuffled_pages=True, seed=6)
+    case = inputs.make_case(cfg, device="cuda")
+    ref = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, 700)
+    large = dataclasses.replace(case.kv, n_pages=(1 << 30) + 8)
+    out, lse, stats, ws = binding.spec_verify_attn(large, case.q_verify, case.ctx_len, 700)
+    assert binding.read_status(ws) == 0
+    assert torch.equal(out, ref[0]) and torch.equal(lse, ref[1]) and torch.equal(stats[..., :700], ref[2][..., :700])
