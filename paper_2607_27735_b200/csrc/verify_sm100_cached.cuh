@@ -696,7 +696,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     spins = 0;
                     continue;
                 }
-                __nanosleep(40);  // idle: leave the issue slots of this sub-core to the softmax warps
+                // (No sleep here: with 40 ns between two looks four layers over an 8-bit cache took 200.5 us instead of 198.1, 16 chats
+                // 372.6 instead of 371.6 a round; the softmax warps do not miss the issue slots.)
                 if ((++spins & 63u) == 0) {
                     if (spins == 64) t_idle = clock64();
                     if (*ctl.abort_flag) ok = false;
