@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libspec_attn.so")
 NATIVE = os.path.join(HERE, "_spec_native.so")
 NATIVE_SRC = os.path.join(CSRC, "py_native.cpp")
 SOURCES = ["spec_api.cu", "verify_generic.cu", "verify_sm100.cu", "verify_sm100_twosweep.cu",
-           "verify_sm100_cached.cu", "verify_sm100_cached_ph.cu",
+           "verify_sm100_cached.cu", "verify_sm100_cached_rows.cu", "verify_sm100_cached_ph.cu", "verify_sm100_cached_ph_rows.cu",
            "verify_sm100_cached_sc.cu", "verify_sm100_cached_f8.cu", "select_recall.cu", "draft_stream.cu", "spec_noalloc.cu",
            "length_ctrl.cu", "kv_expand.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

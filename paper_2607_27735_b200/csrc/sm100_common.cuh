@@ -12,7 +12,7 @@ namespace sm100 {
 
 constexpr int kTile = 128;            // keys per tile = UMMA M
 constexpr int kD = 128;               // head_dim the tiles are laid out for (head_dim 64 uses the lower half)
-constexpr int kSlotBytes = 32768;     // one K or V tile: 2 halves x 128 rows x 128 B (SW128)
+constexpr int kSlotBytes = 32768;     // one K or V tile: 128 rows of two 128-byte halves (SW128)
 constexpr int kThreads = 384;
 constexpr int kMaxClass = 4;          // whole teams, then halves, quarters and eighths
 constexpr int kRing = 4;              // partial buffers are recycled every kRing units
@@ -27,13 +27,9 @@ struct FastParams {
     int n_slots, p_bufs;
     int n_raw;                        // 8-bit cache read directly: raw 16 KB stages in front of the operand slots (else 0)
     int D;                            // head_dim: 128, or 64 (score-cache kernel only)
-    int box_rows, boxes;              // TMA boxes per 64-wide half of a tile, or (whole_rows) per tile
-    // Score-cache kernel: how a tile lies in its slot.  whole_rows: a box holds whole 256-byte rows, the two 1 KB halves of
-    // eight rows side by side; its place in the cache is layer * row_layer + page * row_page + head * row_head.  Else
-    // (head_dim 64, 8-bit) a box holds one 64-wide half of its rows, the halves of a tile 16 KB apart.  The copy unit
-    // takes 100-150 cycles over a box however small it is, so that with the two halves apart 16-token pages (16 boxes of 2 KB
-    // per tile) were bound by it: eight sequences of 9-66 K took 345 us, 241 on 64-token pages; with whole rows 272 and 246.
-    int whole_rows, half_bytes, group_bytes;  // bytes from half to half and from eight rows to the next eight
+    int box_rows, boxes;              // rows of a TMA box; boxes per tile (two 64-wide halves apart: per half)
+    int whole_rows;                   // score-cache kernel: boxes of whole rows (see encode_kv_map_rows), whose place in the
+                                      // cache is layer * row_layer + page * row_page + head * row_head
     int row_layer, row_page, row_head;
     float scale_log2;
     // score-cache kernel: HG teams of cph CTAs; sequences short enough run on a team's parts (see Sched)

@@ -253,6 +253,8 @@ bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_p
 // The cache as rows of two 64-wide halves: dimensions (64, 8 rows, half, groups of 8 rows in a page, (layer, page, head)).
 // One box then brings whole rows, the halves of eight of them as two swizzled 1 KB blocks side by side.  The last
 // dimension counts in the greatest common divisor of the three strides.
+// The copy unit takes 100-150 cycles over a box however small it is, so that 16-token pages were bound by it with the halves
+// in boxes of their own (16 boxes of 2 KB per tile): eight sequences of 9-66 K took 348 us, 262 with whole rows.
 // False where a row cannot be numbered in 31 bits (and for head_dim 64): the caller takes the other map.
 bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
 {
@@ -505,7 +507,7 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows) ||
             !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows))
             return SPEC_ERR_CUDA;
-    } else if (pl.cached && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
+    } else if (pl.cached && !a.kv.k_scale && !a.kv.v_scale && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
                encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
         fp.whole_rows = 1;
     } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows) ||
@@ -514,8 +516,6 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
     }
     if (!encode_q_map(&tq, a.q, a.kv, a.n_q, G)) return SPEC_ERR_CUDA;
     char* ws = static_cast<char*>(a.workspace);
-    fp.half_bytes = fp.whole_rows ? 1024 : 16384;
-    fp.group_bytes = fp.whole_rows ? 2048 : 1024;
     fp.a = a;
     fp.HG = pl.HG;
     fp.NHG = pl.cached ? 1 : a.kv.n_kv_heads / pl.HG;

@@ -331,7 +331,11 @@ struct CBars {  // mbarrier addresses (shared space)
 // fp16 operands: Q is converted once per unit in shared memory, P~ is split into an fp16 rounding of
 // 2^14 P~ and the fp16 rounding of 2^11 times its remainder (the two accumulator halves are added with
 // that weight in the epilogue); the powers of two join the scales.
-template <int NC, int CG, bool LP, bool PH, bool SC, bool F8>
+// WR: a tile lies in its slot as whole rows, the two 1 KB halves of eight rows side by side (see encode_kv_map_rows); else
+// its two 64-wide halves lie 16 KB apart.  A template parameter, since the loops that the distances go into do not bear them
+// as run-time values: the MMA warp's descriptors (eight sequences of 9-66 K on 64-token pages 244 -> 248 us, over an 8-bit cache 323 ->
+// 330) and the clearing of the ragged tail's rows (80 score columns: 315 -> 350 us for two sequences of 40 K).
+template <int NC, int CG, bool LP, bool PH, bool SC, bool F8, bool WR>
 __global__ void __launch_bounds__(128 + 128 * CG, 1)
 verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ FastParams p)
@@ -343,6 +347,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     constexpr int NH = NC;                       // columns per thread
     constexpr int kBlock = 128 + 128 * CG;       // threads per CTA
     constexpr int kSW = 4 * CG;                  // softmax warps
+    constexpr int kHalf = WR ? 1024 : 16384;     // bytes from a row's one half to its other
+    constexpr int kGroup = WR ? 2048 : 1024;     // and from eight rows to the next eight
     const int N = p.N, R = p.R, G = p.G;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q_bytes = N * 256;                       // one Q buffer: 2 halves x N rows x 128 B
@@ -488,21 +494,19 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         // =========================== TMA producer ===========================
         uint32_t ring = 0, ring_ph = 0, qn = 0;  // next slot (F8: raw stage), its phase; Q buffers filled
         const int boxes = p.boxes, box_rows = p.box_rows;
-        const bool whole = !F8 && p.whole_rows;
-        const uint32_t box_bytes = box_rows * (whole ? 256 : 128);
+        const uint32_t box_bytes = box_rows * (WR ? 256 : 128);
         const int halves = p.D / 64;  // 64-wide halves of the head dimension
         bool ok = true;
-        // A tile's boxes, one per lane: at most 16 of 8 whole rows, or that many for either half of the head dimension.
-        // F8: the
-        // tile's bytes (128 per key) go to a raw stage, and the softmax warps expand them into a slot.
+        // A tile's boxes, one per lane: at most 16 of 8 whole rows (WR), or that many for either half of the head dimension.
+        // F8: the tile's bytes (128 per key) go to a raw stage, and the softmax warps expand them into a slot.
         // The page table is read before the wait for a free slot: its latency (a trip to L2 per tile, which bounded
         // the stream of 16-token pages) hides behind that wait.
         auto load_tile = [&](const CUtensorMap* map, const Work& sg, int tile) -> bool {
             const int key0 = tile * kTile;
             // boxes that hold at least one key < T (pages past the context may not exist)
             const int n_box = min(boxes, (sg.T - key0 + box_rows - 1) / box_rows);
-            const int n_ops = F8 || whole ? n_box : halves * n_box;
-            const int half = !F8 && !whole && lane >= n_box ? 1 : 0, bx = lane - half * n_box;
+            const int n_ops = F8 || WR ? n_box : halves * n_box;
+            const int half = !F8 && !WR && lane >= n_box ? 1 : 0, bx = lane - half * n_box;
             const int pos = key0 + bx * box_rows;
             const int page = page_of(p.a.kv, pos), slot_in_page = pos - page * p.a.kv.page_size;
             int phys = 0;
@@ -526,11 +530,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 if (got) mbar_expect_tx(full, (uint32_t)n_ops * box_bytes);
             }
             if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
-            if (whole) {
-                if (lane < n_ops)
-                    tma_load_5d(s_slots + s * kSlotBytes + bx * box_bytes, map, full, 0, 0, 0, slot_in_page >> 3,
-                                sg.layer * p.row_layer + phys * p.row_page + sg.h * p.row_head, kEvictFirst);
-            } else if (lane < n_ops)
+            if (WR && lane < n_ops)
+                tma_load_5d(s_slots + s * kSlotBytes + bx * box_bytes, map, full, 0, 0, 0, slot_in_page >> 3,
+                            sg.layer * p.row_layer + phys * p.row_page + sg.h * p.row_head, kEvictFirst);
+            if (!WR && lane < n_ops)
                 tma_load_5d((F8 ? s_raw + s * 16384 : s_slots + s * kSlotBytes + half * 16384) + bx * box_bytes, map, full,
                             half * 64, slot_in_page, sg.h, phys, sg.layer, kEvictFirst);
             __syncwarp();
@@ -571,12 +574,9 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             // O^T += V^T [P_hi | P_lo]^T : A = V^T and B = P^T both MN-major, N = 2 * rows
             const uint32_t idesc_pv = (1u << 4) | ab_fmt | (1u << 15) | (1u << 16) |
                                       ((uint32_t)((2 * N) >> 3) << 17) | ((128u >> 4) << 24);
-            // Descriptors of slot 0's tiles (a place further on in shared memory only adds to them), the step to a row's
-            // other half and by 16 keys.  (Worked out anew for every product from the layout, which is not known at
-            // compile time, a launch of the 8B shape took 42.4 us instead of 39.1.)
-            const uint64_t k_desc = desc_kmajor(s_slots, p.group_bytes);
-            const uint64_t v_desc = desc_mnmajor(s_slots, p.half_bytes, p.group_bytes);
-            const uint32_t k_half = p.half_bytes >> 4, v_step = p.group_bytes >> 3;
+            // descriptors of slot 0's tiles: a place further on in shared memory only adds to them
+            const uint64_t k_desc = desc_kmajor(s_slots, kGroup);
+            const uint64_t v_desc = desc_mnmajor(s_slots, kHalf, kGroup);
             // Two independent queues, issued in whichever order their inputs become ready: the
             // QK^T tiles of unit u+1 may overtake the P V tiles of unit u that still wait for P.
             struct Queue {
@@ -632,7 +632,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     if (ks * 16 < p.D) {  // head_dim 64: the first four 16-wide steps
-                        const uint64_t a = k_tile + ((ks >> 2) * k_half + (ks & 3) * 2);
+                        const uint64_t a = k_tile + ((ks >> 2) * (kHalf >> 4) + (ks & 3) * 2);
                         const uint64_t b = desc_kmajor(s_q + (ks >> 2) * (N * 128) + (ks & 3) * 32);
                         tc_mma(d_s, a, b, idesc_qk, ks ? 1u : 0u);
                     }
@@ -659,7 +659,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 const uint32_t d_o = tmem_base + col_o;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t a = v_tile + ks * v_step;
+                    const uint64_t a = v_tile + ks * (2 * kGroup >> 4);
                     const uint64_t b = desc_mnmajor_nosw(p_addr + ks * 256);
                     tc_mma(d_o, a, b, idesc_pv, (pq.c == 0 && ks == 0) ? 0u : 1u);
                 }
@@ -1283,8 +1283,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                             ok = bar_wait(B.slot_full + 8 * vs, vsph, ctl);
                             if (!ok) break;
                             if (key >= sg.T && wg < 2) {  // warpgroups 0 and 1 clear one 64-wide half each
-                                uint8_t* vrow = sgen + (s_slots - sbase) + vs * kSlotBytes + wg * p.half_bytes +
-                                                (key_l >> 3) * p.group_bytes + (key_l & 7) * 128;
+                                uint8_t* vrow = sgen + (s_slots - sbase) + vs * kSlotBytes + wg * kHalf +
+                                                (key_l >> 3) * kGroup + (key_l & 7) * 128;
 #pragma unroll
                                 for (int ch = 0; ch < 8; ++ch) *reinterpret_cast<uint4*>(vrow + 16 * ch) = make_uint4(0, 0, 0, 0);
                             }
@@ -1487,11 +1487,11 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     if (!*abort_flag) reset_counters_if_last(p, reinterpret_cast<int*>(const_cast<uint32_t*>(tmem_slot)));
 }
 
-template <int NC, int CG, bool LP, bool PH, bool SC, bool F8>
+template <int NC, int CG, bool LP, bool PH, bool SC, bool F8, bool WR>
 int launch_cfg(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const FastParams& fp,
                int grid, size_t smem_bytes, cudaStream_t stream)
 {
-    auto kern = verify_cached_kernel<NC, CG, LP, PH, SC, F8>;
+    auto kern = verify_cached_kernel<NC, CG, LP, PH, SC, F8, WR>;
     // the largest size any plan of this instance asks for, once per device: the call costs the host as much as a launch
     static std::atomic<bool> opted_in[64] = {};
     int dev = 0;
@@ -1536,22 +1536,22 @@ int launch_cfg(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& 
     return SPEC_OK;
 }
 
-// One combination of statistic and cache format: the instance of a call's row count.
-template <bool PH, bool SC, bool F8>
+// One combination of statistic, cache format and tile layout: the instance of a call's row count.
+template <bool PH, bool SC, bool F8, bool WR>
 int launch_rows(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const FastParams& fp, int grid,
                 size_t smem_bytes, cudaStream_t stream)
 {
     const bool lp = fp.cph <= kLsePubMax;
 #define SPEC_CASE(n, nc, cg)                                                                              \
     case n:                                                                                               \
-        return lp ? launch_cfg<nc, cg, true, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream)        \
-                  : launch_cfg<nc, cg, false, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream);
+        return lp ? launch_cfg<nc, cg, true, PH, SC, F8, WR>(tk, tv, tq, fp, grid, smem_bytes, stream)    \
+                  : launch_cfg<nc, cg, false, PH, SC, F8, WR>(tk, tv, tq, fp, grid, smem_bytes, stream);
     // 17 to 24 rows pad a quarter of the MMA's 32: three warpgroups of eight columns instead of four (16 chats of
     // 0.6-6 K tokens: 57.5 -> 56.1 us per launch, five sequences of 4-30 K: 91.3 -> 88.4.  33 to 36 rows of 48 in
     // three groups of twelve gave nothing: those launches are not bound by the softmax warps.)
     if (fp.N == 32 && fp.R <= 24)
-        return lp ? launch_cfg<8, 3, true, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream)
-                  : launch_cfg<8, 3, false, PH, SC, F8>(tk, tv, tq, fp, grid, smem_bytes, stream);
+        return lp ? launch_cfg<8, 3, true, PH, SC, F8, WR>(tk, tv, tq, fp, grid, smem_bytes, stream)
+                  : launch_cfg<8, 3, false, PH, SC, F8, WR>(tk, tv, tq, fp, grid, smem_bytes, stream);
     switch (fp.N) {  // (columns per warpgroup, warpgroups)
         SPEC_CASE(16, 8, 2)
         SPEC_CASE(32, 8, 4)

@@ -17,7 +17,7 @@ L, H, D, N_Q = 2, 2, 128, 5
 
 def laid_out(kv, order, pad):
     """``kv`` ([layer, page, head, slot, D]) with its first four axes stored in ``order`` and ``pad`` elements behind each row."""
-    axes = [kv.n_layers, kv.k.shape[1], H, kv.page_size]
+    axes = [kv.n_layers, kv.k.shape[1], kv.n_kv_heads, kv.page_size]
     strides, step = [0] * 4, D + pad
     for a in reversed(order):
         strides[a] = step
@@ -61,3 +61,63 @@ def test_rows_beyond_31_bits_take_the_other_map():
     out, lse, stats, ws = binding.spec_verify_attn(large, case.q_verify, case.ctx_len, 700)
     assert binding.read_status(ws) == 0
     assert torch.equal(out, ref[0]) and torch.equal(lse, ref[1]) and torch.equal(stats[..., :700], ref[2][..., :700])
+
+
+def poison(case, ctx):
+    """NaN in every slot behind a sequence's context (in the pages the table gives it)."""
+    kv = case.kv
+    for b, t in enumerate(ctx):
+        for page in range(kv.max_pages):
+            first = max(0, t - page * kv.page_size)
+            if first < kv.page_size:
+                kv.k[:, kv.phys_page(b, page), :, first:] = float("nan")
+                kv.v[:, kv.phys_page(b, page), :, first:] = float("nan")
+
+
+# Rows per KV head that fill one, two, three and four warpgroups of different widths (8, 20, 36, 64, 68, 96, 104 and 128
+# rows are the eight widths of the score columns), each statistic, and tiles as whole rows and as halves (a pool that is
+# said to be too large to number its rows takes the halves).
+@pytest.mark.parametrize("n_q,group,kind", [(2, 4, "sum"), (5, 4, "per_head"), (9, 4, "group_max"), (16, 4, "hist"), (17, 4, "sum"),
+                                            (17, 4, "per_head"), (24, 4, "sum"), (26, 4, "group_max"), (32, 4, "hist"), (32, 4, "sum")])
+def test_rows_and_statistics_in_both_tile_layouts(n_q, group, kind):
+    ctx = [700, 33, 135]
+    cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=n_q, n_q_heads=group * H, n_kv_heads=H, head_dim=D, planted=4, batch=len(ctx),
+                              n_layers=L, page_size=16, shuffled_pages=True, seed=7)
+    case = inputs.make_case(cfg, device="cuda", ctx_override=ctx)
+    o_out, o_lse, o_stats = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, 704,
+                                               per_head=kind == "per_head", group_max=kind == "group_max")
+    poison(case, ctx)
+    heads = group * H if kind == "per_head" else H
+
+    def call(kv):
+        hist = torch.zeros(L, len(ctx), heads, 2048, dtype=torch.int32, device="cuda") if kind == "hist" else None
+        out, lse, stats, ws = binding.spec_verify_attn(kv, case.q_verify, case.ctx_len, 700, per_head=kind == "per_head",
+                                                       group_max=kind == "group_max", score_hist=hist)
+        assert binding.read_status(ws) == 0 and binding.last_verify_impl() == binding.VERIFY_TCGEN05_CACHED
+        return out, lse, stats, hist
+
+    ref = call(case.kv)
+    assert (ref[0].cpu().double() - o_out).abs().max().item() <= TOL
+    assert (ref[1].cpu().double() - o_lse).abs().max().item() <= TOL
+    assert (ref[2].cpu().double() - o_stats).abs().max().item() <= TOL
+    for kv in (dataclasses.replace(case.kv, n_pages=(1 << 30) + 8), laid_out(case.kv, (2, 0, 1, 3), 8), laid_out(case.kv, (0, 1, 3, 2), 0)):
+        got = call(kv)
+        for a, b in zip(ref, got):
+            assert a is None or torch.equal(a, b)
+
+
+def test_rows_in_two_passes_in_another_order_of_the_axes():
+    """68 rows at a context whose share of keys does not fit the score cache: two passes, each over both layouts."""
+    T = 80000
+    cfg = inputs.small_config(ctx=(T, T), n_q=17, n_q_heads=8, n_kv_heads=2, head_dim=D, planted=4, n_layers=1, page_size=16,
+                              shuffled_pages=True, seed=8)
+    case = inputs.make_case(cfg, device="cuda")
+    poison(case, [T])
+    got = []
+    for kv in (case.kv, dataclasses.replace(case.kv, n_pages=(1 << 30) + 8), laid_out(case.kv, (0, 3, 1, 2), 8)):
+        out, lse, stats, ws = binding.spec_verify_attn(kv, case.q_verify, case.ctx_len, T)
+        assert binding.read_status(ws) == 0 and binding.last_verify_impl() == binding.VERIFY_TCGEN05_CACHED_2PASS
+        assert torch.isfinite(out).all()
+        got.append((out, lse, stats))
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0], other))
