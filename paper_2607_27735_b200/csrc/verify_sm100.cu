@@ -253,13 +253,11 @@ bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_p
 // The cache as rows of two 64-wide halves: dimensions (64, 8 rows, half, groups of 8 rows in a page, (layer, page, head)).
 // One box then brings whole rows, the halves of eight of them as two swizzled 1 KB blocks side by side.  The last
 // dimension counts in the greatest common divisor of the three strides.
-// The copy unit takes 100-150 cycles over a box however small it is, so that 16-token pages were bound by it with the halves
-// in boxes of their own (16 boxes of 2 KB per tile): eight sequences of 9-66 K took 348 us, 262 with whole rows.
-// False where a row cannot be numbered in 31 bits (and for head_dim 64): the caller takes the other map.
+// False where a row cannot be numbered in 31 bits: the caller takes the other map.
 bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
 {
     EncodeTiledFn fn = encode_fn();
-    if (!fn || kv.head_dim != kD) return false;
+    if (!fn) return false;
     const int64_t st[3] = {kv.n_layers > 1 ? kv.layer_stride : 0, n_pages > 1 ? kv.page_stride : 0,
                            kv.n_kv_heads > 1 ? kv.head_stride : 0};
     const int64_t n[3] = {kv.n_layers, n_pages, kv.n_kv_heads};
@@ -278,6 +276,17 @@ bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, in
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Whether tiles are copied as whole rows.  The copy unit takes 100-150 cycles over a box however small it is, and with the
+// halves in boxes of their own a tile takes twice as many: where that bounds the stream, whole rows; elsewhere the halves,
+// which products and softmax take slightly faster.  Time with whole rows against halves, by tokens of a page:
+//                                        16        32       64       128     contiguous
+//   up to 48 score columns           -14..-25 %  -2..-9   -3..+0.4  -0.9..0.7   0..1.5     (32 K alone -14, 9-66 K x 8 -25)
+//   more (a tile's softmax is longer)  -9..+0.8  -0.2..1.4  -0.4..1  -0.4..1.3  0..1.2     (52 rows -9, 68 rows at 40 K +0.8)
+bool copy_whole_rows(const KvView& kv, int N, int box_rows)
+{
+    return kv.head_dim == kD && !kv.fp8 && !kv.k_scale && !kv.v_scale && box_rows <= (N <= 48 ? 64 : 16);
 }
 
 // 8-bit cache: a box is box_rows whole rows of 128 bytes, unswizzled (the softmax warps expand it)
@@ -507,7 +516,7 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows) ||
             !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows))
             return SPEC_ERR_CUDA;
-    } else if (pl.cached && !a.kv.k_scale && !a.kv.v_scale && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
+    } else if (pl.cached && copy_whole_rows(a.kv, pl.N, pl.box_rows) && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
                encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
         fp.whole_rows = 1;
     } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows) ||

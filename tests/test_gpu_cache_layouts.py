@@ -77,12 +77,15 @@ def poison(case, ctx):
 # Rows per KV head that fill one, two, three and four warpgroups of different widths (8, 20, 36, 64, 68, 96, 104 and 128
 # rows are the eight widths of the score columns), each statistic, and tiles as whole rows and as halves (a pool that is
 # said to be too large to number its rows takes the halves).
-@pytest.mark.parametrize("n_q,group,kind", [(2, 4, "sum"), (5, 4, "per_head"), (9, 4, "group_max"), (16, 4, "hist"), (17, 4, "sum"),
-                                            (17, 4, "per_head"), (24, 4, "sum"), (26, 4, "group_max"), (32, 4, "hist"), (32, 4, "sum")])
-def test_rows_and_statistics_in_both_tile_layouts(n_q, group, kind):
+# Pages of 64 tokens and of 16 are the largest that are copied as whole rows, up to 48 rows and above.
+@pytest.mark.parametrize("n_q,kind,page", [(2, "sum", 16), (5, "per_head", 64), (9, "group_max", 16), (12, "sum", 64), (13, "sum", 32),
+                                           (13, "per_head", 16), (16, "hist", 16), (17, "sum", 16), (17, "per_head", 16), (24, "sum", 16),
+                                           (26, "group_max", 16), (32, "hist", 16), (32, "sum", 32)])
+def test_rows_and_statistics_in_both_tile_layouts(n_q, kind, page):
+    group = 4
     ctx = [700, 33, 135]
     cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=n_q, n_q_heads=group * H, n_kv_heads=H, head_dim=D, planted=4, batch=len(ctx),
-                              n_layers=L, page_size=16, shuffled_pages=True, seed=7)
+                              n_layers=L, page_size=page, shuffled_pages=True, seed=7)
     case = inputs.make_case(cfg, device="cuda", ctx_override=ctx)
     o_out, o_lse, o_stats = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, 704,
                                                per_head=kind == "per_head", group_max=kind == "group_max")
