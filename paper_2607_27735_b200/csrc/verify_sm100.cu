@@ -232,20 +232,31 @@ bool make_plan(const KvView& kv, int n_q, int max_ctx_len, int variant, Plan* pl
     return true;
 }
 
-bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows)
+// The map's axes behind the head dimension, (slot, head, page, layer), for elements of `es` bytes.  No axis of a map may have
+// stride 0: one that has (every head, page or layer the same rows) gets extent 1, and coordinates on it the factor 0.
+void map_axes(const KvView& kv, int n_pages, int es, cuuint64_t dims[5], cuuint64_t strides[4], FastParams* fp)
+{
+    const cuuint64_t n[4] = {(cuuint64_t)kv.page_size, (cuuint64_t)kv.n_kv_heads, (cuuint64_t)n_pages, (cuuint64_t)kv.n_layers};
+    const int64_t st[4] = {kv.slot_stride, kv.head_stride, kv.page_stride, kv.layer_stride};
+    dims[0] = (cuuint64_t)kv.head_dim;
+    for (int i = 0; i < 4; ++i) {
+        dims[i + 1] = st[i] ? n[i] : 1;
+        strides[i] = st[i] ? (cuuint64_t)st[i] * es : 16;
+    }
+    fp->row_head = st[1] ? 1 : 0;
+    fp->row_page = st[2] ? 1 : 0;
+    fp->row_layer = st[3] ? 1 : 0;
+}
+
+bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[5] = {(cuuint64_t)kv.head_dim, (cuuint64_t)kv.page_size, (cuuint64_t)kv.n_kv_heads,
-                                (cuuint64_t)n_pages, (cuuint64_t)kv.n_layers};
-    const cuuint64_t strides[4] = {(cuuint64_t)kv.slot_stride * 2, (cuuint64_t)kv.head_stride * 2,
-                                   (cuuint64_t)kv.page_stride * 2, (cuuint64_t)kv.layer_stride * 2};
+    cuuint64_t dims[5], strides[4];
+    map_axes(kv, n_pages, 2, dims, strides, fp);
     const cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 1, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    // a stride of 0 is legal only for extent-1 dimensions; give those any multiple of 16
-    cuuint64_t st[4];
-    for (int i = 0; i < 4; ++i) st[i] = strides[i] ? strides[i] : 16;
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, st, box, estr,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -290,19 +301,15 @@ bool copy_whole_rows(const KvView& kv, int N, int box_rows)
 }
 
 // 8-bit cache: a box is box_rows whole rows of 128 bytes, unswizzled (the softmax warps expand it)
-bool encode_kv_map_u8(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows)
+bool encode_kv_map_u8(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[5] = {(cuuint64_t)kv.head_dim, (cuuint64_t)kv.page_size, (cuuint64_t)kv.n_kv_heads,
-                                (cuuint64_t)n_pages, (cuuint64_t)kv.n_layers};
-    const cuuint64_t strides[4] = {(cuuint64_t)kv.slot_stride, (cuuint64_t)kv.head_stride, (cuuint64_t)kv.page_stride,
-                                   (cuuint64_t)kv.layer_stride};
+    cuuint64_t dims[5], strides[4];
+    map_axes(kv, n_pages, 1, dims, strides, fp);
     const cuuint32_t box[5] = {128, (cuuint32_t)box_rows, 1, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    cuuint64_t st[4];
-    for (int i = 0; i < 4; ++i) st[i] = strides[i] ? strides[i] : 16;
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(base), dims, st, box, estr,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -513,14 +520,14 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
     FastParams fp;
     fp.whole_rows = 0;
     if (a.kv.fp8) {
-        if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows) ||
-            !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows))
+        if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows, &fp) ||
+            !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows, &fp))
             return SPEC_ERR_CUDA;
     } else if (pl.cached && copy_whole_rows(a.kv, pl.N, pl.box_rows) && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
                encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
         fp.whole_rows = 1;
-    } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows) ||
-               !encode_kv_map(&tv, a.kv.v, a.kv, n_pages, pl.box_rows)) {
+    } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) ||
+               !encode_kv_map(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
         return SPEC_ERR_CUDA;
     }
     if (!encode_q_map(&tq, a.q, a.kv, a.n_q, G)) return SPEC_ERR_CUDA;

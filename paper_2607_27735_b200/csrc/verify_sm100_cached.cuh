@@ -535,7 +535,7 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                             sg.layer * p.row_layer + phys * p.row_page + sg.h * p.row_head, kEvictFirst);
             if (!WR && lane < n_ops)
                 tma_load_5d((F8 ? s_raw + s * 16384 : s_slots + s * kSlotBytes + half * 16384) + bx * box_bytes, map, full,
-                            half * 64, slot_in_page, sg.h, phys, sg.layer, kEvictFirst);
+                            half * 64, slot_in_page, sg.h * p.row_head, phys * p.row_page, sg.layer * p.row_layer, kEvictFirst);
             __syncwarp();
             return true;
         };

@@ -224,7 +224,8 @@ verify_twosweep_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
                     phys = 0;
                 }
                 const uint32_t dst = s_slots + s * kSlotBytes + half * 16384 + bx * box_bytes;
-                tma_load_5d(dst, map, B.slot_full + 8 * s, half * 64, slot_in_page, sg.h, phys, sg.layer, hint);
+                tma_load_5d(dst, map, B.slot_full + 8 * s, half * 64, slot_in_page, sg.h * p.row_head, phys * p.row_page,
+                            sg.layer * p.row_layer, hint);
             }
             __syncwarp();
             return true;

@@ -124,3 +124,42 @@ def test_rows_in_two_passes_in_another_order_of_the_axes():
         got.append((out, lse, stats))
     for other in got[1:]:
         assert all(torch.equal(a, b) for a, b in zip(got[0], other))
+
+
+# A stride of 0 over an extent above 1: every head, page or layer the same rows.  Each of the maps that copies are built from
+# has to read it so: whole rows, halves (128-token pages, head_dim 64, a pool too large to number its rows), bytes, two sweeps.
+@pytest.mark.parametrize("axis", ["layer", "page", "head"])
+@pytest.mark.parametrize("what", ["rows", "halves", "dim64", "large", "fp8", "fp8_dim64", "two_sweeps"])
+def test_an_axis_of_stride_zero_is_a_broadcast(axis, what):
+    ctx = [400, 129]
+    dim, page = (64 if "dim64" in what else D), (128 if what == "halves" else 16)
+    cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=N_Q, n_q_heads=4 * H, n_kv_heads=H, head_dim=dim, planted=4, batch=len(ctx),
+                              n_layers=L, page_size=page, shuffled_pages=True, seed=9)
+    case = inputs.make_case(cfg, device="cuda", ctx_override=ctx)
+    kv = case.kv
+    if what.startswith("fp8"):
+        kv = inputs.quantize_kv_fp8(kv)
+        # other scales per head and layer, within a factor of 1.5 of the quantisation's: values stay of the order of 1 (up to 7),
+        # which TOL is stated for (it is absolute; probabilities carry 2^-14 and fp32 sums of them)
+        kv = dataclasses.replace(kv, k_scale=kv.k_scale * (torch.rand_like(kv.k_scale) + 0.5),
+                                 v_scale=kv.v_scale * (torch.rand_like(kv.v_scale) + 0.5))
+    at = {"layer": 0, "page": 1, "head": 2}[axis]
+    def spread(x):  # the same rows written out for every place of the axis
+        x = x.clone()
+        x.copy_(x.select(at, 0).unsqueeze(at).expand_as(x))
+        return x
+    dense = dataclasses.replace(kv, k=spread(kv.k), v=spread(kv.v))
+    zero = dataclasses.replace(kv, **{axis + "_stride": 0})
+    if what == "large":
+        zero = dataclasses.replace(zero, n_pages=(1 << 30) + 8)
+    prev = binding.set_verify_impl(binding.VERIFY_TCGEN05_TWOSWEEP if what == "two_sweeps" else binding.VERIFY_AUTO)
+    try:
+        ref = binding.spec_verify_attn(dense, case.q_verify, case.ctx_len, max(ctx))
+        got = binding.spec_verify_attn(zero, case.q_verify, case.ctx_len, max(ctx))
+    finally:
+        binding.set_verify_impl(prev)
+    assert binding.read_status(ref[3]) == 0 and binding.read_status(got[3]) == 0
+    o_out, o_lse, o_stats = oracle.verify_attn(dense.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, ref[2].shape[-1])
+    for a, b, o in zip(ref, got, (o_out, o_lse, o_stats)):
+        assert (a.cpu().double() - o).abs().max().item() <= TOL
+        assert (b.cpu().double() - o).abs().max().item() <= TOL
