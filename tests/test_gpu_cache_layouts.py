@@ -1,7 +1,7 @@
-"""Verification over the same keys and values laid out in memory in different ways: what the copies of a tile are built from
+"""Verification over the same keys and values laid out in memory in different ways: what the copies of whole rows are built from
 is the strides' greatest common divisor, so heads outside pages, heads between rows, padded rows, layers inside
-pages and pages of 8 to 128 tokens have to give the bits that the dense order gives (the arithmetic behind the copies is
-the same)."""
+pages and pages of 8 to 256 tokens have to give the bits that the dense order gives, and whole rows those of the halves (the
+arithmetic behind the copies is the same)."""
 import dataclasses
 
 import pytest
@@ -30,18 +30,31 @@ def laid_out(kv, order, pad):
                                head_stride=strides[2], slot_stride=strides[3], n_pages=kv.k.shape[1])
 
 
-@pytest.mark.parametrize("page", [8, 16, 64, 128])
+def poison(case, ctx):
+    """NaN in every slot behind a sequence's context (in the pages the table gives it)."""
+    kv = case.kv
+    for b, t in enumerate(ctx):
+        for page in range(kv.max_pages):
+            first = max(0, t - page * kv.page_size)
+            if first < kv.page_size:
+                kv.k[:, kv.phys_page(b, page), :, first:] = float("nan")
+                kv.v[:, kv.phys_page(b, page), :, first:] = float("nan")
+
+
+# pages of up to 64 tokens are copied as whole rows, larger ones as halves, those above 128 in pieces
+@pytest.mark.parametrize("page", [8, 16, 64, 128, 256])
 @pytest.mark.parametrize("ctx", [[700, 129, 128], [9]])
 def test_every_order_gives_the_bits_of_the_dense_one(page, ctx):
     cfg = inputs.small_config(ctx=(min(ctx), max(ctx)), n_q=N_Q, n_q_heads=4 * H, n_kv_heads=H, head_dim=D, planted=4,
                               batch=len(ctx), n_layers=L, page_size=page, shuffled_pages=True, seed=5)
     case = inputs.make_case(cfg, device="cuda", ctx_override=ctx)
     T = max(ctx)
+    poison(case, ctx)
     ref = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, T)
     assert binding.read_status(ref[3]) == 0
-    o_out, o_lse, _ = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, ref[2].shape[-1])
-    assert (ref[0].cpu().double() - o_out).abs().max().item() <= TOL
-    assert (ref[1].cpu().double() - o_lse).abs().max().item() <= TOL
+    o_out, o_lse, o_stats = oracle.verify_attn(case.kv.cpu(), case.q_verify.cpu(), case.ctx_len.cpu(), 16, ref[2].shape[-1])
+    for got, want in zip(ref, (o_out, o_lse, o_stats)):
+        assert (got.cpu().double() - want).abs().max().item() <= TOL
     for order, pad in (((0, 1, 2, 3), 8), ((0, 1, 3, 2), 0), ((2, 0, 1, 3), 0), ((1, 0, 2, 3), 24), ((3, 2, 1, 0), 0), ((0, 2, 1, 3), 8)):
         out, lse, stats, ws = binding.spec_verify_attn(laid_out(case.kv, order, pad), case.q_verify, case.ctx_len, T)
         assert binding.read_status(ws) == 0
@@ -56,22 +69,13 @@ def test_rows_beyond_31_bits_take_the_other_map():
     cfg = inputs.small_config(ctx=(700, 700), n_q=N_Q, n_q_heads=4 * H, n_kv_heads=H, head_dim=D, planted=4, n_layers=L,
                               page_size=16, shuffled_pages=True, seed=6)
     case = inputs.make_case(cfg, device="cuda")
+    poison(case, [700])
     ref = binding.spec_verify_attn(case.kv, case.q_verify, case.ctx_len, 700)
+    assert torch.isfinite(ref[0]).all()
     large = dataclasses.replace(case.kv, n_pages=(1 << 30) + 8)
     out, lse, stats, ws = binding.spec_verify_attn(large, case.q_verify, case.ctx_len, 700)
     assert binding.read_status(ws) == 0
     assert torch.equal(out, ref[0]) and torch.equal(lse, ref[1]) and torch.equal(stats[..., :700], ref[2][..., :700])
-
-
-def poison(case, ctx):
-    """NaN in every slot behind a sequence's context (in the pages the table gives it)."""
-    kv = case.kv
-    for b, t in enumerate(ctx):
-        for page in range(kv.max_pages):
-            first = max(0, t - page * kv.page_size)
-            if first < kv.page_size:
-                kv.k[:, kv.phys_page(b, page), :, first:] = float("nan")
-                kv.v[:, kv.phys_page(b, page), :, first:] = float("nan")
 
 
 # Rows per KV head that fill one, two, three and four warpgroups of different widths (8, 20, 36, 64, 68, 96, 104 and 128
