@@ -27,7 +27,7 @@ struct FastParams {
     int n_slots, p_bufs;
     int n_raw;                        // 8-bit cache read directly: raw 16 KB stages in front of the operand slots (else 0)
     int D;                            // head_dim: 128, or 64 (score-cache kernel only)
-    int box_rows, boxes;              // rows of a TMA box; boxes per tile (two 64-wide halves apart: per half)
+    int box_rows, boxes;              // rows of a TMA box; boxes per tile (halves: per half)
     int whole_rows;                   // score-cache kernel: boxes of whole rows (see encode_kv_map_rows)
     int row_layer, row_page, row_head;  // factors of a box's coordinates: whole rows are numbered layer * row_layer +
                                         // page * row_page + head * row_head; else 1, or 0 for an axis of stride 0

@@ -262,10 +262,10 @@ bool encode_kv_map(CUtensorMap* map, const void* base, const KvView& kv, int n_p
 }
 
 // The cache as rows of two 64-wide halves: dimensions (64, 8 rows, half, groups of 8 rows in a page, (layer, page, head)).
-// One box then brings whole rows, the halves of eight of them as two swizzled 1 KB blocks side by side.  The last
+// One box, a page, then brings whole rows, the halves of eight of them as two swizzled 1 KB blocks side by side.  The last
 // dimension counts in the greatest common divisor of the three strides.
 // False where a row cannot be numbered in 31 bits: the caller takes the other map.
-bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, int box_rows, FastParams* fp)
+bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, int n_pages, FastParams* fp)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
@@ -282,7 +282,7 @@ bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, in
     fp->row_head = (int)(st[2] / unit);
     const cuuint64_t dims[5] = {64, 8, 2, (cuuint64_t)kv.page_size / 8, (cuuint64_t)last + 1};
     const cuuint64_t strides[4] = {(cuuint64_t)kv.slot_stride * 2, 128, (cuuint64_t)kv.slot_stride * 16, (cuuint64_t)unit * 2};
-    const cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)box_rows / 8, 1};
+    const cuuint32_t box[5] = {64, 8, 2, (cuuint32_t)kv.page_size / 8, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -293,11 +293,12 @@ bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, in
 // halves in boxes of their own a tile takes twice as many: where that bounds the stream, whole rows; elsewhere the halves,
 // which products and softmax take slightly faster.  Time with whole rows against halves, by tokens of a page:
 //                                        16        32       64       128     contiguous
-//   up to 48 score columns           -14..-25 %  -2..-9   -3..+0.4  -0.9..0.7   0..1.5     (32 K alone -14, 9-66 K x 8 -25)
+//   up to 48 score columns           -14..-25 %  -2..-9   -3..+0.4  -0.9..0.7   0..1.5     (32 K alone -14, 9-66 K x 8 -25,
+//                                                                                           a few hundred keys -1.5)
 //   more (a tile's softmax is longer)  -9..+0.8  -0.2..1.4  -0.4..1  -0.4..1.3  0..1.2     (52 rows -9, 68 rows at 40 K +0.8)
-bool copy_whole_rows(const KvView& kv, int N, int box_rows)
+bool copy_whole_rows(const KvView& kv, int N)
 {
-    return kv.head_dim == kD && !kv.fp8 && !kv.k_scale && !kv.v_scale && box_rows <= (N <= 48 ? 64 : 16);
+    return kv.head_dim == kD && !kv.fp8 && !kv.k_scale && !kv.v_scale && kv.page_size <= (N <= 48 ? 64 : 16);
 }
 
 // 8-bit cache: a box is box_rows whole rows of 128 bytes, unswizzled (the softmax warps expand it)
@@ -523,8 +524,8 @@ int verify_sm100_launch(const VerifyArgs& a, int variant, cudaStream_t stream, i
         if (!encode_kv_map_u8(&tk, a.kv.k8, a.kv, n_pages, pl.box_rows, &fp) ||
             !encode_kv_map_u8(&tv, a.kv.v8, a.kv, n_pages, pl.box_rows, &fp))
             return SPEC_ERR_CUDA;
-    } else if (pl.cached && copy_whole_rows(a.kv, pl.N, pl.box_rows) && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) &&
-               encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {
+    } else if (pl.cached && copy_whole_rows(a.kv, pl.N) && encode_kv_map_rows(&tk, a.kv.k, a.kv, n_pages, &fp) &&
+               encode_kv_map_rows(&tv, a.kv.v, a.kv, n_pages, &fp)) {
         fp.whole_rows = 1;
     } else if (!encode_kv_map(&tk, a.kv.k, a.kv, n_pages, pl.box_rows, &fp) ||
                !encode_kv_map(&tv, a.kv.v, a.kv, n_pages, pl.box_rows, &fp)) {

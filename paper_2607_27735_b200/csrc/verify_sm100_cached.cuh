@@ -530,8 +530,8 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                 if (got) mbar_expect_tx(full, (uint32_t)n_ops * box_bytes);
             }
             if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) return false;
-            if (WR && lane < n_ops)
-                tma_load_5d(s_slots + s * kSlotBytes + bx * box_bytes, map, full, 0, 0, 0, slot_in_page >> 3,
+            if (WR && lane < n_ops)  // (a box is a page: see copy_whole_rows)
+                tma_load_5d(s_slots + s * kSlotBytes + bx * box_bytes, map, full, 0, 0, 0, 0,
                             sg.layer * p.row_layer + phys * p.row_page + sg.h * p.row_head, kEvictFirst);
             if (!WR && lane < n_ops)
                 tma_load_5d((F8 ? s_raw + s * 16384 : s_slots + s * kSlotBytes + half * 16384) + bx * box_bytes, map, full,
