@@ -291,14 +291,13 @@ bool encode_kv_map_rows(CUtensorMap* map, const void* base, const KvView& kv, in
 
 // Whether tiles are copied as whole rows.  The copy unit takes 100-150 cycles over a box however small it is, and with the
 // halves in boxes of their own a tile takes twice as many: where that bounds the stream, whole rows; elsewhere the halves,
-// which products and softmax take slightly faster.  Time with whole rows against halves, by tokens of a page:
-//                                        16        32       64       128     contiguous
-//   up to 48 score columns           -14..-25 %  -2..-9   -3..+0.4  -0.9..0.7   0..1.5     (32 K alone -14, 9-66 K x 8 -25,
-//                                                                                           a few hundred keys -1.5)
-//   more (a tile's softmax is longer)  -9..+0.8  -0.2..1.4  -0.4..1  -0.4..1.3  0..1.2     (52 rows -9, 68 rows at 40 K +0.8)
+// which products and softmax take slightly faster.  Time with whole rows against halves in %, 25 shapes, by tokens of a page:
+//                             8           16          32          64          128
+//   up to 64 score columns  -35..-3    -27..-1    -10..+0.2   -4.3..+0.5  -1.4..+0.5   (short calls gain least)
+//   more: longer softmax     -5..-0.4   -2..+0.3  +0.2..+0.8  +0.2..+0.7      0..+0.9
 bool copy_whole_rows(const KvView& kv, int N)
 {
-    return kv.head_dim == kD && !kv.fp8 && !kv.k_scale && !kv.v_scale && kv.page_size <= (N <= 48 ? 64 : 16);
+    return kv.head_dim == kD && !kv.fp8 && !kv.k_scale && !kv.v_scale && kv.page_size <= (N <= 64 ? 64 : 16);
 }
 
 // 8-bit cache: a box is box_rows whole rows of 128 bytes, unswizzled (the softmax warps expand it)

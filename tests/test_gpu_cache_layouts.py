@@ -81,9 +81,9 @@ def test_rows_beyond_31_bits_take_the_other_map():
 # Rows per KV head that fill one, two, three and four warpgroups of different widths (8, 20, 36, 64, 68, 96, 104 and 128
 # rows are the eight widths of the score columns), each statistic, and tiles as whole rows and as halves (a pool that is
 # said to be too large to number its rows takes the halves).
-# Pages of 64 tokens and of 16 are the largest that are copied as whole rows, up to 48 rows and above.
-@pytest.mark.parametrize("n_q,kind,page", [(2, "sum", 16), (5, "per_head", 64), (9, "group_max", 16), (12, "sum", 64), (13, "sum", 32),
-                                           (13, "per_head", 16), (16, "hist", 16), (17, "sum", 16), (17, "per_head", 16), (24, "sum", 16),
+# Pages of 64 tokens and of 16 are the largest that are copied as whole rows, up to 64 rows and above.
+@pytest.mark.parametrize("n_q,kind,page", [(2, "sum", 16), (5, "per_head", 64), (9, "group_max", 16), (12, "sum", 64), (13, "sum", 64),
+                                           (13, "per_head", 16), (16, "hist", 32), (17, "sum", 16), (17, "per_head", 16), (24, "sum", 16),
                                            (26, "group_max", 16), (32, "hist", 16), (32, "sum", 32)])
 def test_rows_and_statistics_in_both_tile_layouts(n_q, kind, page):
     group = 4
