@@ -698,10 +698,10 @@ verify_cached_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                     spins = 0;
                     continue;
                 }
-                // (No sleep here.  With 40 ns between two looks, 15 shapes of 5 to 128 rows on pages of 16 tokens to whole contexts:
-                // 0 to 1 % slower a launch (68 rows at 40 K 317.8 -> 319.1 us, 85 rows 79.0 -> 79.9, 8B at 128 K, k = 16, 269.0 -> 270.3, 16
-                // chats 49.24 -> 49.6), over an 8-bit cache 0 to 0.7 %; runs of one side differ by 0.3 %.  Only on 8-token pages, whose
-                // copies bound the launch, the sleep was 0.3 to 0.9 % the faster.)
+                // (No sleep here.  With 40 ns between two looks, 25 shapes of 8 to 128 rows on pages of 16 tokens to whole contexts:
+                // 0 to 0.9 % slower a launch (85 rows 78.85 -> 79.6 us, 68 rows at 40 K 314.4 -> 316.3, 32 K alone 39.9 -> 40.2), over an
+                // 8-bit cache -0.5 to +1.6 %; runs of one side differ by 0.3 %, those of a few thousand keys by 1 %.  On 8-token
+                // pages, whose copies bound the launch, -0.3 to +0.8 %.)
                 if ((++spins & 63u) == 0) {
                     if (spins == 64) t_idle = clock64();
                     if (*ctl.abort_flag) ok = false;
