@@ -716,8 +716,10 @@ int launch_shape(const DraftArgs& a, const StreamShape& shp, cudaStream_t stream
 // How a call is split: CTAs per cluster (one cluster per (layer, sequence, KV head)), keys per CTA,
 // warps per CTA and stages per warp: the split that a cost model likes best.  The model was fitted to the measured
 // times (layer-calls back to back, as a drafting round issues them) of every split at 33 shapes: 2 to 128 problems,
-// 260 to 4104 keys, groups of 1 to 8, both cache types, head_dim 64 and 128; its choice is on average 2-4 % above the
-// best split of a shape.  What it counts:
+// 260 to 4104 keys, groups of 1 to 8, both cache types, head_dim 64 and 128.  Against the best split of a shape its choice is
+// 2.7 % slower over 24 other bf16 shapes (worst 13 %) and 6.6 % over 40 with an 8-bit cache (worst 24 %): the factors for
+// that cache (0.63 and 5.5 below) were fitted before its conversions took one instruction each, and short key lists
+// would rather have four warps now (24 problems of 500 keys in groups of one: 3.95 us, 3.2 at best).  What it counts:
 //  - how many CTAs the GPU holds: shared memory, registers (16 warps of 128 registers, 20 at head_dim 64), and clusters
 //    that have to fit the 18 SMs of a GPC;
 //  - few problems (a cluster of 8 each would not fill the GPU): a call is a chain of latencies.  Two consecutive calls
